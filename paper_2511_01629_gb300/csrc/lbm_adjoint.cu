@@ -142,35 +142,6 @@ __device__ __forceinline__ void node_adjoint(const float* f, const float* a, con
     }
 }
 
-// Pre-collision population q at node (x, y, z) of step n: pull streaming
-// from the recorded populations, with bounce-back and the wall term where
-// x - c_q lies beyond a wall (the first such axis names the wall, as in the
-// forward kernels).  Selects instead of branches, so that the lanes of a warp
-// on a face stay together.
-template <int Q, class S, int q>
-__device__ __forceinline__ float pull_pre_any(const InstDesc& in, const S* __restrict__ fin, int x, int y, int z,
-                                              int qs) {
-    using L = Lat<Q>;
-    constexpr int c[3] = {L::c(q, 0), L::c(q, 1), L::c(q, 2)};
-    int src[3] = {x - c[0], y - c[1], z - c[2]};
-    int axis = -1, face = 0;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        if (c[d] == 0) continue;
-        const bool out = src[d] < 0 || src[d] >= in.n[d];
-        if (out && in.periodic[d]) src[d] += src[d] < 0 ? in.n[d] : -in.n[d];
-        else if (out && axis < 0) {
-            axis = d;
-            face = src[d] < 0 ? 0 : 1;
-        }
-    }
-    const int node = (z * in.n[1] + y) * in.pitch + x;
-    const int off = axis >= 0 ? (L::opp(q) - 1) * qs + node
-                              : (q - 1) * qs + (src[2] * in.n[1] + src[1]) * in.pitch + src[0];
-    const float v = VecIO<S, 1 + (sizeof(S) == 2)>::load1(fin + off, in.s_load);
-    return axis >= 0 ? v + in.wterm[axis][face][q] : v;
-}
-
 // Transposed streaming: the adjoint of f*_q at x is the adjoint of f_q at
 // x + c_q (wrapped on periodic axes), or of f_opp(q) at x when x + c_q lies
 // beyond a wall (the population bounced back at x).

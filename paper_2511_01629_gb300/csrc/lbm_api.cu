@@ -20,7 +20,7 @@ cudaError_t launch_fluid(int Q, int fp16, const InstDesc* insts, const uint16_t*
                          int ntiles, int par, const Shape& sh, int commit, int persistent, int grid,
                          int* tile_ctr, cudaStream_t st);
 int fluid_max_blocks_per_sm(int Q, int fp16, const Shape& sh);
-cudaError_t launch_fields(int Q, int fp16, const InstDesc* insts, int inst, long long N, int par,
+cudaError_t launch_fields(int Q, int fp16, const InstDesc* insts, int inst, const int* n, int par,
                           const Shape& sh, float* u, float* p, int* owner, cudaStream_t st);
 cudaError_t launch_pack(int Q, int fp16, const InstDesc* insts, int inst, long long N, int par,
                         const float* src, cudaStream_t st);
@@ -985,7 +985,7 @@ int lbm_get_fields(lbm_ctx* ctx, int i, float* u, float* p, int* owner, int on_d
     Instance& I = ctx->inst[i];
     const long long N = (long long)I.n[0] * I.n[1] * I.n[2];
     if (on_device) {
-        CK(launch_fields(ctx->Q, ctx->fp16, P<InstDesc>(ctx->d_insts), i, N, ctx->par, ctx->shape, u,
+        CK(launch_fields(ctx->Q, ctx->fp16, P<InstDesc>(ctx->d_insts), i, I.n, ctx->par, ctx->shape, u,
                          p, owner, ctx->st));
         return LBM_OK;
     }
@@ -996,7 +996,7 @@ int lbm_get_fields(lbm_ctx* ctx, int i, float* u, float* p, int* owner, int on_d
         dfree(ctx, du); dfree(ctx, dp); dfree(ctx, dow);
         return rc;
     }
-    cudaError_t e = launch_fields(ctx->Q, ctx->fp16, P<InstDesc>(ctx->d_insts), i, N, ctx->par,
+    cudaError_t e = launch_fields(ctx->Q, ctx->fp16, P<InstDesc>(ctx->d_insts), i, I.n, ctx->par,
                                   ctx->shape, P<float>(du), P<float>(dp), P<int>(dow), ctx->st);
     if (e == cudaSuccess && u) e = cudaMemcpyAsync(u, du.ptr, sizeof(float) * ctx->D * N, cudaMemcpyDeviceToHost, ctx->st);
     if (e == cudaSuccess && p) e = cudaMemcpyAsync(p, dp.ptr, sizeof(float) * N, cudaMemcpyDeviceToHost, ctx->st);

@@ -891,4 +891,45 @@ __device__ __noinline__ float pull_scalar(const InstDesc& in, const S* fin, int 
     return VecIO<S, 1 + (sizeof(S) == 2)>::load1(p, in.s_load) + add;
 }
 
+// Pre-collision population q at node (x, y, z): pull_scalar for a
+// compile-time q, with bounce-back and the wall term where x - c_q lies beyond
+// a wall (the first such axis names the wall).  Selects instead of branches, so that the lanes of a warp
+// on a face stay together.
+template <int Q, class S, int q>
+__device__ __forceinline__ float pull_pre_any(const InstDesc& in, const S* __restrict__ fin, int x, int y, int z,
+                                              int qs) {
+    using L = Lat<Q>;
+    constexpr int c[3] = {L::c(q, 0), L::c(q, 1), L::c(q, 2)};
+    int src[3] = {x - c[0], y - c[1], z - c[2]};
+    int axis = -1, face = 0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        if (c[d] == 0) continue;
+        const bool out = src[d] < 0 || src[d] >= in.n[d];
+        if (out && in.periodic[d]) src[d] += src[d] < 0 ? in.n[d] : -in.n[d];
+        else if (out && axis < 0) {
+            axis = d;
+            face = src[d] < 0 ? 0 : 1;
+        }
+    }
+    const int node = (z * in.n[1] + y) * in.pitch + x;
+    const int off = axis >= 0 ? (L::opp(q) - 1) * qs + node
+                              : (q - 1) * qs + (src[2] * in.n[1] + src[1]) * in.pitch + src[0];
+    // the wall term is loaded whether it is needed or not: a load under a
+    // condition would hold back the next population's (one memory latency each)
+    const float term = __ldg(&in.wterm[axis >= 0 ? axis : 0][face][q]);
+    const float v = VecIO<S, 1 + (sizeof(S) == 2)>::load1(fin + off, in.s_load);
+    return axis >= 0 ? v + term : v;
+}
+
+// All populations of a node by pull_pre_any (independent loads in flight).
+template <int Q, class S, int q = 1>
+__device__ __forceinline__ void pull_pre_all(const InstDesc& in, const S* __restrict__ fin, int x, int y, int z, int qs,
+                                             float* f) {
+    if constexpr (q < Q) {
+        f[q - 1] = pull_pre_any<Q, S, q>(in, fin, x, y, z, qs);
+        pull_pre_all<Q, S, q + 1>(in, fin, x, y, z, qs, f);
+    }
+}
+
 }  // namespace lbmpen

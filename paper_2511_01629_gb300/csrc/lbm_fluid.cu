@@ -304,51 +304,105 @@ __global__ void __launch_bounds__(256) k_fluid(const InstDesc* __restrict__ inst
 }
 
 // u, p, owner of every node of one instance (no collision, state unchanged).
+// Bound by HBM: Q - 1 populations read, D + 2 words written per node.  A warp
+// takes 64 nodes of one row, each lane one node of every 32 (coalesced
+// 4- or 2-byte loads), all populations of all its nodes in flight before the
+// first is used; rows and chunks inside the box read at fixed offsets, the
+// others through selects (pull_pre_any), so no lane waits on another's
+// boundary case.  The owner comes from the tile's candidate records by the
+// fused kernel's own filter, exact FP64 only in its band.
+// 1024 x 4096, 500 disks, FP32: 216 us before (a call per population with
+// dependent descriptor loads, every candidate tested in FP64 at every node),
+// 64.5 us now (3.1 TB/s).  128 nodes per warp (80 registers) took 70 us.
+template <int Q> __host__ __device__ constexpr int field_chunks() { return 2; }
+
 template <int Q, class S>
-__global__ void k_fields(const InstDesc* __restrict__ insts, int inst, int par, Shape sh, float* u,
-                         float* pout, int* owner) {
+__global__ void __launch_bounds__(256, Q == 9 ? 4 : 2) k_fields(const InstDesc* __restrict__ insts, int inst, int par, Shape sh,
+                                                int nseg, unsigned nwork, float* u, float* pout, int* owner) {
     using L = Lat<Q>;
     constexpr int D = L::D;
+    constexpr int NK = field_chunks<Q>();
     const InstDesc& in = insts[inst];
-    const long long N = (long long)in.n[0] * in.n[1] * in.n[2];
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const int x = (int)(i % in.n[0]), y = (int)((i / in.n[0]) % in.n[1]),
-              z = (int)(i / ((long long)in.n[0] * in.n[1]));
-    const S* fin = static_cast<const S*>(in.f[par]);
-    float f[Q - 1];
-    for (int q = 1; q < Q; ++q) f[q - 1] = pull_scalar<Q, S>(in, fin, q, x, y, z);
-    // owner through the same tile candidate lists the fused kernel uses
-    int own = -1;
-    float a[3] = {in.gdrive[0], in.gdrive[1], in.gdrive[2]};
-    if (in.np > 0) {
-        const Geo geo = make_geo(in);
-        const int tw = sh.tw;
-        const int local = (z / sh.tz * in.ntile[1] + y / sh.ty) * in.ntile[0] + x / tw;
-        const int nc = min(in.list_cnt[par][local], LIST_CAP);
-        const int xyz[3] = {x, y, z};
-        for (int c = 0; c < nc; ++c) {
-            const uint32_t e = in.list_ent[par][(long long)local * LIST_CAP + c];
-            const int p = (int)(e >> KBITS);
-            if (own >= 0 && p > own) continue;
-            if (inside_exact<D>(geo, in.prec[p], xyz)) own = p;
+    const int lane = threadIdx.x & 31;
+    const unsigned w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (w >= nwork) return;  // warp-uniform
+    const int nx = in.n[0], ny = in.n[1], nz = in.n[2], pitch = in.pitch;
+    const int seg = (int)(w % (unsigned)nseg);
+    const int row = (int)(w / (unsigned)nseg);
+    const int y = row % ny, z = row / ny;
+    const long long N = (long long)nx * ny * nz;
+    const int qs = (int)in.qstride;  // (Q - 1) * qstride < 2^31 (validated at creation)
+    const S* __restrict__ fin = static_cast<const S*>(in.f[par]);
+    const float sl = in.s_load;
+    const bool row_in = y >= 1 && y + 1 < ny && (D == 2 || (z >= 1 && z + 1 < nz));
+    float f[NK][Q - 1];
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+        const int xc = (seg * NK + k) * 32;
+        if (xc >= nx) break;
+        const int x = min(xc + lane, nx - 1);  // lanes past the row read a valid node and write nothing
+        if (row_in && xc >= 1 && xc + 32 < nx) {
+            const S* base = fin + (row * pitch + x);
+#pragma unroll
+            for (int q = 1; q < Q; ++q)
+                f[k][q - 1] = VecIO<S, 1 + (sizeof(S) == 2)>::load1(
+                    base + ((q - 1) * qs - (L::c(q, 2) * ny + L::c(q, 1)) * pitch - L::c(q, 0)), sl);
+        } else {
+            pull_pre_all<Q, S>(in, fin, x, y, z, qs, f[k]);
         }
-        if (own >= 0)
-            for (int d = 0; d < 3; ++d) a[d] += in.prec[own].a[d];
     }
-    float m[3] = {0, 0, 0}, s = 0.f;
-    for (int q = 1; q < Q; ++q) {
-        s += f[q - 1];
-        for (int d = 0; d < D; ++d) m[d] += L::c(q, d) * f[q - 1];
+    const Geo geo = make_geo(in);
+    const float gd[3] = {in.gdrive[0], in.gdrive[1], in.gdrive[2]};
+    // the tile of the current chunk (its width is a multiple of 32; usually
+    // one tile holds the whole segment): its candidates, and those of them that
+    // reach the warp's part of the row, looked up while the populations arrive
+    int tile_end = in.np > 0 ? 0 : nx, nc = 0;
+    unsigned act = 0;
+    const Cand* cand = nullptr;
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+        const int xc = (seg * NK + k) * 32;
+        if (xc >= nx) break;
+        const int x = xc + lane;
+        const int xyz[3] = {x, y, z};
+        if (xc >= tile_end) {
+            const int tx = xc / sh.tw;
+            const int local = (z / sh.tz * in.ntile[1] + y / sh.ty) * in.ntile[0] + tx;
+            tile_end = (tx + 1) * sh.tw;
+            nc = min(in.list_cnt[par][local], LIST_CAP);
+            cand = static_cast<const Cand*>(in.list_rec[par]) + (long long)local * LIST_CAP;
+            act = nc == 0 ? 0u : nc > 32 ? 0xffffffffu
+                  : segment_candidates<D>(geo, cand, nc, xc, y, z, min(tile_end, (seg + 1) * NK * 32) - xc, lane);
+        }
+        int own = -1;
+        float a[3] = {gd[0], gd[1], gd[2]};
+        if (act) {
+            int slot = -1;
+            own = nc > 32 ? owner_of<D>(geo, cand, nc, xyz, &slot) : owner_masked<D>(geo, cand, act, xyz, &slot);
+            if (own >= 0)
+#pragma unroll
+                for (int d = 0; d < D; ++d) a[d] += cand[slot].a[d];
+        }
+        float m[3] = {0, 0, 0}, s = 0.f;
+#pragma unroll
+        for (int q = 1; q < Q; ++q) {
+            s += f[k][q - 1];
+#pragma unroll
+            for (int d = 0; d < D; ++d)
+                if (L::c(q, d) != 0) m[d] += L::c(q, d) > 0 ? f[k][q - 1] : -f[k][q - 1];
+        }
+        if (x >= nx) continue;
+        const long long i = (long long)row * nx + x;
+        float uu = 0.f;
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            const float ud = m[d] + 0.5f * a[d];
+            uu += ud * ud;
+            if (u) u[(long long)d * N + i] = ud;
+        }
+        if (pout) pout[i] = (s - (float)(1.5 - 0.5 * L::SUMA) * uu) * (float)(1.0 / L::SUMA);
+        if (owner) owner[i] = own;
     }
-    float uu = 0.f;
-    for (int d = 0; d < D; ++d) {
-        const float ud = m[d] + 0.5f * a[d];
-        uu += ud * ud;
-        if (u) u[(long long)d * N + i] = ud;
-    }
-    if (pout) pout[i] = (s - (float)(1.5 - 0.5 * L::SUMA) * uu) * (float)(1.0 / L::SUMA);
-    if (owner) owner[i] = own;
 }
 
 // populations between the dense [Q][N] FP32 exchange layout and storage
@@ -436,15 +490,22 @@ int fluid_max_blocks_per_sm(int Q, int fp16, const Shape& sh) {
     return 0;
 }
 
-cudaError_t launch_fields(int Q, int fp16, const InstDesc* insts, int inst, long long N, int par,
-                          const Shape& sh, float* u, float* p, int* owner, cudaStream_t st) {
-    const int thr = 256;
-    const unsigned blocks = (unsigned)((N + thr - 1) / thr);
-    if (Q == 9 && !fp16) k_fields<9, float><<<blocks, thr, 0, st>>>(insts, inst, par, sh, u, p, owner);
-    else if (Q == 9) k_fields<9, __half><<<blocks, thr, 0, st>>>(insts, inst, par, sh, u, p, owner);
-    else if (!fp16) k_fields<19, float><<<blocks, thr, 0, st>>>(insts, inst, par, sh, u, p, owner);
-    else k_fields<19, __half><<<blocks, thr, 0, st>>>(insts, inst, par, sh, u, p, owner);
+template <int Q, class S>
+static cudaError_t launch_fields_t(const InstDesc* insts, int inst, const int* n, int par, const Shape& sh, float* u,
+                                   float* p, int* owner, cudaStream_t st) {
+    const int width = 32 * field_chunks<Q>();
+    const int nseg = (n[0] + width - 1) / width;
+    const unsigned nwork = (unsigned)nseg * n[1] * n[2];  // < 2^31: at most 2e9 populations
+    k_fields<Q, S><<<(nwork + 7) / 8, 256, 0, st>>>(insts, inst, par, sh, nseg, nwork, u, p, owner);
     return cudaGetLastError();
+}
+
+cudaError_t launch_fields(int Q, int fp16, const InstDesc* insts, int inst, const int* n, int par,
+                          const Shape& sh, float* u, float* p, int* owner, cudaStream_t st) {
+    if (Q == 9 && !fp16) return launch_fields_t<9, float>(insts, inst, n, par, sh, u, p, owner, st);
+    if (Q == 9) return launch_fields_t<9, __half>(insts, inst, n, par, sh, u, p, owner, st);
+    if (!fp16) return launch_fields_t<19, float>(insts, inst, n, par, sh, u, p, owner, st);
+    return launch_fields_t<19, __half>(insts, inst, n, par, sh, u, p, owner, st);
 }
 
 cudaError_t launch_pack(int Q, int fp16, const InstDesc* insts, int inst, long long N, int par,
