@@ -39,6 +39,10 @@ int fluid_tma_blocks_per_sm(int Q, int fp16, const Shape& sh, int stages, int ni
 cudaError_t launch_fluid_tma(int Q, int fp16, const InstDesc* insts, const void* tmaps,
                              const uint16_t* tile_inst, int ntiles, int par, const Shape& sh,
                              int commit, int grid, int* tile_ctr, int stages, int ninst, cudaStream_t st);
+int direct_tile_width();
+int fluid_direct_blocks_per_sm(int fp16, const Shape& sh);
+cudaError_t launch_fluid_direct(int fp16, const InstDesc* insts, const uint16_t* tile_inst, int ntiles, int par,
+                                const Shape& sh, int commit, cudaStream_t st);
 cudaError_t launch_adj_fluid(int Q, int fp16, const InstDesc* insts, const AdjFluid* afs,
                              const uint16_t* tile_inst, int ntiles, int lam_mode, const Shape& sh,
                              cudaStream_t st);
@@ -475,7 +479,7 @@ int build_tmaps(lbm_ctx* ctx) {
 int configure_shape(lbm_ctx* ctx, const Shape& sh_in) {
     Shape sh = sh_in;
     if (ctx->D == 2) sh.tz = 1;
-    sh.tw = sh.tma ? tma_tile_width(ctx->Q) : 32 * sh.vec;
+    sh.tw = !sh.tma ? 32 * sh.vec : ctx->D == 2 ? tma_tile_width(ctx->Q) : direct_tile_width();
     ctx->shape = sh;
     const int T[3] = {sh.tw, sh.ty, sh.tz};
     int tile0 = 0;
@@ -505,11 +509,12 @@ int configure_shape(lbm_ctx* ctx, const Shape& sh_in) {
     CK(cudaMemcpyAsync(ctx->d_tile_inst.ptr, tab.data(), sizeof(uint16_t) * tab.size(),
                        cudaMemcpyHostToDevice, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));
-    const int occ = sh.tma ? fluid_tma_blocks_per_sm(ctx->Q, ctx->fp16, sh, sh.stages, (int)ctx->inst.size())
-                           : fluid_max_blocks_per_sm(ctx->Q, ctx->fp16, sh);
+    const int occ = !sh.tma ? fluid_max_blocks_per_sm(ctx->Q, ctx->fp16, sh)
+                    : ctx->D == 2 ? fluid_tma_blocks_per_sm(ctx->Q, ctx->fp16, sh, sh.stages, (int)ctx->inst.size())
+                                  : fluid_direct_blocks_per_sm(ctx->fp16, sh);
     if (occ < 1) return set_err(ctx, LBM_ERR_INVALID, "kernel shape does not fit on an SM%s");
     ctx->grid = occ * ctx->num_sms;
-    if (sh.tma && (rc = build_tmaps(ctx))) return rc;
+    if (sh.tma && ctx->D == 2 && (rc = build_tmaps(ctx))) return rc;
     if ((rc = upload_descs(ctx))) return rc;
     invalidate_graphs(ctx);
     return republish(ctx);
@@ -525,18 +530,22 @@ Shape default_shape(int Q, int fp16) {
     return Shape{fp16 ? 4 : 2, 2, 2, 4, 1, 1, 2, 64};
 }
 
-int enqueue_fluid(lbm_ctx* ctx, int commit, cudaStream_t st) {
+// The fluid kernel over the instances of descriptor array insts (tensor maps
+// tmaps, D2Q9 staged path only), reading buffer par.
+int enqueue_fluid_on(lbm_ctx* ctx, const InstDesc* insts, const void* tmaps, int par, int commit, cudaStream_t st) {
     const Shape& sh = ctx->shape;
-    if (sh.tma) {
-        CK(launch_fluid_tma(ctx->Q, ctx->fp16, P<InstDesc>(ctx->d_insts), ctx->d_tmaps.ptr,
-                            P<uint16_t>(ctx->d_tile_inst), ctx->ntiles, ctx->par, sh, commit,
+    if (sh.tma && ctx->D == 2)
+        CK(launch_fluid_tma(ctx->Q, ctx->fp16, insts, tmaps, P<uint16_t>(ctx->d_tile_inst), ctx->ntiles, par, sh, commit,
                             ctx->grid, P<int>(ctx->d_tile_ctr), sh.stages, (int)ctx->inst.size(), st));
-        return LBM_OK;
-    }
-    CK(launch_fluid(ctx->Q, ctx->fp16, P<InstDesc>(ctx->d_insts), P<uint16_t>(ctx->d_tile_inst),
-                    ctx->ntiles, ctx->par, sh, commit, sh.persistent, ctx->grid,
-                    P<int>(ctx->d_tile_ctr), st));
+    else if (sh.tma)
+        CK(launch_fluid_direct(ctx->fp16, insts, P<uint16_t>(ctx->d_tile_inst), ctx->ntiles, par, sh, commit, st));
+    else
+        CK(launch_fluid(ctx->Q, ctx->fp16, insts, P<uint16_t>(ctx->d_tile_inst), ctx->ntiles, par, sh, commit,
+                        sh.persistent, ctx->grid, P<int>(ctx->d_tile_ctr), st));
     return LBM_OK;
+}
+int enqueue_fluid(lbm_ctx* ctx, int commit, cudaStream_t st) {
+    return enqueue_fluid_on(ctx, P<InstDesc>(ctx->d_insts), ctx->d_tmaps.ptr, ctx->par, commit, st);
 }
 int enqueue_fluid(lbm_ctx* ctx, int commit) { return enqueue_fluid(ctx, commit, ctx->st); }
 
@@ -1477,7 +1486,8 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
     // k + 1, its records go to record k (and k + 1 for the next step's input);
     // entry L is the publish of a segment's first state into record 0
     std::vector<InstDesc> rd((size_t)(L + 1) * ni);
-    std::vector<CUtensorMap> tm(sh.tma ? (size_t)L * ni * 2 : 0);
+    const bool tma = sh.tma && ctx->D == 2;  // the fluid kernel reads through tensor maps
+    std::vector<CUtensorMap> tm(tma ? (size_t)L * ni * 2 : 0);
     for (int k = 0; k <= L; ++k)
         for (int i = 0; i < ni; ++i) {
             Instance& I = ctx->inst[i];
@@ -1507,7 +1517,7 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
                 d.list_rec[par ^ 1] = lr + (size_t)CAND_BYTES * I.ntiles * LIST_CAP * (k + 1);
                 d.adj_geo = P<double>(a.rgeo) + NPV * n1 * k;
                 d.rec_state = P<double>(a.rstate) + 16 * n1 * (k + 1);
-                if (sh.tma) {
+                if (tma) {
                     if ((rc = encode_pop_map(ctx, I, a.slot[k].ptr, &tm[(size_t)k * ni * 2 + 2 * i + par]))) return rc;
                     if ((rc = encode_pop_map(ctx, I, a.slot[k + 1].ptr, &tm[(size_t)k * ni * 2 + 2 * i + (par ^ 1)])))
                         return rc;
@@ -1517,7 +1527,7 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
         }
     if ((rc = dalloc(ctx, A.d_rdesc, sizeof(InstDesc) * rd.size()))) return rc;
     CK(cudaMemcpyAsync(A.d_rdesc.ptr, rd.data(), sizeof(InstDesc) * rd.size(), cudaMemcpyHostToDevice, ctx->st));
-    if (sh.tma) {
+    if (tma) {
         if ((rc = dalloc(ctx, A.d_rtmaps, sizeof(CUtensorMap) * tm.size()))) return rc;
         CK(cudaMemcpyAsync(A.d_rtmaps.ptr, tm.data(), sizeof(CUtensorMap) * tm.size(), cudaMemcpyHostToDevice,
                            ctx->st));
@@ -1599,13 +1609,9 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
         for (int k = 0; k < len; ++k) {
             const int par = k & 1;
             const InstDesc* dk = dR + (size_t)k * ni;
-            if (sh.tma)
-                CK(launch_fluid_tma(ctx->Q, ctx->fp16, dk, P<CUtensorMap>(A.d_rtmaps) + (size_t)k * ni * 2,
-                                    P<uint16_t>(ctx->d_tile_inst), ctx->ntiles, par, sh, 1, ctx->grid,
-                                    P<int>(ctx->d_tile_ctr), sh.stages, ni, st));
-            else
-                CK(launch_fluid(ctx->Q, ctx->fp16, dk, P<uint16_t>(ctx->d_tile_inst), ctx->ntiles, par, sh, 1,
-                                sh.persistent, ctx->grid, P<int>(ctx->d_tile_ctr), st));
+            const int err = enqueue_fluid_on(ctx, dk, tma ? P<CUtensorMap>(A.d_rtmaps) + (size_t)k * ni * 2 : nullptr, par,
+                                             1, st);
+            if (err) return err;
             if (ctx->np_total > 0) CK(launch_box_sums(dk, P<PartRef>(ctx->d_refs), ctx->np_total, ctx->D, st));
             if (ctx->np_total > 0)
                 CK(launch_particles(dk, P<PartRef>(ctx->d_refs), ctx->np_total, ctx->D, K, par ^ 1, sh,

@@ -345,7 +345,9 @@ __device__ __forceinline__ float2 cdot2(const float2* v) {
     using L = Lat<Q>;
     constexpr int c0 = L::c(q, 0), c1 = L::c(q, 1), c2 = L::c(q, 2);
     float2 r;
-    if constexpr (c0 != 0) {
+    if constexpr (c0 < 0 && c1 > 0 && c2 == 0) {
+        r = sub2(v[1], v[0]);  // one rounding, like (-v0) + v1
+    } else if constexpr (c0 != 0) {
         r = c0 > 0 ? v[0] : mul2(v[0], bc2(-1.0f));
         if constexpr (c1 != 0) r = c1 > 0 ? add2(r, v[1]) : sub2(r, v[1]);
         if constexpr (c2 != 0) r = c2 > 0 ? add2(r, v[2]) : sub2(r, v[2]);
@@ -589,6 +591,58 @@ __device__ __forceinline__ void collide2(float2* f, const float2* a, bool solid0
     }
 }
 
+// Two fluid nodes without a local acceleration (no particle owns them and the
+// instance has no body force): collide2 with a = 0.  Every forcing term is then
+// an exact zero (F_q = 0, u = m), and adding it rounds nothing, so the
+// populations are the same values as collide2's; leaving the terms out saves
+// about half of the collision's instructions.  Almost every node of a
+// sedimentation run is of this kind.  k is CollK, or with SCALED (tau = 1) the
+// one of collide2_t1_scaled.  Returns u . u (the divergence test).
+template <int Q, int q, bool T1>
+__device__ __forceinline__ void collide_pair2_free(float2* f, const float2* u, float2 base, const CollK& k) {
+    if constexpr (q < Q) {
+        if constexpr (pair_head<Q>(q)) {
+            using L = Lat<Q>;
+            constexpr int qo = L::opp(q);
+            constexpr int cls = (Q == 9 ? q >= 5 : q >= 7) ? 1 : 0;
+            const float2 cu = cdot2<Q, q>(u);
+            const float2 t = fma2(mul2(bc2(1.5f), cu), cu, base);
+            if constexpr (T1) {
+                const float2 At = mul2(bc2(k.A[cls]), t);
+                f[q - 1] = fma2(bc2(k.A[cls]), cu, At);
+                f[qo - 1] = fma2(bc2(-k.A[cls]), cu, At);
+            } else {
+                const float2 eq = add2(t, cu), eo = sub2(t, cu);
+                f[q - 1] = fma2(bc2(k.keep), f[q - 1], mul2(bc2(k.omk), mul2(bc2(k.A[cls]), eq)));
+                f[qo - 1] = fma2(bc2(k.keep), f[qo - 1], mul2(bc2(k.omk), mul2(bc2(k.A[cls]), eo)));
+            }
+        }
+        collide_pair2_free<Q, q + 1, T1>(f, u, base, k);
+    }
+}
+template <int Q, bool SCALED>
+__device__ __forceinline__ float2 collide2_free(float2* f, const CollK& k, float sload) {
+    using L = Lat<Q>;
+    constexpr int D = L::D;
+    constexpr float inv_sa = (float)(1.0 / L::SUMA);
+    constexpr float kuu = (float)(1.5 - 0.5 * L::SUMA);
+    float2 s, u[3];
+    moments2<Q>(f, s, u);
+    if constexpr (SCALED) {
+        s = mul2(s, bc2(sload));
+        u[0] = mul2(u[0], bc2(sload));
+        u[1] = mul2(u[1], bc2(sload));
+        if (D == 3) u[2] = mul2(u[2], bc2(sload));
+    }
+    const float2 uu = D == 3 ? fma2(u[2], u[2], fma2(u[1], u[1], mul2(u[0], u[0])))
+                             : fma2(u[1], u[1], mul2(u[0], u[0]));
+    const float2 p = mul2(fma2(bc2(-kuu), uu, s), bc2(inv_sa));  // Eq. 15b
+    const float2 base = fma2(bc2(-0.5f), uu, p);
+    if (SCALED || k.keep == 0.f) collide_pair2_free<Q, 1, true>(f, u, base, k);
+    else collide_pair2_free<Q, 1, false>(f, u, base, k);
+    return uu;
+}
+
 // FP16 storage at tau = 1: f holds the populations at the storage scale
 // (2^14 f, as read, without the 2^-14 multiply), and ks is CollK with A, fA
 // and sA multiplied by 2^14, so f* comes out at the storage scale too.  The
@@ -711,6 +765,84 @@ __device__ __forceinline__ void box_store(float* ubox, const Geo& g, const Cand&
         reinterpret_cast<float4*>(ubox)[cd.boff + ((long long)dz * side + dy) * side + dx] =
             make_float4(ux, uy, uz, 0.f);
     }
+}
+
+// The rest of a fused step for two adjacent nodes (x, x + 1) of a row, x even,
+// one pair per lane of a converged warp whose 64 nodes start at xseg: owner,
+// collision, store and the solid nodes' velocities.  f: the pulled
+// populations (at the storage scale with FOLD); out: population 1 of node x in
+// the new buffer.  Env gives the instance (n, per, prec, gdrive, ubox).
+// Returns whether a velocity left the stable range.
+template <int Q, class S, bool FOLD, class Env>
+__device__ __forceinline__ bool finish_pair(const Env& e, float2* f, const CollK& ck, float sload, float sstore, bool free,
+                                            const Cand* cand, int ncand, int xseg, int x, int y, int z, int lane,
+                                            S* out, int qs) {
+    using L = Lat<Q>;
+    constexpr int D = L::D;
+    constexpr int QS = Q - 1;
+    const bool v0 = x < e.n(0), v1 = x + 1 < e.n(0);
+    int own0 = -1, own1 = -1, sl0 = -1, sl1 = -1;
+    auto geo_of = [&]() {
+        Geo g;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            g.n[d] = e.n(d);
+            g.per[d] = e.per(d);
+        }
+        g.prec = e.prec();
+        return g;
+    };
+    if (ncand > 0) {
+        const Geo geo = geo_of();
+        const int xyz0[3] = {x, y, z}, xyz1[3] = {x + 1, y, z};
+        if (ncand > 32) {  // more candidates than mask bits: test them all
+            own0 = owner_of<D>(geo, cand, ncand, xyz0, &sl0);
+            own1 = owner_of<D>(geo, cand, ncand, xyz1, &sl1);
+        } else {
+            const unsigned act = segment_candidates<D>(geo, cand, ncand, xseg, y, z, 64, lane);
+            if (act) {
+                own0 = owner_masked<D>(geo, cand, act, xyz0, &sl0);
+                own1 = owner_masked<D>(geo, cand, act, xyz1, &sl1);
+            }
+        }
+    }
+    float2 uu, u[3];
+    const bool solid = own0 >= 0 || own1 >= 0;
+    if (free && !__any_sync(0xffffffffu, solid)) {
+        uu = collide2_free<Q, FOLD>(f, ck, sload);
+    } else {
+        float2 a[3], p;
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            a[d] = add2(bc2(e.gdrive(d)),
+                        make_float2(own0 >= 0 ? cand[sl0].a[d] : 0.f, own1 >= 0 ? cand[sl1].a[d] : 0.f));
+        if constexpr (FOLD) collide2_t1_scaled<Q>(f, a, own0 >= 0, own1 >= 0, ck, sload, u, &p);
+        else collide2<Q>(f, a, own0 >= 0, own1 >= 0, ck, u, &p);
+        uu = mul2(u[0], u[0]);
+#pragma unroll
+        for (int d = 1; d < D; ++d) uu = fma2(u[d], u[d], uu);
+    }
+    if (v1) {
+#pragma unroll
+        for (int q = 0; q < QS; ++q) {
+            if constexpr (FOLD) *reinterpret_cast<__half2*>(out) = __floats2half2_rn(f[q].x, f[q].y);
+            else store_pair(out, f[q], sstore);
+            out += qs;
+        }
+    } else if (v0) {
+#pragma unroll
+        for (int q = 0; q < QS; ++q) {
+            if constexpr (FOLD) *out = __float2half_rn(f[q].x);
+            else *out = to_store<S>(f[q].x, sstore);
+            out += qs;
+        }
+    }
+    if (solid) {  // the solid nodes' velocities into their particles' boxes (Eq. 22)
+        const Geo geo = geo_of();
+        if (v0 && own0 >= 0) box_store<D>(e.ubox(), geo, cand[sl0], x, y, z, u[0].x, u[1].x, D == 3 ? u[2].x : 0.f);
+        if (v1 && own1 >= 0) box_store<D>(e.ubox(), geo, cand[sl1], x + 1, y, z, u[0].y, u[1].y, D == 3 ? u[2].y : 0.f);
+    }
+    return (v0 && !(uu.x < 0.25f)) || (v1 && !(uu.y < 0.25f));
 }
 
 // ----------------------------------------------- per-particle finalisation --

@@ -1,0 +1,168 @@
+// Fused stream-collide-penalize kernel for D3Q19: loads straight into
+// registers, one warp per 64-node row of a tile.
+//
+// Pull streaming reads every population value once, so staging a D3Q19 tile
+// through shared memory saves no traffic, and its tensor copies are small (18
+// boxes of a few 64-node rows): the copy engine, not HBM, set the time of the
+// staged kernel (FP32 and FP16 storage took the same time per node).  Here a
+// lane takes two adjacent nodes: populations with c_x = 0 arrive by one
+// 8-byte (FP16: 4-byte) load, the others by two scalar loads of the shifted
+// pair; all 18 are in flight before the first is used, and enough warps are
+// resident to cover the latency.  Rows at a y or z face take pull_pre_all;
+// the x faces only change the address of an edge node's load.
+// 256 x 256 x 512, 8 spheres, the kernel alone: FP32 1.28 -> 0.905 ms (5.3 TB/s),
+// FP16 storage 1.28 -> 0.78 ms; 128 threads of 4 rows each against 8 rows per
+// 4 warps: 0.83 ms.
+#include "lbm_common.cuh"
+
+namespace lbmpen {
+
+namespace {
+
+constexpr int TW = 64;
+
+struct DescEnv {
+    const InstDesc& in;
+    float* box;
+    __device__ __forceinline__ int n(int d) const { return in.n[d]; }
+    __device__ __forceinline__ int per(int d) const { return in.periodic[d]; }
+    __device__ __forceinline__ const PRec* prec() const { return in.prec; }
+    __device__ __forceinline__ float gdrive(int d) const { return in.gdrive[d]; }
+    __device__ __forceinline__ float* ubox() const { return box; }
+};
+
+template <class S> __device__ __forceinline__ float load_one(const S* p, float s) {
+    return VecIO<S, 1 + (sizeof(S) == 2)>::load1(p, s);
+}
+__device__ __forceinline__ float2 load_pair(const float* p, float) { return __ldg(reinterpret_cast<const float2*>(p)); }
+__device__ __forceinline__ float2 load_pair(const __half* p, float s) {
+    const unsigned int t = __ldg(reinterpret_cast<const unsigned int*>(p));
+    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&t));
+    return make_float2(a.x * s, a.y * s);
+}
+
+// Populations of nodes x, x + 1 (x even) of a row whose y and z sources lie
+// inside the box; EDGE: the warp's nodes include x = 0 or reach x = nx - 1, so
+// the shifted loads of those nodes come from across the x face (bounce-back at
+// a wall, plus its term; the far column on a periodic axis).  Lanes past nx
+// read valid nodes, and their values are not stored.
+template <int Q, class S, bool EDGE>
+__device__ __forceinline__ void pull_pair(const InstDesc& in, const S* __restrict__ fin, int x, int y, int z, float2* f) {
+    using L = Lat<Q>;
+    const int nx = in.n[0], pitch = in.pitch, zs = in.n[1] * pitch, qs = (int)in.qstride;
+    const float sl = in.s_load;
+    const int own = z * zs + y * pitch;
+    const bool wall = !in.periodic[0];
+#pragma unroll
+    for (int q = 1; q < Q; ++q) {
+        const int cx = L::c(q, 0);
+        const int row = (q - 1) * qs + own - L::c(q, 2) * zs - L::c(q, 1) * pitch;
+        if (cx == 0) {
+            f[q - 1] = load_pair(fin + (row + (EDGE && x >= nx ? 0 : x)), sl);
+        } else if constexpr (!EDGE) {
+            f[q - 1] = make_float2(load_one(fin + (row + x - cx), sl), load_one(fin + (row + x + 1 - cx), sl));
+        } else {
+            float v[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int xe = min(x + e, nx - 1), xs = xe - cx;
+                const bool out = cx > 0 ? xs < 0 : xs >= nx;
+                const int face = cx > 0 ? 0 : 1;
+                const int off = !out ? row + xs : wall ? (L::opp(q) - 1) * qs + own + xe : row + (cx > 0 ? nx - 1 : 0);
+                const float term = __ldg(&in.wterm[0][face][q]);  // always: no load waits on a condition
+                const float w = load_one(fin + off, sl);
+                v[e] = out && wall ? w + term : w;
+            }
+            f[q - 1] = make_float2(v[0], v[1]);
+        }
+    }
+}
+
+}  // namespace
+
+template <int Q, class S>
+__global__ void __launch_bounds__(256, 2) k_fluid_direct(const InstDesc* __restrict__ insts,
+                                                         const uint16_t* __restrict__ tile_inst, int par, Shape sh,
+                                                         int commit) {
+    using L = Lat<Q>;
+    constexpr int D = L::D;
+    constexpr int QS = Q - 1;
+    __shared__ Cand cand[LIST_CAP];
+    const int t = blockIdx.x;
+    const InstDesc& in = insts[tile_inst[t]];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int local = t - in.tile0;
+    const int ntx = in.ntile[0], nty = in.ntile[1];
+    const int rest = local / ntx;
+    const int x0 = (local - rest * ntx) * TW, y0 = (rest % nty) * sh.ty, z0 = (rest / nty) * sh.tz;
+    const int nx = in.n[0], ny = in.n[1], nz = in.n[2];
+    const int rows = sh.ty * sh.tz, lty = __ffs(sh.ty) - 1;  // tile rows along y: a power of two
+    const int x = x0 + 2 * lane;
+    const bool edge = x0 == 0 || x0 + TW >= nx;
+    const float sload = in.s_load;
+    const S* __restrict__ fin = static_cast<const S*>(in.f[par]);
+    float2 f[QS];
+    auto pull_row = [&](int r) {  // false: the row lies beyond the box
+        const int y = y0 + (r & (sh.ty - 1)), z = z0 + (r >> lty);
+        if (r >= rows || y >= ny || z >= nz) return false;
+        if (y >= 1 && y + 1 < ny && (D == 2 || (z >= 1 && z + 1 < nz))) {
+            if (edge) pull_pair<Q, S, true>(in, fin, x, y, z, f);
+            else pull_pair<Q, S, false>(in, fin, x, y, z, f);
+        } else {
+            float g[QS];
+            pull_pre_all<Q, S>(in, fin, min(x, nx - 1), y, z, (int)in.qstride, g);
+#pragma unroll
+            for (int q = 0; q < QS; ++q) f[q].x = g[q];
+            pull_pre_all<Q, S>(in, fin, min(x + 1, nx - 1), y, z, (int)in.qstride, g);
+#pragma unroll
+            for (int q = 0; q < QS; ++q) f[q].y = g[q];
+        }
+        return true;
+    };
+    // the first row's populations are in flight while the candidates arrive
+    int r = warp;
+    bool have = pull_row(r);
+    int ncand = 0;
+    if (in.np > 0) {
+        ncand = min(in.list_cnt[par][local], LIST_CAP);
+        const uint4* src = reinterpret_cast<const uint4*>(static_cast<const Cand*>(in.list_rec[par]) +
+                                                          (long long)local * LIST_CAP);
+        for (int i = threadIdx.x; i < ncand * (CAND_BYTES / 16); i += blockDim.x) reinterpret_cast<uint4*>(cand)[i] = src[i];
+        if (commit && threadIdx.x == 0) in.list_cnt[par ^ 1][local] = 0;  // the next step's list starts empty
+        __syncthreads();
+    }
+    const CollK ck = make_collk<Q>(make_collp(in));
+    const bool free = in.gdrive[0] == 0.f && in.gdrive[1] == 0.f && in.gdrive[2] == 0.f;
+    const DescEnv env{in, commit ? in.ubox : in.ubox_scratch};
+    S* __restrict__ fout = static_cast<S*>(in.f[par ^ 1]);
+    bool bad = false;
+    for (;;) {
+        if (have) {
+            const int y = y0 + (r & (sh.ty - 1)), z = z0 + (r >> lty);
+            bad |= finish_pair<Q, S, false>(env, f, ck, sload, in.s_store, free, cand, ncand, x0, x, y, z, lane,
+                                            fout + ((z * ny + y) * in.pitch + x), (int)in.qstride);
+        }
+        r += nwarps;
+        if (r >= rows) break;
+        have = pull_row(r);
+    }
+    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(in.status, ST_DIVERGED);
+}
+
+int direct_tile_width() { return TW; }
+
+int fluid_direct_blocks_per_sm(int fp16, const Shape& sh) {
+    int nb = 0;
+    if (fp16) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_fluid_direct<19, __half>, 32 * sh.warps, 0);
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_fluid_direct<19, float>, 32 * sh.warps, 0);
+    return nb;
+}
+
+cudaError_t launch_fluid_direct(int fp16, const InstDesc* insts, const uint16_t* tile_inst, int ntiles, int par,
+                                const Shape& sh, int commit, cudaStream_t st) {
+    if (fp16) k_fluid_direct<19, __half><<<ntiles, 32 * sh.warps, 0, st>>>(insts, tile_inst, par, sh, commit);
+    else k_fluid_direct<19, float><<<ntiles, 32 * sh.warps, 0, st>>>(insts, tile_inst, par, sh, commit);
+    return cudaGetLastError();
+}
+
+}  // namespace lbmpen

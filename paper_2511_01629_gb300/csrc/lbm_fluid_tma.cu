@@ -123,6 +123,7 @@ struct __align__(16) TInst {
     int tile0, ntx, nty, pitch, np, maxk;
     int n[3], per[3];
     float gdrive[3], sload, sstore, keep, fpref, alpha;
+    int free;                  // no body force: fluid nodes take collide2_free
     float ewt[2][5];           // moving-wall term of the populations an x-edge node pulls
                                //   across the low (0) / high (1) x face
 };
@@ -157,6 +158,7 @@ __device__ __forceinline__ void make_tinst(TInst& t, const InstDesc& in) {
     t.keep = in.keep;
     t.fpref = in.fpref;
     t.alpha = in.alpha;
+    t.free = in.gdrive[0] == 0.f && in.gdrive[1] == 0.f && in.gdrive[2] == 0.f;
     for (int face = 0; face < 2; ++face)
         for (int k = 0; k < 5; ++k) t.ewt[face][k] = 0.f;
     for (int face = 0; face < 2; ++face) {  // face 0 is pulled across by c_x = +1, face 1 by c_x = -1
@@ -166,6 +168,17 @@ __device__ __forceinline__ void make_tinst(TInst& t, const InstDesc& in) {
     }
 }
 
+// What finish_pair needs of the instance, read from the shared copy when it does.
+struct TileEnv {
+    const TInst& ti;
+    float* box;
+    __device__ __forceinline__ int n(int d) const { return ti.n[d]; }
+    __device__ __forceinline__ int per(int d) const { return ti.per[d]; }
+    __device__ __forceinline__ const PRec* prec() const { return ti.prec; }
+    __device__ __forceinline__ float gdrive(int d) const { return ti.gdrive[d]; }
+    __device__ __forceinline__ float* ubox() const { return box; }
+};
+
 // Per-tile record the producer writes next to the staged populations.
 struct __align__(16) StageHdr {
     TInst ti;   // the tile's instance
@@ -173,25 +186,23 @@ struct __align__(16) StageHdr {
     int ncand;
     int inst;
     int x0, y0, z0;
-    int ex;     // x of the tile's edge node whose face values are staged, -1 none,
-                //   -2 both edges in one tile (those take the direct gathers)
-    int ecx;    // c_x of the staged populations: +1 at x = 0, -1 at x = nx - 1
+    int ex;     // bit 0: the tile holds x = 0, bit 1: it holds x = nx - 1 (the values
+                //   these nodes pull across the face are staged, side by side)
 };
 
-// The next tile of the producer, prepared one iteration ahead: its place,
-// its list count (lane 0) and the values its x-edge node pulls across the face
-// (two per lane, loads in flight while the producer waits for a free stage).
 // The next tile of the producer, prepared one iteration ahead: its place in
-// registers; its list count and the values its x-edge node pulls across the
-// face in flight to the shared prefetch buffer (cp.async) while the producer
+// registers; its list count and the values its x-edge nodes pull across the
+// faces in flight to the shared prefetch buffer (cp.async) while the producer
 // waits for a free stage.
+constexpr int EDGE_ITERS = 3;  // edge values per lane: 2 sides x 8 rows x 5 populations at most
 struct TileAhead {
-    int t, ii, local, x0, y0, z0, ex, ecx, np;
+    int t, ii, local, x0, y0, z0, ex, np;
     float sload;
-    float add[2];
+    float add[EDGE_ITERS];
     int hsel;  // FP16: bit j set = value j is the upper half of its 4-byte word
 };
-constexpr int PRE_WORDS = 72;  // per prefetch buffer: 64 edge values, the list count
+constexpr int PRE_WORDS = 32 * EDGE_ITERS + 8;  // per prefetch buffer: edge values, the list count
+constexpr int PRE_CNT = 32 * EDGE_ITERS;
 
 }  // namespace
 
@@ -224,7 +235,7 @@ __host__ __device__ inline TmaLayout tma_layout(int Q, int ssize, int tw, int ro
     L.hdr_off = L.pops_bytes;
     L.cand_off = L.hdr_off + (int)sizeof(StageHdr) * stages;  // 16-byte aligned (bulk copies)
     L.edge_off = L.cand_off + CAND_BYTES * LIST_CAP * stages;
-    L.tab_off = (L.edge_off + (int)sizeof(float) * rows * edge_pops(Q) * stages + 15) & ~15;
+    L.tab_off = (L.edge_off + (int)sizeof(float) * 2 * rows * edge_pops(Q) * stages + 15) & ~15;
     L.pre_off = L.tab_off + (int)sizeof(TInst) * ntab;
     L.bar_off = L.pre_off + 4 * 2 * PRE_WORDS;
     L.bytes = L.bar_off + 16 * stages + 128;  // + alignment slack of the base
@@ -268,7 +279,7 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
     const TmaLayout LY = tma_layout(Q, (int)sizeof(S), TW, rows, stages, ninst);
     StageHdr* hdr = reinterpret_cast<StageHdr*>(smem + LY.hdr_off);
     Cand* cands = reinterpret_cast<Cand*>(smem + LY.cand_off);
-    float* edgev = reinterpret_cast<float*>(smem + LY.edge_off);  // [stages][rows][QE]
+    float* edgev = reinterpret_cast<float*>(smem + LY.edge_off);  // [stages][side][rows][QE]
     TInst* tab = reinterpret_cast<TInst*>(smem + LY.tab_off);
     uint32_t* pre = reinterpret_cast<uint32_t*>(smem + LY.pre_off);  // [2][PRE_WORDS]
     constexpr int QE = edge_pops(Q);
@@ -277,6 +288,7 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nc = (blockDim.x >> 5) - 1;  // consumer warps
     const int ntab = ninst < TI_MAX ? ninst : TI_MAX;
+    const int lty = __ffs(sh.ty) - 1;  // tile rows along y: a power of two
     if (threadIdx.x == 0) {
         for (int s = 0; s < stages; ++s) {
             mbar_init(&full[s], 1);
@@ -309,10 +321,10 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
             TileAhead a;
             a.t = -1;
             a.np = 0;
-            a.ex = -1;
-            a.ecx = 1;
+            a.ex = 0;
             a.sload = 1.f;
-            a.add[0] = a.add[1] = 0.f;
+#pragma unroll
+            for (int j = 0; j < EDGE_ITERS; ++j) a.add[j] = 0.f;
             a.hsel = 0;
             uint32_t* pb = pre + buf * PRE_WORDS;
             const int cc = __shfl_sync(0xffffffffu, c, 0);
@@ -337,36 +349,36 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
             a.y0 = (rest % nty) * sh.ty;
             a.z0 = (rest / nty) * sh.tz;
             if (lane == 0) {
-                if (a.np > 0) cp_async4(pb + 64, (tb ? tab[a.ii].lcnt[par] : in.list_cnt[par]) + a.local);
-                else pb[64] = 0u;
+                if (a.np > 0) cp_async4(pb + PRE_CNT, (tb ? tab[a.ii].lcnt[par] : in.list_cnt[par]) + a.local);
+                else pb[PRE_CNT] = 0u;
             }
-            const bool eleft = a.x0 == 0, eright = a.x0 + TW >= n[0];
-            a.ex = eleft && eright ? -2 : eleft ? 0 : eright ? n[0] - 1 : -1;
-            a.ecx = eleft ? 1 : -1;
-            if (a.ex >= 0) {
-                // the value edge node x = ex pulls across its x face in a row whose
-                // other sources lie inside the box (rows that do not use it may
-                // get any in-bounds value)
+            a.ex = (a.x0 == 0 ? 1 : 0) | (a.x0 + TW >= n[0] ? 2 : 0);
+            if (a.ex) {
+                // the values the edge nodes x = 0 (side 0) and x = n - 1 (side 1) pull
+                // across their x face in rows whose other sources lie inside the box
+                // (rows that do not use them may get any in-bounds value)
                 const S* fin = static_cast<const S*>(tb ? tab[a.ii].f[par] : in.f[par]);
                 const long long qstr = tb ? tab[a.ii].qstride : in.qstride;
                 const int pitch = tb ? tab[a.ii].pitch : in.pitch;
                 const bool xper = (tb ? tab[a.ii].per[0] : in.periodic[0]) != 0;
-                const int face = a.ecx > 0 ? 0 : 1;
 #pragma unroll
-                for (int j = 0; j < 2; ++j) {
+                for (int j = 0; j < (2 * ROWS * QE + 31) / 32; ++j) {
                     const int l = lane + 32 * j;
-                    if (l >= rows * QE) continue;
-                    const int r = l / QE, k = l % QE;
-                    const int q = edge_pop<Q>(a.ecx, k);
-                    const int y = a.y0 + r % sh.ty, z = a.z0 + r / sh.ty;
+                    if (l >= 2 * rows * QE) continue;
+                    const int side = l >= rows * QE ? 1 : 0;
+                    if (!((a.ex >> side) & 1)) continue;
+                    const int r = (l - side * rows * QE) / QE, k = (l - side * rows * QE) % QE;
+                    const int ecx = side ? -1 : 1, xe = side ? n[0] - 1 : 0;
+                    const int q = edge_pop<Q>(ecx, k);
+                    const int y = a.y0 + (r & (sh.ty - 1)), z = a.z0 + (r >> lty);
                     const int ys = y - L::c(q, 1), zs = z - L::c(q, 2);
                     const S* src = nullptr;
                     if (!xper) {  // bounce-back at the x wall
                         if (y < n[1] && z < n[2])
-                            src = fin + (long long)(L::opp(q) - 1) * qstr + ((long long)z * n[1] + y) * pitch + a.ex;
-                        a.add[j] = tb ? tab[a.ii].ewt[face][k] : in.wterm[0][face][q];
+                            src = fin + (long long)(L::opp(q) - 1) * qstr + ((long long)z * n[1] + y) * pitch + xe;
+                        a.add[j] = tb ? tab[a.ii].ewt[side][k] : in.wterm[0][side][q];
                     } else if (y < n[1] && z < n[2] && ys >= 0 && ys < n[1] && zs >= 0 && zs < n[2]) {
-                        const int xs = a.ecx > 0 ? n[0] - 1 : 0;  // periodic wrap
+                        const int xs = side ? 0 : n[0] - 1;  // periodic wrap
                         src = fin + (long long)(q - 1) * qstr + ((long long)zs * n[1] + ys) * pitch + xs;
                     }
                     if (src) {
@@ -400,7 +412,7 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
             }
             cp_async_wait_all();  // this tile's count and edge values, copied one iteration ago
             __syncwarp();
-            const int ncand = min((int)pb[64], LIST_CAP);
+            const int ncand = min((int)pb[PRE_CNT], LIST_CAP);
             StageHdr& h = hdr[s];
             if (lane == 0) {
                 const CUtensorMap* map = tmaps + 2 * a.ii + par;
@@ -429,12 +441,12 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
             } else if (lane == 0) {
                 make_tinst<Q>(h.ti, insts[a.ii]);
             }
-            if (a.ex >= 0) {
-                float* ev = edgev + s * rows * QE;
+            if (a.ex) {
+                float* ev = edgev + s * 2 * rows * QE;
 #pragma unroll
-                for (int j = 0; j < 2; ++j) {
+                for (int j = 0; j < (2 * ROWS * QE + 31) / 32; ++j) {
                     const int l = lane + 32 * j;
-                    if (l < rows * QE) {
+                    if (l < 2 * rows * QE && ((a.ex >> (l >= rows * QE ? 1 : 0)) & 1)) {
                         const uint32_t w = pb[l];
                         float v;
                         if (sizeof(S) == 2) {
@@ -455,7 +467,6 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
                 h.z0 = a.z0;
                 h.ncand = ncand;
                 h.ex = a.ex;
-                h.ecx = a.ecx;
                 if (commit && a.np > 0)  // this tile's list of the next step starts empty
                     (ninst <= TI_MAX ? tab[a.ii].lcnt[par ^ 1] : insts[a.ii].list_cnt[par ^ 1])[a.local] = 0;
             }
@@ -500,58 +511,51 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
         const StageHdr& h = hdr[s];
         const int ncand = h.ncand;
         const Cand* cand = cands + s * LIST_CAP;
-        Geo geo;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            geo.n[d] = h.ti.n[d];
-            geo.per[d] = h.ti.per[d];
-        }
-        geo.prec = h.ti.prec;
         const int nx = h.ti.n[0], ny = h.ti.n[1], nz = h.ti.n[2];
         const float sload = h.ti.sload;
         const CollK ck = make_collk<Q>(CollP{h.ti.keep, h.ti.fpref, h.ti.alpha});
-        float* const ubox = h.ti.ubox[commit ? 0 : 1];
         const int x0 = h.x0, y0 = h.y0, z0 = h.z0;
         const S* stage = reinterpret_cast<const S*>(smem + s * LY.stage);
-        const int ex = h.ex, ecx = h.ecx;
-        const float* ev = edgev + s * rows * QE;
+        const int ex = h.ex;
+        const bool free = h.ti.free != 0;
+        const TileEnv env{h.ti, h.ti.ubox[commit ? 0 : 1]};
+        const float* ev = edgev + s * 2 * rows * QE;
         bool bad = false;
-        const float sstore_t = h.ti.sstore;
         // FOLD (D2Q9, FP16 storage at tau = 1): the populations stay at the
         // storage scale from the stage to the store (collide2_t1_scaled)
         auto tile_rows = [&](auto fold_tag) {
             constexpr bool FOLD = decltype(fold_tag)::value;
+            const float sstore = h.ti.sstore;
             CollK cks = ck;
             if constexpr (FOLD) {
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
-                    cks.A[i] *= sstore_t;
-                    cks.fA[i] *= sstore_t;
-                    cks.sA[i] *= sstore_t;
+                    cks.A[i] *= sstore;
+                    cks.fA[i] *= sstore;
+                    cks.sA[i] *= sstore;
                 }
             }
             for (int r = cw; r < rows; r += nc) {
-                const int y = y0 + r % sh.ty, z = z0 + r / sh.ty;
+                const int y = y0 + (r & (sh.ty - 1)), z = z0 + (r >> lty);
                 if (y >= ny || z >= nz) continue;
-                // populations whose source row lies inside the staged box
-                unsigned rowok = 0;
-#pragma unroll
-                for (int q = 1; q < Q; ++q) {
-                    const int ys = y - L::c(q, 1), zs = z - L::c(q, 2);
-                    if (ys >= 0 && ys < ny && zs >= 0 && zs < nz) rowok |= 1u << q;
-                }
-                const bool rowfast = rowok == (((1u << Q) - 1) & ~1u);
+                // every source row lies inside the box (and so in the stage), or (D2Q9)
+                // beyond a y wall: then the node's own opposite population, staged
+                // too, comes back
+                const bool lo_y = y < 1, hi_y = y + 1 >= ny;
+                const bool rowfast = D == 2 ? !(lo_y || hi_y) || !h.ti.per[1]
+                                            : !(lo_y || hi_y) && z >= 1 && z + 1 < nz;
                 const S* rowbase = stage + r * BW + H;
                 // element of population q's source row in the stage, relative to rowbase
                 auto qoff = [&](int q) { return (q - 1) * SLAB + (Q == 9 ? (1 - L::c(q, 1)) * BW : 0); };
+                auto beyond_y = [&](int q) { return D == 2 && (L::c(q, 1) > 0 ? lo_y : L::c(q, 1) < 0 && hi_y); };
                 S* outrow = static_cast<S*>(const_cast<void*>(h.ti.f[par ^ 1])) + ((long long)z * ny + y) * h.ti.pitch;
                 // two adjacent nodes per lane: packed FP32x2 arithmetic, 8-byte stores
                 for (int j = 0; j < TW / 64; ++j) {
                     const int lx = j * 64 + 2 * lane;
                     const int x = x0 + lx;
-                    const bool v0 = x < nx, v1 = x + 1 < nx;
+                    if (x0 + j * 64 >= nx) break;  // ragged tile: nothing left in this row
                     float2 f[QS];
-                    if (rowfast && (ex >= 0 || __all_sync(0xffffffffu, x > 0 && x + 1 < nx - 1))) {
+                    if (rowfast) {
 #pragma unroll
                         for (int q = 1; q < Q; ++q) {
                             const S* src = rowbase + qoff(q) + lx - L::c(q, 0);
@@ -565,93 +569,59 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
                                                            to_float_scaled(src[1], sload));
                             }
                         }
-                        // the edge node's populations from across the face (the box
-                        // holds zero fill or a neighbour column there); nodes past
-                        // nx in a ragged tile are computed but never stored
-                        const int e = ex - x;
-                        if (ex >= 0 && (e == 0 || e == 1)) {
-                            int k = 0;
+                        if (D == 2 && (lo_y || hi_y)) {  // bounce-back at the y walls (Eq. 10)
 #pragma unroll
                             for (int q = 1; q < Q; ++q) {
-                                if (L::c(q, 0) != 1 && L::c(q, 0) != -1) continue;
-                                if (L::c(q, 0) != ecx) continue;
-                                const float vv = FOLD ? ev[r * QE + k] * sstore_t : ev[r * QE + k];
-                                ++k;
-                                if (e == 0) f[q - 1].x = vv;
-                                else f[q - 1].y = vv;
+                                const int cy = L::c(q, 1);
+                                if (!(cy > 0 ? lo_y : cy < 0 && hi_y)) continue;
+                                const float wt = __ldg(&insts[h.inst].wterm[1][cy > 0 ? 0 : 1][q]);
+                                const float2 v = smem_pair(rowbase + (L::opp(q) - 1) * SLAB + BW + lx, sload);
+                                f[q - 1] = make_float2(v.x + wt, v.y + wt);
+                                if constexpr (FOLD) f[q - 1] = make_float2(f[q - 1].x * sstore, f[q - 1].y * sstore);
+                            }
+                        }
+                        // the edge nodes' populations from across the x faces (the box
+                        // holds zero fill or a neighbour column there); nodes past
+                        // nx in a ragged tile are computed but never stored
+                        if (ex) {
+                            if ((ex & 1) && x == 0) {
+                                int k = 0;
+#pragma unroll
+                                for (int q = 1; q < Q; ++q)
+                                    if (L::c(q, 0) == 1) {
+                                        const float vv = FOLD ? ev[r * QE + k] * sstore : ev[r * QE + k];
+                                        ++k;
+                                        if (!beyond_y(q)) f[q - 1].x = vv;
+                                    }
+                            }
+                            const int e = nx - 1 - x;
+                            if ((ex & 2) && (e == 0 || e == 1)) {
+                                int k = 0;
+#pragma unroll
+                                for (int q = 1; q < Q; ++q)
+                                    if (L::c(q, 0) == -1) {
+                                        const float vv = FOLD ? ev[(rows + r) * QE + k] * sstore : ev[(rows + r) * QE + k];
+                                        ++k;
+                                        if (beyond_y(q)) continue;
+                                        if (e == 0) f[q - 1].x = vv;
+                                        else f[q - 1].y = vv;
+                                    }
                             }
                         }
                     } else {
+                        // a row at a y or z face: every population straight from the
+                        // previous buffer (L2 holds it), all loads in flight
+                        const S* fin = static_cast<const S*>(h.ti.f[par]);
+                        float g[QS];
+                        pull_pre_all<Q, S>(insts[h.inst], fin, min(x, nx - 1), y, z, (int)h.ti.qstride, g);
 #pragma unroll
-                        for (int q = 1; q < Q; ++q) {
-                            const int cx = L::c(q, 0);
-                            float v[2];
+                        for (int q = 0; q < QS; ++q) f[q].x = FOLD ? g[q] * sstore : g[q];
+                        pull_pre_all<Q, S>(insts[h.inst], fin, min(x + 1, nx - 1), y, z, (int)h.ti.qstride, g);
 #pragma unroll
-                            for (int e = 0; e < 2; ++e) {
-                                const int xe = x + e;
-                                if (((rowok >> q) & 1u) && xe - cx >= 0 && xe - cx < nx) {
-                                    if constexpr (FOLD) v[e] = __half2float(rowbase[qoff(q) + lx + e - cx]);
-                                    else v[e] = to_float_scaled(rowbase[qoff(q) + lx + e - cx], sload);
-                                } else {
-                                    const S* fin = static_cast<const S*>(h.ti.f[par]);
-                                    v[e] = xe < nx ? pull_scalar<Q, S>(insts[h.inst], fin, q, xe, y, z) : 0.f;
-                                    if constexpr (FOLD) v[e] *= sstore_t;
-                                }
-                            }
-                            f[q - 1] = make_float2(v[0], v[1]);
-                        }
+                        for (int q = 0; q < QS; ++q) f[q].y = FOLD ? g[q] * sstore : g[q];
                     }
-                    const int xyz0[3] = {x, y, z}, xyz1[3] = {x + 1, y, z};
-                    int own0 = -1, own1 = -1, sl0 = -1, sl1 = -1;
-                    unsigned act = 0;
-                    if (ncand > 32) {  // more candidates than mask bits: test them all
-                        act = 0xffffffffu;
-                        own0 = owner_of<D>(geo, cand, ncand, xyz0, &sl0);
-                        own1 = owner_of<D>(geo, cand, ncand, xyz1, &sl1);
-                    } else if (ncand > 0) {
-                        act = segment_candidates<D>(geo, cand, ncand, x0 + j * 64, y, z, 64, lane);
-                        if (act) {
-                            own0 = owner_masked<D>(geo, cand, act, xyz0, &sl0);
-                            own1 = owner_masked<D>(geo, cand, act, xyz1, &sl1);
-                        }
-                    }
-                    float2 a[3];
-#pragma unroll
-                    for (int d = 0; d < 3; ++d)
-                        a[d] = add2(bc2(h.ti.gdrive[d]),
-                                    make_float2(own0 >= 0 ? cand[sl0].a[d] : 0.f, own1 >= 0 ? cand[sl1].a[d] : 0.f));
-                    float2 u[3], p;
-                    if constexpr (FOLD) collide2_t1_scaled<Q>(f, a, own0 >= 0, own1 >= 0, cks, sload, u, &p);
-                    else collide2<Q>(f, a, own0 >= 0, own1 >= 0, ck, u, &p);
-                    float2 uu = mul2(u[0], u[0]);
-#pragma unroll
-                    for (int d = 1; d < D; ++d) uu = fma2(u[d], u[d], uu);
-                    bad |= (v0 && !(uu.x < 0.25f)) || (v1 && !(uu.y < 0.25f));
-                    if (v0) {
-                        S* o = outrow + x;
-                        const int qs = (int)h.ti.qstride;  // < 2^31 elements per population
-                        const float sstore = h.ti.sstore;
-                        if (v1) {
-#pragma unroll
-                            for (int q = 0; q < QS; ++q) {
-                                if constexpr (FOLD) *reinterpret_cast<__half2*>(o) = __floats2half2_rn(f[q].x, f[q].y);
-                                else store_pair(o, f[q], sstore);
-                                o += qs;
-                            }
-                        } else {
-#pragma unroll
-                            for (int q = 0; q < QS; ++q) {
-                                if constexpr (FOLD) *o = __float2half_rn(f[q].x);
-                                else *o = to_store<S>(f[q].x, sstore);
-                                o += qs;
-                            }
-                        }
-                    }
-                    // the solid nodes' velocities into their particles' boxes (Eq. 22)
-                    if (v0 && own0 >= 0)
-                        box_store<D>(ubox, geo, cand[sl0], x, y, z, u[0].x, u[1].x, D == 3 ? u[2].x : 0.f);
-                    if (v1 && own1 >= 0)
-                        box_store<D>(ubox, geo, cand[sl1], x + 1, y, z, u[0].y, u[1].y, D == 3 ? u[2].y : 0.f);
+                    bad |= finish_pair<Q, S, FOLD>(env, f, FOLD ? cks : ck, sload, sstore, free, cand, ncand,
+                                                   x0 + j * 64, x, y, z, lane, outrow + x, (int)h.ti.qstride);
                 }
             }
         };
@@ -695,17 +665,13 @@ static int tma_blocks_t(const Shape& sh, int stages, int ninst) {
     return nb;
 }
 
-#define LBM_TMA_DISPATCH(CALL)                                                          \
-    {                                                                                   \
-        const int rows = sh.ty * sh.tz;                                                 \
-        if (Q == 9 && !fp16 && rows == 4) return CALL(9, float, 128, 4);                \
-        if (Q == 9 && !fp16 && rows == 8) return CALL(9, float, 128, 8);                \
-        if (Q == 9 && fp16 && rows == 4) return CALL(9, __half, 128, 4);                \
-        if (Q == 9 && fp16 && rows == 8) return CALL(9, __half, 128, 8);                \
-        if (Q == 19 && !fp16 && rows == 4) return CALL(19, float, 64, 4);               \
-        if (Q == 19 && !fp16 && rows == 8) return CALL(19, float, 64, 8);               \
-        if (Q == 19 && fp16 && rows == 4) return CALL(19, __half, 64, 4);               \
-        if (Q == 19 && fp16 && rows == 8) return CALL(19, __half, 64, 8);               \
+#define LBM_TMA_DISPATCH(CALL)                                       \
+    {                                                                \
+        const int rows = sh.ty;                                      \
+        if (Q == 9 && !fp16 && rows == 4) return CALL(9, float, 128, 4);  \
+        if (Q == 9 && !fp16 && rows == 8) return CALL(9, float, 128, 8);  \
+        if (Q == 9 && fp16 && rows == 4) return CALL(9, __half, 128, 4);  \
+        if (Q == 9 && fp16 && rows == 8) return CALL(9, __half, 128, 8);  \
     }
 
 int fluid_tma_blocks_per_sm(int Q, int fp16, const Shape& sh, int stages, int ninst) {
