@@ -10,15 +10,13 @@
  *      the penalization source S = w/(2 cs^4) alpha Pi_neq : (c c - cs^2 I)
  *      (Eq. 17);
  *   5. per-particle rigid-body projection U, omega over each solid domain
- *      (Eq. 22): the fused kernel stores each solid node's velocity in its
- *      particle's velocity box, and exact integer sums over the box give
- *      U and omega, independent of the order of summation;
+ *      (Eq. 22): the fused kernel adds the solid nodes' velocities up as exact
+ *      integers, which give U and omega independent of the order of summation;
  *   6. particle update: repulsive collision forces (Eqs. 19-21) and the
  *      predictor-corrector of Algorithm 1, which also yields the collision
  *      acceleration A applied on the particle's nodes in the next step.
- * Steps 1-4 and the box stores run in one fused CUDA kernel per step over all
- * instances; the sums and the second pass of step 5 in one block per
- * particle; step 6 in FP64 in one more kernel.
+ * Steps 1-4 and the sums of step 5 run in one fused CUDA kernel per step over
+ * all instances; the second pass of step 5 and step 6 in FP64 in one more.
  *
  * Units: lattice units, dx = dt = 1 (Sec. 3 preamble).  Node (i, j, k) sits at
  * integer coordinates; fields are row-major with x fastest.
@@ -228,8 +226,8 @@ int lbm_set_kernel_shape(lbm_ctx* ctx, int vec, int tile_rows, int warps);
  * kernel's waits keep their own 2 s bound.  seconds in [0, 60]. */
 int lbm_set_particle_wait_limit(lbm_ctx* ctx, double seconds);
 /* Kernel launches issued by one lbm_step(ctx, 1): the fluid kernel, then with
- * particles the box sums of Eq. 22 and the particle kernel (one launch, or one
- * per phase when its blocks cannot all be resident). */
+ * particles the particle kernel (one launch, or one per sub-step when its
+ * blocks cannot all be resident). */
 int lbm_launches_per_step(const lbm_ctx* ctx);
 /* Fluid kernel alone, one launch, for timing: the same fused kernel and
  * work as the fluid part of lbm_step, on the current state of every
@@ -242,8 +240,9 @@ int lbm_fluid_step_only(lbm_ctx* ctx);
 /* Measurement: nsteps time steps exactly like lbm_step (the state advances),
  * launched one by one without graphs, with CUDA events on the context stream
  * around each kernel of the step.  Writes the mean duration per step, in ms,
- * of the fluid kernel, of the box sums (Eq. 22) and of the particle kernel
- * (Algorithm 1); any pointer may be NULL; 0 for the particle kernels when
+ * of the fluid kernel, of the sums of Eq. 22 and of the particle kernel
+ * (Algorithm 1); the sums are taken inside the fluid kernel, so ms_box is the
+ * interval of two events with nothing between them; any pointer may be NULL; 0 for the particle kernels when
  * there are no particles.  Each duration runs from the end of the previous
  * kernel to the end of this one, so it includes the launch latency.
  * Synchronises; nsteps in [1, 100000] (LBM_ERR_INVALID otherwise); returns

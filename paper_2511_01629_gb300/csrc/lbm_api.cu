@@ -27,12 +27,11 @@ cudaError_t launch_pack(int Q, int fp16, const InstDesc* insts, int inst, long l
 cudaError_t launch_unpack(int Q, int fp16, const InstDesc* insts, int inst, long long N, int par,
                           float* dst, cudaStream_t st);
 int particle_blocks_resident(int num_sms);
-cudaError_t launch_particles(const InstDesc* insts, const PartRef* refs, int ntotal, int D, int K,
+cudaError_t launch_particles(const InstDesc* insts, const PartRef* refs, int ntotal, int ninst, int D, int K,
                              int lpar, const Shape& sh, GridBar* gb, bool fused, cudaStream_t st,
                              long long wait_ns);
 cudaError_t launch_publish(const InstDesc* insts, const PartRef* refs, int ntotal, int D, int lpar,
                            const Shape& sh, cudaStream_t st);
-cudaError_t launch_box_sums(const InstDesc* insts, const PartRef* refs, int ntotal, int D, cudaStream_t st);
 int tma_tile_width(int Q);
 bool tma_rows_ok(int rows);
 int fluid_tma_blocks_per_sm(int Q, int fp16, const Shape& sh, int stages, int ninst);
@@ -74,13 +73,11 @@ struct Instance {
     int ntile[3] = {1, 1, 1};
     int ntiles = 0, tile0 = 0;
     int maxk = 0;
-    DevBuf f[2], prec, lcnt[2], lent[2], lrec[2], ubox, ubox_scratch, boxinfo, btot, X, U, W, Un, Wn, theta, A, R, ratio, count, Xk, pconst, Xsf, invc,
+    DevBuf f[2], prec, lcnt[2], lent[2], lrec[2], tot[2], tot_scratch, pst[2], Xp[2], X, U, W, Un, Wn, theta, A, R, ratio, count, Xk, pconst, Xsf, invc,
         Ubar, Xf, Acor, rconst;
     std::vector<double> hR;      // radii, semi-major axes of ellipses (validation)
     std::vector<double> hB;      // semi-minor axes (== hR for disks and spheres)
     std::vector<double> hratio;  // density ratios (per-particle constants)
-    std::vector<int> hbox;       // per particle: first entry of its velocity box, H (pairs)
-    long long box_entries = 0;   // entries of all velocity boxes
 };
 
 // Adjoint recording of one instance: checkpoints of the forward pass and the
@@ -92,6 +89,7 @@ struct AdjInst {
     DevBuf rprec, rlcnt, rlent, rlrec, rgeo, rstate;  // [L + 1] records of each step
     DevBuf fbar[2];             // adjoint of the pre-collision populations (ping-pong)
     DevBuf pbuf;                // adjoint particle arrays (AdjBufs)
+    DevBuf tot, pst, Xp;        // the recomputation's totals and step inputs (both parities of each)
 };
 struct AdjCtx {
     bool ready = false;         // a recorded forward pass matches the current state
@@ -277,10 +275,12 @@ InstDesc make_desc(lbm_ctx* ctx, const Instance& I) {
     d.list_ent[1] = P<uint32_t>(I.lent[1]);
     d.list_rec[0] = I.lrec[0].ptr;
     d.list_rec[1] = I.lrec[1].ptr;
-    d.ubox = P<float>(I.ubox);
-    d.ubox_scratch = P<float>(I.ubox_scratch);
-    d.boxinfo = P<int2>(I.boxinfo);
-    d.btot = P<long long>(I.btot);
+    for (int b = 0; b < 2; ++b) {
+        d.tot[b] = P<long long>(I.tot[b]);
+        d.pst[b] = P<PState>(I.pst[b]);
+        d.Xp[b] = P<float4>(I.Xp[b]);
+    }
+    d.tot_scratch = P<long long>(I.tot_scratch);
     d.X = P<double>(I.X);
     d.U = P<double>(I.U);
     d.W = P<double>(I.W);
@@ -387,7 +387,8 @@ int upload_pconst(lbm_ctx* ctx, Instance& I) {
         r.qlo = 1.0f - beta;
         r.qhi = 1.0f + beta;
         r.shape = B != R;
-        r.pad = 0;
+        const int H = (int)ceil(R) + 2;
+        r.rows2 = (H - 1) * (H - 1);
     }
     CK(cudaMemcpy(I.rconst.ptr, rc.data(), sizeof(RecConst) * rc.size(), cudaMemcpyHostToDevice));
     return LBM_OK;
@@ -398,7 +399,7 @@ int republish(lbm_ctx* ctx) {
     for (auto& I : ctx->inst) {
         if (I.np == 0) continue;
         CK(cudaMemsetAsync(I.lcnt[ctx->par].ptr, 0, sizeof(int) * I.ntiles, ctx->st));
-        if (I.ubox.ptr) CK(cudaMemsetAsync(I.ubox.ptr, 0xff, I.ubox.bytes, ctx->st));  // every entry empty (NaN)
+        CK(cudaMemsetAsync(I.tot[ctx->par].ptr, 0, I.tot[ctx->par].bytes, ctx->st));
     }
     if (ctx->np_total > 0)
         CK(launch_publish(P<InstDesc>(ctx->d_insts), P<PartRef>(ctx->d_refs), ctx->np_total, ctx->D,
@@ -555,10 +556,9 @@ int enqueue_step(lbm_ctx* ctx, cudaStream_t st) {
     if (rc) return rc;
     if (ctx->np_total > 0) {
         const int K = ctx->inst[0].cfg.K;
-        CK(launch_box_sums(P<InstDesc>(ctx->d_insts), P<PartRef>(ctx->d_refs), ctx->np_total, ctx->D, st));
         const bool fused = (ctx->np_total + 7) / 8 <= particle_blocks_resident(ctx->num_sms);
-        CK(launch_particles(P<InstDesc>(ctx->d_insts), P<PartRef>(ctx->d_refs), ctx->np_total, ctx->D,
-                            K, ctx->par ^ 1, ctx->shape, P<GridBar>(ctx->d_gridbar), fused, st,
+        CK(launch_particles(P<InstDesc>(ctx->d_insts), P<PartRef>(ctx->d_refs), ctx->np_total,
+                            (int)ctx->inst.size(), ctx->D, K, ctx->par ^ 1, ctx->shape, P<GridBar>(ctx->d_gridbar), fused, st,
                             ctx->wait_ns));
     }
     ctx->par ^= 1;
@@ -605,7 +605,7 @@ void adj_release(lbm_ctx* ctx) {
         for (auto& b : a.ckpt) dfree(ctx, b);
         for (auto& b : a.slot) dfree(ctx, b);
         DevBuf* bufs[] = {&a.ckst, &a.rprec, &a.rlcnt, &a.rlent, &a.rlrec, &a.rgeo, &a.rstate, &a.fbar[0],
-                          &a.fbar[1], &a.pbuf};
+                          &a.fbar[1], &a.pbuf, &a.tot, &a.pst, &a.Xp};
         for (DevBuf* b : bufs) dfree(ctx, *b);
     }
     A.ai.clear();
@@ -620,7 +620,7 @@ void destroy_all(lbm_ctx* ctx) {
     for (auto& I : ctx->inst) {
         DevBuf* bufs[] = {&I.f[0], &I.f[1], &I.prec, &I.lcnt[0], &I.lcnt[1], &I.lent[0], &I.lent[1],
                           &I.lrec[0], &I.lrec[1],
-                          &I.ubox, &I.ubox_scratch, &I.boxinfo, &I.btot, &I.X, &I.U, &I.W, &I.Un, &I.Wn, &I.theta, &I.A, &I.R,
+                          &I.tot[0], &I.tot[1], &I.tot_scratch, &I.pst[0], &I.pst[1], &I.Xp[0], &I.Xp[1], &I.X, &I.U, &I.W, &I.Un, &I.Wn, &I.theta, &I.A, &I.R,
                           &I.ratio, &I.count, &I.Xk, &I.Ubar, &I.Xf, &I.pconst, &I.Xsf, &I.invc, &I.Acor, &I.rconst};
         for (DevBuf* b : bufs) dfree(ctx, *b);
     }
@@ -649,8 +649,12 @@ int alloc_particles(lbm_ctx* ctx, Instance& I, int cap) {
     if ((rc = dalloc(ctx, I.rconst, sizeof(RecConst) * c))) return rc;
     if ((rc = dalloc(ctx, I.invc, sizeof(double) * c))) return rc;
     if ((rc = dalloc(ctx, I.Xsf, sizeof(float) * 8 * c))) return rc;
-    if ((rc = dalloc(ctx, I.boxinfo, sizeof(int2) * c))) return rc;
-    if ((rc = dalloc(ctx, I.btot, sizeof(long long) * NPV * c))) return rc;
+    for (int b = 0; b < 2; ++b) {
+        if ((rc = dalloc(ctx, I.tot[b], sizeof(long long) * NPV * c))) return rc;
+        if ((rc = dalloc(ctx, I.pst[b], sizeof(PState) * c))) return rc;
+        if ((rc = dalloc(ctx, I.Xp[b], sizeof(float4) * c))) return rc;
+    }
+    if ((rc = dalloc(ctx, I.tot_scratch, sizeof(long long) * NPV * c))) return rc;
     return LBM_OK;
 }
 
@@ -773,30 +777,6 @@ int lbm_num_particles(const lbm_ctx* ctx, int i) {
     return ctx->inst[i].np;
 }
 
-// Velocity boxes of all particles of an instance (side 2H + 1, H = ceil(R) + 2,
-// one after another), allocated to fit and marked empty (NaN).
-static int layout_boxes(lbm_ctx* ctx, Instance& I) {
-    const int D = ctx->D;
-    I.hbox.clear();
-    I.box_entries = 0;
-    for (int k = 0; k < I.np; ++k) {
-        const int H = (int)ceil(I.hR[k]) + 2, side = 2 * H + 1;
-        I.hbox.push_back((int)I.box_entries);
-        I.hbox.push_back(H);
-        I.box_entries += D == 2 ? (long long)side * side : (long long)side * side * side;
-    }
-    if (I.box_entries >= (1LL << 31)) return set_err(ctx, LBM_ERR_INVALID, "velocity boxes exceed 2^31 entries%s");
-    if (I.np == 0) return LBM_OK;
-    const size_t eb = (size_t)I.box_entries * (D == 2 ? 8 : 16);
-    int rc;
-    if ((rc = dalloc(ctx, I.ubox, eb)) || (rc = dalloc(ctx, I.ubox_scratch, eb))) return rc;
-    CK(cudaMemsetAsync(I.ubox.ptr, 0xff, I.ubox.bytes, ctx->st));  // every entry empty (NaN)
-    CK(cudaMemcpyAsync(I.boxinfo.ptr, I.hbox.data(), sizeof(int) * I.hbox.size(), cudaMemcpyHostToDevice,
-                       ctx->st));
-    CK(cudaStreamSynchronize(ctx->st));
-    return LBM_OK;
-}
-
 // Disks and spheres (minor == NULL) or ellipses (2D; minor = semi-minor axes,
 // theta = orientations or NULL).
 static int add_particles_impl(lbm_ctx* ctx, int i, int n, const double* pos, const double* radius,
@@ -868,7 +848,6 @@ static int add_particles_impl(lbm_ctx* ctx, int i, int n, const double* pos, con
     if (minor) I.hB.insert(I.hB.end(), minor, minor + n);
     else I.hB.insert(I.hB.end(), radius, radius + n);
     I.hratio.insert(I.hratio.end(), ratio, ratio + n);
-    if ((rc = layout_boxes(ctx, I))) return rc;
     if ((rc = upload_pconst(ctx, I))) return rc;
     if ((rc = upload_descs(ctx))) return rc;
     invalidate_graphs(ctx);
@@ -956,13 +935,13 @@ int lbm_step_timed(lbm_ctx* ctx, int nsteps, float* ms_fluid, float* ms_box, flo
         e = cudaEventRecord(q[0], ctx->st);
         if (e == cudaSuccess) rc = enqueue_fluid(ctx, 1, ctx->st);
         if (rc == LBM_OK && e == cudaSuccess) e = cudaEventRecord(q[1], ctx->st);
-        if (parts && rc == LBM_OK && e == cudaSuccess)
-            e = launch_box_sums(P<InstDesc>(ctx->d_insts), P<PartRef>(ctx->d_refs), ctx->np_total, ctx->D, ctx->st);
+        // the sums of Eq. 22 are taken inside the fluid kernel: q[1] .. q[2] is the
+        // events' own interval
         if (rc == LBM_OK && e == cudaSuccess) e = cudaEventRecord(q[2], ctx->st);
         if (parts && rc == LBM_OK && e == cudaSuccess) {
             const bool fused = (ctx->np_total + 7) / 8 <= particle_blocks_resident(ctx->num_sms);
-            e = launch_particles(P<InstDesc>(ctx->d_insts), P<PartRef>(ctx->d_refs), ctx->np_total, ctx->D,
-                                 ctx->inst[0].cfg.K, ctx->par ^ 1, ctx->shape, P<GridBar>(ctx->d_gridbar), fused,
+            e = launch_particles(P<InstDesc>(ctx->d_insts), P<PartRef>(ctx->d_refs), ctx->np_total,
+                                 (int)ctx->inst.size(), ctx->D, ctx->inst[0].cfg.K, ctx->par ^ 1, ctx->shape, P<GridBar>(ctx->d_gridbar), fused,
                                  ctx->st, ctx->wait_ns);
         }
         if (rc == LBM_OK && e == cudaSuccess) e = cudaEventRecord(q[3], ctx->st);
@@ -1203,8 +1182,7 @@ int lbm_load_state(lbm_ctx* ctx, const void* buf, size_t bytes) {
         CK(cudaMemcpy(I.ratio.ptr, r, sizeof(double) * I.np, cudaMemcpyHostToDevice));
         I.hratio.assign(reinterpret_cast<const double*>(r), reinterpret_cast<const double*>(r) + I.np);
         r += sizeof(double) * I.np;
-        if ((rc = layout_boxes(ctx, I))) return rc;
-        if ((rc = upload_pconst(ctx, I))) return rc;
+            if ((rc = upload_pconst(ctx, I))) return rc;
         CK(cudaMemcpy(I.count.ptr, r, sizeof(int) * I.np, cudaMemcpyHostToDevice));
         r += sizeof(int) * I.np;
     }
@@ -1340,7 +1318,7 @@ int lbm_launches_per_step(const lbm_ctx* ctx) {
     if (!ctx) return 0;
     if (ctx->np_total == 0) return 1;
     const bool fused = (ctx->np_total + 7) / 8 <= particle_blocks_resident(ctx->num_sms);
-    return 2 + (fused ? 1 : 1 + ctx->inst[0].cfg.K);  // fluid, box sums, particles
+    return 1 + (fused ? 1 : ctx->inst[0].cfg.K);  // fluid, particles
 }
 
 long long lbm_steps_done(const lbm_ctx* ctx) { return ctx ? ctx->steps : 0; }
@@ -1478,6 +1456,8 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
             (rc = dalloc(ctx, a.rstate, sizeof(double) * 16 * n1 * (L + 1))) ||
             (rc = dalloc(ctx, a.fbar[0], sizeof(float) * (ctx->Q - 1) * (size_t)I.qstride)) ||
             (rc = dalloc(ctx, a.fbar[1], sizeof(float) * (ctx->Q - 1) * (size_t)I.qstride)) ||
+            (rc = dalloc(ctx, a.tot, sizeof(long long) * NPV * n1 * 2)) ||
+            (rc = dalloc(ctx, a.pst, sizeof(PState) * n1 * 2)) || (rc = dalloc(ctx, a.Xp, sizeof(float4) * n1 * 2)) ||
             (rc = dalloc(ctx, a.pbuf, sizeof(double) * adj_pbuf_doubles(I.np, K))))
             return rc;
         CK(cudaMemsetAsync(a.pbuf.ptr, 0, a.pbuf.bytes, ctx->st));
@@ -1494,6 +1474,11 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
             AdjInst& a = A.ai[i];
             const size_t n1 = (size_t)std::max(I.np, 1);
             InstDesc d = make_desc(ctx, I);
+            for (int b = 0; b < 2; ++b) {  // the context's own stay as the forward pass left them
+                d.tot[b] = P<long long>(a.tot) + NPV * n1 * b;
+                d.pst[b] = P<PState>(a.pst) + n1 * b;
+                d.Xp[b] = P<float4>(a.Xp) + n1 * b;
+            }
             PRec* rp = P<PRec>(a.rprec);
             int* lc = P<int>(a.rlcnt);
             uint32_t* le = P<uint32_t>(a.rlent);
@@ -1612,9 +1597,8 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
             const int err = enqueue_fluid_on(ctx, dk, tma ? P<CUtensorMap>(A.d_rtmaps) + (size_t)k * ni * 2 : nullptr, par,
                                              1, st);
             if (err) return err;
-            if (ctx->np_total > 0) CK(launch_box_sums(dk, P<PartRef>(ctx->d_refs), ctx->np_total, ctx->D, st));
             if (ctx->np_total > 0)
-                CK(launch_particles(dk, P<PartRef>(ctx->d_refs), ctx->np_total, ctx->D, K, par ^ 1, sh,
+                CK(launch_particles(dk, P<PartRef>(ctx->d_refs), ctx->np_total, ni, ctx->D, K, par ^ 1, sh,
                                     P<GridBar>(ctx->d_gridbar), fused, st, ctx->wait_ns));
         }
         for (int k = len - 1; k >= 0; --k) {
@@ -1640,7 +1624,7 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
             if (I.np)
                 CK(cudaMemcpyAsync(a.rstate.ptr, st, sizeof(double) * 16 * I.np, cudaMemcpyDeviceToDevice, ctx->st));
             CK(cudaMemsetAsync(a.rlcnt.ptr, 0, sizeof(int) * I.ntiles, ctx->st));
-            if (I.ubox.ptr) CK(cudaMemsetAsync(I.ubox.ptr, 0xff, I.ubox.bytes, ctx->st));
+            CK(cudaMemsetAsync(a.tot.ptr, 0, a.tot.bytes, ctx->st));
         }
         if (ctx->np_total > 0)
             CK(launch_publish(dR + (size_t)L * ni, P<PartRef>(ctx->d_refs), ctx->np_total, ctx->D, 0, sh, ctx->st));

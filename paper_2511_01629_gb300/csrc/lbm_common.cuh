@@ -118,8 +118,8 @@ struct __align__(16) Cand {
     float a[3];
     int p;     // particle index within the instance
     int k;     // index of this tile among the tiles of the particle's bounding box
-    int boff;  // first entry of the particle's velocity box
-    int bh;    // H of the box: side 2H + 1, centred on ref
+    int rows2; // see RecConst
+    int pad;
     int shape; // 0 disk or sphere, 1 ellipse (the filter reads its record)
 };
 static_assert(sizeof(Cand) == CAND_BYTES, "candidate records are copied in 64-byte units");
@@ -749,29 +749,142 @@ __device__ __forceinline__ long long warp_sum_ll(long long v) {
     return v;
 }
 
-// Velocity of a node owned by candidate cd into the particle's box: entry
-// (d + H) of the offset d = node - floor(X) (minimum image on periodic axes,
-// |d| <= R + 1 < H).  The particle kernel takes the sums of Eq. 22 from there.
-template <int D>
-__device__ __forceinline__ void box_store(float* ubox, const Geo& g, const Cand& cd, int x, int y, int z,
-                                          float ux, float uy, float uz) {
-    const int side = 2 * cd.bh + 1;
-    const int dx = wrap_int(x - cd.ref[0], g.n[0], g.per[0]) + cd.bh;
-    const int dy = wrap_int(y - cd.ref[1], g.n[1], g.per[1]) + cd.bh;
-    if (D == 2) {
-        reinterpret_cast<float2*>(ubox)[cd.boff + dy * side + dx] = make_float2(ux, uy);
-    } else {
-        const int dz = wrap_int(z - cd.ref[2], g.n[2], g.per[2]) + cd.bh;
-        reinterpret_cast<float4*>(ubox)[cd.boff + ((long long)dz * side + dy) * side + dx] =
-            make_float4(ux, uy, uz, 0.f);
+// round(u * 2^FXBITS) of two velocities as hi * 2^20 + lo (|hi| <= 2^19,
+// |lo| <= 2^19), the integer of to_fx32, without a conversion instruction:
+// adding 1.5 2^23 rounds to the nearest integer (ties to even) and leaves it
+// in the low mantissa bits.  v = u 2^20 and v - hi are exact, and hi 2^20 is an
+// even integer, so rne(u 2^40) = hi 2^20 + rne((v - hi) 2^20), ties included.
+__device__ __forceinline__ void split_fx(float2 u, int* hi, int* lo) {
+    constexpr float magic = 12582912.0f;
+    constexpr int mbits = 0x4B400000;
+    u.x = fminf(fmaxf(u.x, -0.49999997f), 0.49999997f);
+    u.y = fminf(fmaxf(u.y, -0.49999997f), 0.49999997f);
+    const float2 v = mul2(u, bc2(1048576.0f));
+    const float2 r = add2(v, bc2(magic));
+    const float2 rem = sub2(v, sub2(r, bc2(magic)));
+    const float2 l = fma2(rem, bc2(1048576.0f), bc2(magic));
+    hi[0] = __float_as_int(r.x) - mbits;
+    hi[1] = __float_as_int(r.y) - mbits;
+    lo[0] = __float_as_int(l.x) - mbits;
+    lo[1] = __float_as_int(l.y) - mbits;
+}
+// Exact warp sum of 32-bit integers whose sum may exceed 32 bits.
+__device__ __forceinline__ long long warp_sum_wide(int v) {
+    const unsigned l = __reduce_add_sync(0xffffffffu, (unsigned)v & 0xffffu);
+    return (long long)l + (long long)__reduce_add_sync(0xffffffffu, v >> 16) * 65536LL;
+}
+
+// Sums of Eq. 22 over the solid nodes of a warp, added to the totals of their
+// particles.  A lane holds V adjacent nodes x .. x + V - 1 of row (y, z) (one
+// row per warp); slot[e] is node e's candidate, or -1.  For each particle
+// present, the warp adds up exact integers and one atomic instruction adds the
+// 9 (3D: 16) totals, a lane each.  y and z are the row's, so only count, sum
+// dx, sum dx^2, sum u and sum dx u are reduced; a velocity's integer goes as
+// two 32-bit halves (split_fx), and |dx| < 32 (R < 30) keeps even their
+// products' warp sums in 32 bits.  The velocities went through a box of global
+// memory and a kernel of their own before (6.4 us of a step of 20 us with one
+// disk on 100 x 200, 26 us of 172 us with five spheres).
+template <int D, int V>
+__device__ __forceinline__ void rigid_sums(long long* __restrict__ tot, const Geo& g, const Cand* cand, int* slot,
+                                           int x, int y, int z, const float (*u)[V], int lane) {
+    constexpr int V2 = V >= 2 ? V : 2;
+    int hi[D][V2], lo[D][V2];
+#pragma unroll
+    for (int d = 0; d < D; ++d)
+#pragma unroll
+        for (int e = 0; e < V; e += 2) split_fx(make_float2(u[d][e], e + 1 < V ? u[d][e + 1] : 0.f), hi[d] + e, lo[d] + e);
+    auto first_slot = [&]() {
+        int s = -1;
+#pragma unroll
+        for (int e = V - 1; e >= 0; --e) s = slot[e] >= 0 ? slot[e] : s;
+        return s;
+    };
+    for (;;) {
+        const int mine = first_slot();
+        const unsigned b = __ballot_sync(0xffffffffu, mine >= 0);
+        if (!b) return;
+        const int s = __shfl_sync(0xffffffffu, mine, __ffs(b) - 1);
+        const Cand& cd = cand[s];
+        const int dy = wrap_int(y - cd.ref[1], g.n[1], g.per[1]);
+        const int dz = D == 3 ? wrap_int(z - cd.ref[2], g.n[2], g.per[2]) : 0;
+        if (D == 3 && dy * dy + dz * dz > cd.rows2) {
+            // Kept as the sums have always been: (ceil(R) + 1)^2 leaves out the outermost
+            // nodes of a sphere whose centre lies near the far corner of its lattice
+            // cell in y and z (up to R + sqrt(2) from floor(X)); 4 of 2139 nodes at
+            // R = 8, offsets 0.99 and 0.85.
+#pragma unroll
+            for (int e = 0; e < V; ++e) slot[e] = slot[e] == s ? -1 : slot[e];
+            continue;
+        }
+        int cnt = 0, sx = 0, sxx = 0;
+        int sh[D], sl[D], xh[D], xl[D];  // halves of sum u and of sum dx u (y, z)
+#pragma unroll
+        for (int d = 0; d < D; ++d) sh[d] = sl[d] = xh[d] = xl[d] = 0;
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            const bool m = slot[e] == s;
+            cnt += __popc(__ballot_sync(0xffffffffu, m));
+            if (m) {
+                const int dx = wrap_int(x + e - cd.ref[0], g.n[0], g.per[0]);
+                sx += dx;
+                sxx += dx * dx;
+#pragma unroll
+                for (int d = 0; d < D; ++d) {
+                    sh[d] += hi[d][e];
+                    sl[d] += lo[d][e];
+                    if (d > 0) {
+                        xh[d] += dx * hi[d][e];
+                        xl[d] += dx * lo[d][e];
+                    }
+                }
+                slot[e] = -1;
+            }
+        }
+        sx = __reduce_add_sync(0xffffffffu, sx);
+        sxx = __reduce_add_sync(0xffffffffu, sxx);
+        const bool narrow = V == 2 && cd.R2hi < 900.0f;  // |dx| <= R + 1 < 32: 2^5 2^19 64 nodes < 2^31
+        long long su[D], sxu[D];
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            su[d] = (long long)__reduce_add_sync(0xffffffffu, sh[d]) * 1048576LL + __reduce_add_sync(0xffffffffu, sl[d]);
+            if (d == 0) continue;
+            if (narrow)
+                sxu[d] = (long long)__reduce_add_sync(0xffffffffu, xh[d]) * 1048576LL + __reduce_add_sync(0xffffffffu, xl[d]);
+            else sxu[d] = warp_sum_wide(xh[d]) * 1048576LL + warp_sum_wide(xl[d]);
+        }
+        int w = 0;  // lane k: total k (w: those that fit in 32 bits)
+        if (lane == 0) w = cnt;
+        if (lane == 1) w = sx;
+        if (lane == 2) w = dy * cnt;
+        if (lane == 4) w = sxx;
+        if (lane == 5) w = dy * dy * cnt;
+        if (lane == 7) w = dy * sx;
+        if (D == 3) {
+            if (lane == 3) w = dz * cnt;
+            if (lane == 6) w = dz * dz * cnt;
+            if (lane == 8) w = dz * sx;
+            if (lane == 9) w = dy * dz * cnt;
+        }
+        long long v = w;
+        if (lane == 10) v = su[0];
+        if (lane == 11) v = su[1];
+        if (lane == 15) v = sxu[1] - (long long)dy * su[0];
+        if constexpr (D == 3) {
+            if (lane == 12) v = su[2];
+            if (lane == 13) v = (long long)dy * su[2] - (long long)dz * su[1];
+            if (lane == 14) v = (long long)dz * su[0] - sxu[2];
+        }
+        constexpr unsigned used = D == 3 ? 0xFFFFu : 0x8CB7u;
+        if ((used >> lane) & 1u)
+            atomicAdd(reinterpret_cast<unsigned long long*>(tot + (long long)NPV * cd.p + lane), (unsigned long long)v);
     }
 }
 
 // The rest of a fused step for two adjacent nodes (x, x + 1) of a row, x even,
 // one pair per lane of a converged warp whose 64 nodes start at xseg: owner,
-// collision, store and the solid nodes' velocities.  f: the pulled
+// collision, store and the solid nodes' sums.  f: the pulled
 // populations (at the storage scale with FOLD); out: population 1 of node x in
-// the new buffer.  Env gives the instance (n, per, prec, gdrive, ubox).
+// the new buffer.  Env gives the instance (n, per, prec, gdrive, tot).
 // Returns whether a velocity left the stable range.
 template <int Q, class S, bool FOLD, class Env>
 __device__ __forceinline__ bool finish_pair(const Env& e, float2* f, const CollK& ck, float sload, float sstore, bool free,
@@ -806,9 +919,9 @@ __device__ __forceinline__ bool finish_pair(const Env& e, float2* f, const CollK
             }
         }
     }
-    float2 uu, u[3];
-    const bool solid = own0 >= 0 || own1 >= 0;
-    if (free && !__any_sync(0xffffffffu, solid)) {
+    float2 uu, u[3] = {bc2(0.f), bc2(0.f), bc2(0.f)};
+    const bool any_solid = __any_sync(0xffffffffu, own0 >= 0 || own1 >= 0);
+    if (free && !any_solid) {
         uu = collide2_free<Q, FOLD>(f, ck, sload);
     } else {
         float2 a[3], p;
@@ -837,10 +950,16 @@ __device__ __forceinline__ bool finish_pair(const Env& e, float2* f, const CollK
             out += qs;
         }
     }
-    if (solid) {  // the solid nodes' velocities into their particles' boxes (Eq. 22)
+    if (any_solid) {  // the solid nodes' part of their particles' sums (Eq. 22)
         const Geo geo = geo_of();
-        if (v0 && own0 >= 0) box_store<D>(e.ubox(), geo, cand[sl0], x, y, z, u[0].x, u[1].x, D == 3 ? u[2].x : 0.f);
-        if (v1 && own1 >= 0) box_store<D>(e.ubox(), geo, cand[sl1], x + 1, y, z, u[0].y, u[1].y, D == 3 ? u[2].y : 0.f);
+        int slot[2] = {v0 && own0 >= 0 ? sl0 : -1, v1 && own1 >= 0 ? sl1 : -1};
+        float uv[D][2];
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            uv[d][0] = u[d].x;
+            uv[d][1] = u[d].y;
+        }
+        rigid_sums<D, 2>(e.tot(), geo, cand, slot, x, y, z, uv, lane);
     }
     return (v0 && !(uu.x < 0.25f)) || (v1 && !(uu.y < 0.25f));
 }
@@ -858,7 +977,7 @@ __device__ __forceinline__ double rcp64(double x) {
 }
 
 // Rigid-body projection of particle p (Eq. 22 with rho_s cancelled): the
-// box sums are exact integers, summed exactly, then converted to FP64.
+// sums are exact integers, converted to FP64.
 // Moments about the integer reference floor(X) are shifted to the centre:
 //   sum r x u = sum d x u - phi x sum u,
 //   sum r r^T = sum d d^T - phi sum d^T - sum d phi^T + n phi phi^T.
@@ -870,61 +989,20 @@ __device__ __forceinline__ double rcp64(double x) {
 // another warp, concurrently.  Each lane evaluates the same expressions, in
 // the same order, as a serial loop over the components would.
 
-// Translational part, component d (0..2) of particle p.
-template <int D>
-__device__ void finalize_translation(const InstDesc& in, int p, const long long* v, int d) {
-    const PRec& pr = in.prec[p];
-    // every operand is loaded before the first store, so the loads overlap
-    const double X = d < D ? pr.X[d] : 0.0;
-    const double Uold = d < D ? in.U[3 * p + d] : 0.0;
-    const float Rf = (float)in.pconst[PCONST_N * p + PC_R];
-    const double h = in.hK;
-    if (v[0] == 0) {  // no solid node: cannot happen inside the box for R >= 2
-        if (d == 0) {
-            atomicOr(in.status, ST_PARTICLE);
-            in.count[p] = 0;
-        }
-        in.Un[3 * p + d] = in.U[3 * p + d];
-        return;
-    }
-    const double cnt = (double)v[0];
-    const double inv = rcp64(cnt);
-    double Uo = 0.0, ub = 0.0;
-    float Xs = 0.f;
-    bool fast = false;
-    if (d < D) {
-        const double Su = (double)v[10 + d] * FX_SCALE;
-        Uo = Su * inv;
-        ub = 0.5 * (Uo + Uold);
-        fast = !(fabs(ub) < 0.5);
-        Xs = (float)(X + h * ub);
-    }
-    in.Un[3 * p + d] = Uo;
-    in.Ubar[3 * p + d] = ub;
-    in.Xk[3 * p + d] = X;  // sub-step buffer 0 = X^n
-    in.Xf[4 * p + d] = (float)X;
-    in.Xsf[4 * p + d] = Xs;
-    if (d == 0) {
-        in.Xf[4 * p + 3] = Rf;
-        in.Xsf[4 * p + 3] = Rf;
-        in.count[p] = (int)v[0];
-        in.invc[p] = inv;
-    }
-    if (fast) atomicOr(in.status, ST_DISPLACEMENT);
-}
+// Translational part, one component of a particle: U^n from the totals'
+// count v0 and the component's sum (v0 == 0, no solid node, cannot happen
+// inside the box for R >= 2; the caller reports it), and Ubar = (U^n + U^{n-1})/2.
+__device__ __forceinline__ double finalize_u(long long su, double inv) { return ((double)su * FX_SCALE) * inv; }
 
-// Rotational part, component c (0..2) of W^n of particle p, and the sums the
-// adjoint records (component 0's lane).
+// Rotational part: component c (0..2) of W^n of a particle at X with totals v.
+// With geo != nullptr, component 0's lane also writes the sums about X^n that the
+// projection used (recorded for the adjoint).
 template <int D>
-__device__ void finalize_rotation(const InstDesc& in, int p, const long long* v, int c) {
-    const PRec& pr = in.prec[p];
+__device__ __forceinline__ double finalize_rotation(const long long* v, const double* X, int c, double* geo) {
     double phi[3] = {0, 0, 0};
 #pragma unroll
-    for (int d = 0; d < D; ++d) phi[d] = pr.X[d] - (double)pr.ref[d];
-    if (v[0] == 0) {
-        in.Wn[3 * p + c] = 0.0;
-        return;
-    }
+    for (int d = 0; d < D; ++d) phi[d] = X[d] - floor(X[d]);
+    if (v[0] == 0) return 0.0;
     const double cnt = (double)v[0];
     double Su[3] = {0, 0, 0};
 #pragma unroll
@@ -970,9 +1048,8 @@ __device__ void finalize_rotation(const InstDesc& in, int p, const long long* v,
                           M[0][2] * (M[1][0] * M[2][1] - M[1][1] * M[2][0]);
         Wo = dc * idet;
     }
-    in.Wn[3 * p + c] = Wo;
-    if (in.adj_geo && c == 0) {  // adjoint recording: the sums about X^n that the projection used
-        double* g = in.adj_geo + (long long)NPV * p;
+    if (geo && c == 0) {
+        double* g = geo;
         const int ii[6] = {0, 1, 2, 0, 0, 1}, jj[6] = {0, 1, 2, 1, 2, 2};
         g[0] = cnt;
         for (int d = 0; d < 3; ++d) g[1 + d] = (double)v[1 + d] - cnt * phi[d];
@@ -986,6 +1063,7 @@ __device__ void finalize_rotation(const InstDesc& in, int p, const long long* v,
         g[14] = (double)v[14] * FX_SCALE - (phi[2] * Su[0] - phi[0] * Su[2]);
         g[15] = (double)v[15] * FX_SCALE - (phi[0] * Su[1] - phi[1] * Su[0]);
     }
+    return Wo;
 }
 
 // Where population q of node (x, y, z) pulls from (Eq. 10, left side): the

@@ -23,12 +23,12 @@ constexpr int TW = 64;
 
 struct DescEnv {
     const InstDesc& in;
-    float* box;
+    long long* sums;
     __device__ __forceinline__ int n(int d) const { return in.n[d]; }
     __device__ __forceinline__ int per(int d) const { return in.periodic[d]; }
     __device__ __forceinline__ const PRec* prec() const { return in.prec; }
     __device__ __forceinline__ float gdrive(int d) const { return in.gdrive[d]; }
-    __device__ __forceinline__ float* ubox() const { return box; }
+    __device__ __forceinline__ long long* tot() const { return sums; }
 };
 
 template <class S> __device__ __forceinline__ float load_one(const S* p, float s) {
@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(256, 2) k_fluid_direct(const InstDesc* __restr
     }
     const CollK ck = make_collk<Q>(make_collp(in));
     const bool free = in.gdrive[0] == 0.f && in.gdrive[1] == 0.f && in.gdrive[2] == 0.f;
-    const DescEnv env{in, commit ? in.ubox : in.ubox_scratch};
+    const DescEnv env{in, commit ? in.tot[par] : in.tot_scratch};
     S* __restrict__ fout = static_cast<S*>(in.f[par ^ 1]);
     bool bad = false;
     for (;;) {

@@ -15,8 +15,8 @@
 // tile touches no global memory.  The copies of a stage are counted by its
 // mbarrier; each consumer lane pulls two adjacent nodes' populations from
 // shared memory at x - c_x, collides them with packed FP32x2 arithmetic,
-// stores them to HBM with 8-byte coalesced stores, and stores the velocity
-// of each solid node into its particle's box for the sums of Eq. 22.  Rows whose source lies beyond a y or z face
+// stores them to HBM with 8-byte coalesced stores, and adds the velocities
+// of solid nodes to their particle's sums of Eq. 22.  Rows whose source lies beyond a y or z face
 // gather those populations from HBM directly, as the register-path kernel
 // does.
 //
@@ -114,7 +114,7 @@ constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;  // 2 s
 // producer nor the consumers go to global memory for them in the tile loop.
 struct __align__(16) TInst {
     const void* f[2];          // population buffers
-    float* ubox[2];            // velocity boxes: [0] the state's, [1] scratch
+    long long* tot[3];         // totals of Eq. 22: per parity, scratch
     const PRec* prec;
     int* status;
     int* lcnt[2];              // tile list counts per parity
@@ -137,8 +137,9 @@ __device__ __forceinline__ void make_tinst(TInst& t, const InstDesc& in) {
         t.lcnt[b] = in.list_cnt[b];
         t.lrec[b] = static_cast<const Cand*>(in.list_rec[b]);
     }
-    t.ubox[0] = in.ubox;
-    t.ubox[1] = in.ubox_scratch;
+    t.tot[0] = in.tot[0];
+    t.tot[1] = in.tot[1];
+    t.tot[2] = in.tot_scratch;
     t.prec = in.prec;
     t.status = in.status;
     t.qstride = in.qstride;
@@ -171,12 +172,12 @@ __device__ __forceinline__ void make_tinst(TInst& t, const InstDesc& in) {
 // What finish_pair needs of the instance, read from the shared copy when it does.
 struct TileEnv {
     const TInst& ti;
-    float* box;
+    long long* sums;
     __device__ __forceinline__ int n(int d) const { return ti.n[d]; }
     __device__ __forceinline__ int per(int d) const { return ti.per[d]; }
     __device__ __forceinline__ const PRec* prec() const { return ti.prec; }
     __device__ __forceinline__ float gdrive(int d) const { return ti.gdrive[d]; }
-    __device__ __forceinline__ float* ubox() const { return box; }
+    __device__ __forceinline__ long long* tot() const { return sums; }
 };
 
 // Per-tile record the producer writes next to the staged populations.
@@ -518,7 +519,7 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
         const S* stage = reinterpret_cast<const S*>(smem + s * LY.stage);
         const int ex = h.ex;
         const bool free = h.ti.free != 0;
-        const TileEnv env{h.ti, h.ti.ubox[commit ? 0 : 1]};
+        const TileEnv env{h.ti, h.ti.tot[commit ? par : 2]};
         const float* ev = edgev + s * 2 * rows * QE;
         bool bad = false;
         // FOLD (D2Q9, FP16 storage at tau = 1): the populations stay at the

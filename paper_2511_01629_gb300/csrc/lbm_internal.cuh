@@ -10,12 +10,14 @@
 //   tile lists   list_cnt[2][ntiles], list_ent[2][ntiles][cap]: for each
 //                tile the particles whose bounding box overlaps it, built by
 //                the particle kernel for the next step (no per-node mask);
-//   velocity boxes  ubox: per particle a box of (2H + 1)^D entries, H =
-//                ceil(R) + 2, centred on floor(X): the fluid kernel stores the
-//                velocity of each node the particle owns there (float2 in 2D,
-//                float4 in 3D), the particle kernel sums the entries into the
-//                exact fixed-point totals of Eq. 22 and resets them to NaN,
-//                the mark of an empty entry.
+//   totals       tot[2][np][NPV]: the exact fixed-point sums of Eq. 22, added
+//                up by the fluid kernel (integer atomics, so the order does
+//                not matter) in the buffer of the step's parity; the particle
+//                kernel reads them and clears the other parity's buffer, which
+//                the next step adds to;
+//   step inputs  pst[2][np], Xp[2][np]: what a particle's neighbours read of it
+//                during a step (state and float position at the step's
+//                parity); the particle kernel writes the next parity's.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -121,6 +123,16 @@ struct GridBar {
     unsigned gen;
 };
 
+// What the particle kernel reads of any particle, its own or a neighbour, at
+// a step: the state entering it.  Kept per parity, because a block may still
+// read its neighbours while their blocks write the next step's.
+struct __align__(16) PState {
+    double X[3];     // X^n
+    double U[3];     // U^{n-1}
+    double ec, es;   // cos, sin of theta^n (ellipse; 1, 0 otherwise)
+};
+static_assert(sizeof(PState) == 64, "particle state layout");
+
 // Particle record read by the fluid kernel; written by the particle kernel
 // for the next step.  A disk (sphere) is inside |x - X|^2 <= R^2; an ellipse
 // (2D, shape = 1) with semi-axes a = R and b along e = (cos theta, sin theta)
@@ -135,7 +147,7 @@ struct __align__(16) PRec {
                        //   (an ellipse: only d2 > R2hi, its circumscribed circle)
     float a[3];      // solid-node acceleration (1 - rho_f/rho_s) g + A_i
     int shape;       // 0 disk or sphere, 1 ellipse
-    int pad;
+    int rows2;       // see RecConst
     double ec, es;   // cos, sin of theta^n (ellipse; 1, 0 otherwise)
     double b2;       // b * b
     float fc, fs;    // ec, es as float (filter test)
@@ -151,7 +163,8 @@ static_assert(sizeof(PRec) == 144, "particle record layout");
 struct RecConst {
     double R2, b2;
     float R2lo, R2hi, ia2, ib2, qlo, qhi;
-    int shape, pad;
+    int shape;
+    int rows2;  // 3D: rows at dy^2 + dz^2 > rows2 from floor(X) stay out of the sums of Eq. 22
 };
 static_assert(sizeof(RecConst) == 48, "record constants layout");
 
@@ -179,10 +192,10 @@ struct InstDesc {
     int* list_cnt[2];         // [ntiles]
     uint32_t* list_ent[2];    // [ntiles][LIST_CAP]
     void* list_rec[2];        // [ntiles][LIST_CAP] 64-byte candidate records (Cand), same slots
-    float* ubox;              // velocity boxes of the particles (see above), NaN when empty
-    float* ubox_scratch;      // same shape: sink of launches that do not advance the state
-    int2* boxinfo;            // [np] box of particle p: first entry, H
-    long long* btot;          // [np][NPV] the box's totals of Eq. 22 (k_box_sums)
+    long long* tot[2];        // [np][NPV] totals of Eq. 22 per parity (see above)
+    long long* tot_scratch;   // same shape: sink of launches that do not advance the state
+    PState* pst[2];           // [np] step inputs per parity (see above)
+    float4* Xp[2];            // [np] float copy of X^n (w = R) for the pair filter, per parity
     // particle state (FP64), [np][3] unless noted
     double* X;
     double* U;                // U^{n-1} entering the step, U^n after it
@@ -194,10 +207,10 @@ struct InstDesc {
     double* R;                // [np]
     double* ratio;            // [np] rho_s / rho_f
     int* count;               // [np]
-    double* Xk;               // [2][np][3] Algorithm-1 sub-step positions
+    double* Xk;               // [2][np][3] Algorithm-1 sub-step positions (K > 1)
     double* Ubar;             // [np][3]
     double* Acor;             // [np][3] sum of the sub-step corrections of Algorithm 1 (K > 1)
-    float* Xf;                // [2][np][4] float copy of X^{k} (w = R) for the pair filter
+    float* Xf;                // [2][np][4] float copy of X^{k} (w = R) for the pair filter (K > 1)
     float* Xsf;               // [2][np][4] float copy of X^{k} + Ubar/K (w = R): predicted positions
     const RecConst* rconst;   // [np] size and shape fields of the records
     double* pconst;           // [np][8]: 1 - rho_f/rho_s, C/eps_p, C/eps_w, 1/delta,

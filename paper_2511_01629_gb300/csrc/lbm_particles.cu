@@ -1,8 +1,14 @@
-// Per-particle FP64 kernels of lbmpen: the second pass of the rigid-body
-// projection (Eq. 22; the per-component finalisation is in lbm_common.cuh),
-// the predictor-corrector of Algorithm 1 with the repulsive collision forces
+// Per-particle FP64 kernel of lbmpen: the second pass of the rigid-body
+// projection (Eq. 22) from the totals that the fluid kernel added up, the
+// predictor-corrector of Algorithm 1 with the repulsive collision forces
 // (Eqs. 19-21), and the rebuild of each particle's record and tile-list
 // entries for the next step.
+//
+// One launch does all of it, with no barrier between the projection and the
+// pair forces: a particle's U^n follows from its totals by a few operations,
+// so a block takes the U^n of the few neighbours it needs from their totals
+// itself.  What a block reads of other particles (totals, state) is kept per
+// step parity, and a block writes only the other parity's.
 //
 // GB300 runs FP64 at a small fraction of its FP32 rate, and an FP64
 // instruction occupies a sub-partition's FP64 pipe for ~64 cycles whether one
@@ -30,53 +36,87 @@ __device__ __forceinline__ double extent_along(double R, double B, double ec, do
                           __dmul_rn(__dmul_rn(B, B), __dmul_rn(np, np))));
 }
 
-// Pair part of Eq. 21 on particle i at two position sets: Xk[src] (F1) and
-// Xk[src] + h Ubar (F2).  The block's particles all belong to one instance;
+// Position X^{k} of particle j and, with ub, its Ubar (FP64): before the first
+// sub-step from its state and totals of this step, later from the arrays that
+// its block wrote.
+template <bool FIRST>
+__device__ __forceinline__ void pair_operands(const InstDesc& in, int j, int src, int par, int D, bool ub, double* X,
+                                              double* Ub) {
+    for (int d = 0; d < 3; ++d) Ub[d] = 0.0;
+    if (!FIRST) {
+        for (int d = 0; d < 3; ++d) {
+            X[d] = in.Xk[(long long)src * in.np * 3 + 3 * j + d];
+            if (ub) Ub[d] = in.Ubar[3 * j + d];
+        }
+        return;
+    }
+    const PState& ps = in.pst[par][j];
+    for (int d = 0; d < 3; ++d) X[d] = ps.X[d];
+    if (!ub) return;
+    const long long* v = in.tot[par] + (long long)NPV * j;
+    if (v[0] == 0) return;
+    const double inv = rcp64((double)v[0]);
+    for (int d = 0; d < D; ++d) Ub[d] = 0.5 * (finalize_u(v[10 + d], inv) + ps.U[d]);
+}
+
+// Pair part of Eq. 21 on particle i at two position sets: X^{k} (F1) and
+// X^{k} + h Ubar (F2).  The block's particles all belong to one instance;
 // its positions are staged in shared memory in chunks and the lanes split
-// them.  An FP32 filter with a margin of 2.5 lattice units (a sub-step moves
-// a particle by |h Ubar| < 1/2) leaves only pairs near the interaction range
-// for the FP64 evaluation, which follows the reference operation order.
-__device__ void pair_chunk(const InstDesc& in, int i, int src, double h, int lane, const float4* xs,
+// them.  An FP32 filter leaves only pairs near the interaction range for the
+// FP64 evaluation, which follows the reference operation order.  The
+// predicted positions of the filter: staged (xs2) after the first sub-step; in the
+// first one taken from the totals, in FP32, for the few pairs within 2 of
+// range (a predicted position lies within |h Ubar| < sqrt(3)/2 of X^n, a larger
+// step is reported as ST_DISPLACEMENT).
+template <bool FIRST>
+__device__ void pair_chunk(const InstDesc& in, int i, int src, int par, double h, int D, int lane, const float4* xs,
                            const float4* xs2, int j0, int nj, float4 xi, float4 xi2, double cp,
                            double inv_delta, double* f1, double* f2) {
-    const double* Xb = in.Xk + (long long)src * in.np * 3;
     if (cp == 0.0) return;  // cp = C / eps_p of particle i
     const float reach = xi.w + (float)in.delta + 0.01f;  // FP32 positions carry < 1e-3 error
     const float nf[3] = {(float)in.n[0], (float)in.n[1], (float)in.n[2]};
     const bool per[3] = {in.periodic[0] && in.n[0] > 1, in.periodic[1] && in.n[1] > 1,
                          in.periodic[2] && in.n[2] > 1};
+    auto dist2 = [&](float4 a, float4 b) {
+        float dv[3] = {a.x - b.x, a.y - b.y, a.z - b.z};
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            if (per[d]) dv[d] -= nf[d] * rintf(dv[d] / nf[d]);
+        return dv[0] * dv[0] + dv[1] * dv[1] + dv[2] * dv[2];
+    };
+    // X + h Ubar of a particle in FP32, from its totals (sums below 2^62: exact to FP32's last bit)
+    auto predicted = [&](int j, float4 x) {
+        const long long* v = in.tot[par] + (long long)NPV * j;
+        const float s = v[0] > 0 ? 9.094947017729282e-13f / (float)v[0] : 0.f;  // 2^-40 / count
+        const PState& ps = in.pst[par][j];
+        const float hh = 0.5f * (float)h;
+        x.x += hh * ((float)v[10] * s + (float)ps.U[0]);
+        x.y += hh * ((float)v[11] * s + (float)ps.U[1]);
+        if (D == 3) x.z += hh * ((float)v[12] * s + (float)ps.U[2]);
+        return x;
+    };
     for (int jj = lane; jj < nj; jj += 32) {
         const int j = j0 + jj;
         if (j == i) continue;
-        bool near[2];
-        bool far = false;
-#pragma unroll
-        for (int pass = 0; pass < 2; ++pass) {
-            if (pass == 1 && far) break;
-            const float4 a = pass ? xi2 : xi, b = pass ? xs2[jj] : xs[jj];
-            float dv[3] = {a.x - b.x, a.y - b.y, a.z - b.z};
-#pragma unroll
-            for (int d = 0; d < 3; ++d)
-                if (per[d]) dv[d] -= nf[d] * rintf(dv[d] / nf[d]);
-            const float lim = reach + b.w;
-            const float d2 = dv[0] * dv[0] + dv[1] * dv[1] + dv[2] * dv[2];
-            near[pass] = d2 <= lim * lim;
-            // a predicted position lies within |h Ubar| < sqrt(3)/2 of X^n (a larger
-            // step is reported as ST_DISPLACEMENT), so a pair more than 2 beyond
-            // range at X^n is out of range at both position sets
-            if (pass == 0) far = d2 > (lim + 2.0f) * (lim + 2.0f);
-        }
-        if (far) continue;
+        const float4 b = xs[jj];
+        const float lim = reach + b.w;
+        const float d2 = dist2(xi, b);
+        if (d2 > (lim + 2.0f) * (lim + 2.0f)) continue;  // out of range at both position sets
+        const float e2 = FIRST ? dist2(predicted(i, xi), predicted(j, b)) : dist2(xi2, xs2[jj]);
+        const bool near[2] = {d2 <= lim * lim, e2 <= lim * lim};
         if (!near[0] && !near[1]) continue;
         const double Bi = in.pconst[PCONST_N * i + PC_B], Bj = in.pconst[PCONST_N * j + PC_B];
         const bool ell = Bi != in.R[i] || Bj != in.R[j];
+        double Xi[3], Xj[3], Ui[3], Uj[3];
+        pair_operands<FIRST>(in, i, src, par, D, near[1], Xi, Ui);
+        pair_operands<FIRST>(in, j, src, par, D, near[1], Xj, Uj);
         for (int pass = 0; pass < 2; ++pass) {
             if (!near[pass]) continue;
             const double sh = pass ? h : 0.0;
             double dd[3];
             for (int d = 0; d < 3; ++d) {
-                const double xi_d = Xb[3 * i + d] + sh * in.Ubar[3 * i + d];
-                const double xj_d = Xb[3 * j + d] + sh * in.Ubar[3 * j + d];
+                const double xi_d = Xi[d] + sh * Ui[d];
+                const double xj_d = Xj[d] + sh * Uj[d];
                 dd[d] = xi_d - xj_d;
                 if (per[d]) {
                     const double half = 0.5 * in.n[d];
@@ -89,7 +129,7 @@ __device__ void pair_chunk(const InstDesc& in, int i, int src, double h, int lan
             double range = in.R[i] + in.R[j] + in.delta;
             if (ell && dij > 0.0) {  // ellipses (2D): extents along the line of centres
                 const double nx = dd[0] / dij, ny = dd[1] / dij;
-                const PRec &ri = in.prec[i], &rj = in.prec[j];
+                const PState &ri = in.pst[par][i], &rj = in.pst[par][j];
                 range = extent_along(in.R[i], Bi, ri.ec, ri.es, nx, ny) +
                         extent_along(in.R[j], Bj, rj.ec, rj.es, nx, ny) + in.delta;
             }
@@ -155,7 +195,7 @@ __device__ AxisTiles axis_tiles_f(float X, float R, int n, int T, int ntile, int
     int lo = (int)floorf(X - R) - 1, hi = (int)floorf(X + R) + 1;
     AxisTiles t{0, 1, 0, 0};
     if (!periodic) {
-        lo = max(lo, 0);
+        lo = min(max(lo, 0), n - 1);  // in range wherever a failed run may have put X
         hi = max(min(hi, n - 1), lo);
         t.a0 = lo / T;
         t.na = hi / T - t.a0 + 1;
@@ -225,7 +265,7 @@ __device__ __forceinline__ void record_radius(const InstDesc& in, PRec& pr, cons
     pr.R2hi = rc.R2hi;
     pr.ntiles = nt;
     pr.shape = rc.shape;
-    pr.pad = 0;
+    pr.rows2 = rc.rows2;
     pr.b2 = rc.b2;
     pr.ia2 = rc.ia2;
     pr.ib2 = rc.ib2;
@@ -249,7 +289,7 @@ __device__ __forceinline__ void record_orientation(PRec& pr, bool ellipse, doubl
 // Record of particle p from its state (X, A, theta) and constants (R, B,
 // 1 - rho_f/rho_s), with the tiles of its bounding box (slots k enumerate them
 // x-fastest; no tile is listed twice).  One thread.
-__device__ void make_record_from(const InstDesc& in, int p, int D, const Shape& sh, AxisTiles* at,
+__device__ PRec make_record_from(const InstDesc& in, int p, int D, const Shape& sh, AxisTiles* at,
                                  const double* Xp, const double* Ap, double R, double B, double theta,
                                  float gfac) {
     PRec pr;
@@ -266,43 +306,54 @@ __device__ void make_record_from(const InstDesc& in, int p, int D, const Shape& 
     record_radius(in, pr, in.rconst[p], nt);
     record_orientation(pr, B != R, theta);
     in.prec_out[p] = pr;
+    return pr;
 }
 
-__device__ void make_record(const InstDesc& in, int p, int D, const Shape& sh, AxisTiles* at) {
-    double X[3], A[3];
-    for (int d = 0; d < 3; ++d) {
-        X[d] = in.X[3 * p + d];
-        A[d] = in.A[3 * p + d];
-    }
-    make_record_from(in, p, D, sh, at, X, A, in.pconst[PCONST_N * p + PC_R],
-                     in.pconst[PCONST_N * p + PC_B], in.theta[3 * p + 2],
-                     (float)in.pconst[PCONST_N * p + PC_GFAC]);
-}
-
-// List entries of particle p in the tiles of its bounding box (lanes share),
-// from its record for the next step (prec_out[p]): the entry p << KBITS | k
-// and, in the same slot, the 64-byte candidate record the TMA kernel copies.
-__device__ void append_tiles(const InstDesc& in, int p, const AxisTiles* at, int lpar, int lane,
-                             int nl) {
-    const int cnt[3] = {at[0].na + at[0].nb, at[1].na + at[1].nb, at[2].na + at[2].nb};
-    const int nt = cnt[0] * cnt[1] * cnt[2];
-    if (lane >= nt) return;
-    const PRec& pr = in.prec_out[p];
+// The candidate record of a particle (Cand) from its record's fields.
+__device__ __forceinline__ Cand make_cand(const PRec& pr, int p) {
     Cand cd;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         cd.ref[d] = pr.ref[d];
         cd.frac[d] = pr.frac[d];
         cd.a[d] = pr.a[d];
-
     }
     cd.R2lo = pr.R2lo;
     cd.R2hi = pr.R2hi;
     cd.p = p;
-    const int2 bi = in.boxinfo[p];
-    cd.boff = bi.x;
-    cd.bh = bi.y;
+    cd.k = 0;
+    cd.rows2 = pr.rows2;
+    cd.pad = 0;
     cd.shape = pr.shape;
+    return cd;
+}
+
+__device__ Cand make_record(const InstDesc& in, int p, int D, const Shape& sh, AxisTiles* at, int lpar) {
+    double X[3], A[3];
+    for (int d = 0; d < 3; ++d) {
+        X[d] = in.X[3 * p + d];
+        A[d] = in.A[3 * p + d];
+    }
+    const double R = in.pconst[PCONST_N * p + PC_R];
+    const PRec pr = make_record_from(in, p, D, sh, at, X, A, R, in.pconst[PCONST_N * p + PC_B], in.theta[3 * p + 2],
+                                     (float)in.pconst[PCONST_N * p + PC_GFAC]);
+    PState& ps = in.pst[lpar][p];
+    for (int d = 0; d < 3; ++d) {
+        ps.X[d] = X[d];
+        ps.U[d] = in.U[3 * p + d];
+    }
+    ps.ec = pr.ec;
+    ps.es = pr.es;
+    in.Xp[lpar][p] = make_float4((float)X[0], (float)X[1], (float)X[2], (float)R);
+    return make_cand(pr, p);
+}
+
+// List entries of particle p in the tiles of its bounding box (lanes share):
+// the entry p << KBITS | k and, in the same slot, the 64-byte candidate record
+// cd that the fluid kernel copies.
+__device__ void append_tiles(const InstDesc& in, int p, const AxisTiles* at, Cand cd, int lpar, int lane, int nl) {
+    const int cnt[3] = {at[0].na + at[0].nb, at[1].na + at[1].nb, at[2].na + at[2].nb};
+    const int nt = cnt[0] * cnt[1] * cnt[2];
     Cand* rec = static_cast<Cand*>(in.list_rec[lpar]);
     for (int k = lane; k < nt && k < in.maxk; k += nl) {
         const int kx = k % cnt[0], ky = (k / cnt[0]) % cnt[1], kz = k / (cnt[0] * cnt[1]);
@@ -327,26 +378,23 @@ __device__ void append_tiles(const InstDesc& in, int p, const AxisTiles* at, int
 // sub-step A^{n+1}, theta^{n+1}, U^{n-1} <- U^n and the record for the next
 // step.  Each lane evaluates the expressions of a serial loop over d.
 // The operands of update_lane, loaded in one batch before the pair search so
-// that their latency overlaps it.
+// that their latency overlaps it; on the first sub-step the projection's
+// translation (Eq. 22) is part of it.
 struct LaneIn {
-    double X0, Ub, Wn, Un, Wo, Th, invrhos, cw, idl, Ri, Bi, gfac, invc, Acor, ec, es;
+    double X0, Ub, Un, invrhos, cw, idl, Ri, Bi, gfac, invc, Acor, ec, es;
     int cnt;
     RecConst rc;
 };
 
-__device__ __forceinline__ LaneIn load_lane(const InstDesc& in, int i, int d, bool valid, int src, int first) {
+__device__ __forceinline__ LaneIn load_lane(const InstDesc& in, int i, int d, bool valid, int src, int par, double h,
+                                            int first, int D) {
     if (!valid) {  // in-range operands for the shuffle-only lanes
         i = 0;
         d = 0;
     }
     const long long j = 3LL * i + d;
     LaneIn L;
-    L.X0 = in.Xk[(long long)src * in.np * 3 + j];
-    L.Ub = in.Ubar[j];
-    L.Wn = in.Wn[j];
-    L.Un = in.Un[j];
-    L.Wo = in.W[j];
-    L.Th = in.theta[j];
+    const PState& ps = in.pst[par][i];
     const double* pc = in.pconst + PCONST_N * i;
     L.invrhos = pc[PC_INVRHOS];
     L.cw = pc[PC_CWALL];
@@ -354,38 +402,99 @@ __device__ __forceinline__ LaneIn load_lane(const InstDesc& in, int i, int d, bo
     L.Ri = pc[PC_R];
     L.Bi = pc[PC_B];
     L.gfac = pc[PC_GFAC];
-    L.invc = in.invc[i];
-    L.cnt = in.count[i];
-    L.Acor = first ? 0.0 : in.Acor[j];
-    L.ec = in.prec[i].ec;  // orientation theta^n of this step's record
-    L.es = in.prec[i].es;
+    L.ec = ps.ec;  // orientation theta^n of this step's record
+    L.es = ps.es;
     L.rc = in.rconst[i];
+    if (first) {
+        const long long* v = in.tot[par] + (long long)NPV * i;
+        const long long n = v[0], su = v[10 + d];
+        const double Uold = ps.U[d];
+        L.X0 = ps.X[d];
+        L.Acor = 0.0;
+        L.cnt = (int)n;
+        L.invc = 0.0;
+        L.Un = Uold;
+        L.Ub = 0.0;
+        if (n != 0) {
+            L.invc = rcp64((double)n);
+            L.Un = d < D ? finalize_u(su, L.invc) : 0.0;
+            L.Ub = d < D ? 0.5 * (L.Un + Uold) : 0.0;
+        }
+        if (valid) {
+            in.Un[j] = L.Un;
+            if (n == 0 && d == 0) atomicOr(in.status, ST_PARTICLE);
+            if (!(fabs(L.Ub) < 0.5)) atomicOr(in.status, ST_DISPLACEMENT);
+            if (d == 0) in.count[i] = (int)n;
+            if (in.K > 1) {  // the later sub-steps read these
+                in.Ubar[j] = L.Ub;
+                if (d == 0) in.invc[i] = L.invc;
+            }
+        }
+    } else {
+        L.X0 = in.Xk[(long long)src * in.np * 3 + j];
+        L.Ub = in.Ubar[j];
+        L.Un = in.Un[j];
+        L.invc = in.invc[i];
+        L.cnt = in.count[i];
+        L.Acor = in.Acor[j];
+    }
     return L;
 }
 
+// Rotation of particle i, component d: W^n (first sub-step, Eq. 22) and, on
+// the last one, theta^{n+1} (reading: trapezoid of W) with the record's
+// orientation.  Runs on its own warp beside update_lane.
+__device__ __forceinline__ void rotate_lane(const InstDesc& in, int i, int d, int par, int first, int last, int D) {
+    const long long j = 3LL * i + d;
+    const double Th = in.theta[j], Wo = in.W[j];
+    double Wn;
+    if (first) {
+        double* geo = in.adj_geo ? in.adj_geo + (long long)NPV * i : nullptr;
+        const long long* v = in.tot[par] + (long long)NPV * i;
+        Wn = D == 2 ? finalize_rotation<2>(v, in.pst[par][i].X, d, geo) : finalize_rotation<3>(v, in.pst[par][i].X, d, geo);
+        in.Wn[j] = Wn;
+    } else {
+        Wn = in.Wn[j];
+    }
+    if (!last) return;
+    const double Tn = Th + 0.5 * (Wn + Wo);
+    in.theta[j] = Tn;
+    in.W[j] = Wn;
+    if (in.rec_state) {
+        in.rec_state[16LL * i + 6 + d] = Wn;
+        in.rec_state[16LL * i + 9 + d] = Tn;
+    }
+    if (d == 2) {
+        const double* pc = in.pconst + PCONST_N * i;
+        PRec& pr = in.prec_out[i];
+        record_orientation(pr, pc[PC_B] != pc[PC_R], Tn);
+        PState& ps = in.pst[par ^ 1][i];
+        ps.ec = pr.ec;
+        ps.es = pr.es;
+    }
+}
+
 __device__ void update_lane(const InstDesc& in, int i, int d, int sl, bool valid, const double* F1in,
-                            const double* F2in, int src, double h, int first, int last, int D,
-                            const Shape& sh, AxisTiles* at, const LaneIn& L) {
+                            const double* F2in, int src, int par, double h, int first, int last, int D,
+                            const Shape& sh, AxisTiles* at, Cand& cd, const LaneIn& L) {
     if (!valid) {  // in-range operands for the shuffle-only lanes; nothing is stored
         i = 0;
         d = 0;
     }
     const int dst = src ^ 1;
     const long long j = 3LL * i + d;
-    const double X0 = L.X0, Ub = L.Ub, Wn = L.Wn, Un = L.Un, Wo = L.Wo, Th = L.Th;
-    double F1 = F1in[d], F2 = F2in[d];
-    const double invrhos = L.invrhos, cw = L.cw, idl = L.idl, Ri = L.Ri, Bi = L.Bi, gfac = L.gfac;
-    const double invc = L.invc;
-    const int cnt = L.cnt;
-    const double invM = invrhos * invc;  // 1 / (rho_s n)
+    const double X0 = L.X0, Ub = L.Ub;
+    double F1 = F1in ? F1in[d] : 0.0, F2 = F2in ? F2in[d] : 0.0;
+    const double Ri = L.Ri, Bi = L.Bi;
+    const double invM = L.invrhos * L.invc;  // 1 / (rho_s n)
     const double Xst = fma(h, Ub, X0);
     // extent along axis d: the radius, or for an ellipse at theta^n (this
     // step's record) its support distance normal to the walls of axis d
     double Rd = Ri;
     if (Bi != Ri && d < 2)
         Rd = d == 0 ? extent_along(Ri, Bi, L.ec, L.es, 1.0, 0.0) : extent_along(Ri, Bi, L.ec, L.es, 0.0, 1.0);
-    wall_force_d(in, d, X0, F1, cw, idl, Rd);
-    wall_force_d(in, d, Xst, F2, cw, idl, Rd);
+    wall_force_d(in, d, X0, F1, L.cw, L.idl, Rd);
+    wall_force_d(in, d, Xst, F2, L.cw, L.idl, Rd);
     const double c = 0.25 * h * h * invM;  // (1 / 2M) h^2 / 2
     const double cor = c * (F1 + F2);      // this sub-step's correction
     const double Xn = Xst + cor;
@@ -419,38 +528,46 @@ __device__ void update_lane(const InstDesc& in, int i, int d, int sl, bool valid
             left = true;
         }
     }
-    const double Tn = Th + 0.5 * (Wn + Wo);
-    if (valid) {
-        in.A[j] = An;
-        in.X[j] = xn;
-        in.theta[j] = Tn;
-        in.U[j] = Un;
-        in.W[j] = Wn;
-        if (left) atomicOr(in.status, ST_PARTICLE);
-        if (in.rec_state) {  // adjoint recording: the state this step hands to the next
-            double* r = in.rec_state + 16LL * i;
-            r[d] = xn;
-            r[3 + d] = Un;
-            r[6 + d] = Wn;
-            r[9 + d] = Tn;
-            r[12 + d] = An;
-            if (d == 0) r[15] = (double)cnt;
-        }
-    }
-    const RecComp r = record_component(in, d, D, sh, xn, An, Rf, (float)gfac);
+    const RecComp r = record_component(in, d, D, sh, xn, An, Rf, (float)L.gfac);
     const int ct = r.t.na + r.t.nb;
     const int nt = __shfl_sync(0xffffffffu, ct, sl) * __shfl_sync(0xffffffffu, ct, sl + PB) *
                    __shfl_sync(0xffffffffu, ct, sl + 2 * PB);
-    if (valid) {
-        PRec& pr = in.prec_out[i];
-        pr.X[d] = xn;
-        pr.ref[d] = r.ref;
-        pr.frac[d] = r.frac;
-        pr.a[d] = r.a;
-        at[d] = r.t;
-        if (d == 0) record_radius(in, pr, L.rc, nt);
-        if (d == 2) record_orientation(pr, Bi != Ri, Tn);
+    if (!valid) return;
+    at[d] = r.t;  // shared: what append_tiles needs
+    cd.ref[d] = r.ref;
+    cd.frac[d] = r.frac;
+    cd.a[d] = r.a;
+    if (d == 0) {
+        cd.R2lo = L.rc.R2lo;
+        cd.R2hi = L.rc.R2hi;
+        cd.p = i;
+        cd.rows2 = L.rc.rows2;
+        cd.pad = 0;
+        cd.shape = L.rc.shape;
     }
+    in.A[j] = An;
+    in.X[j] = xn;
+    in.U[j] = L.Un;
+    PState& ps = in.pst[par ^ 1][i];
+    ps.X[d] = xn;
+    ps.U[d] = L.Un;
+    float* xp = reinterpret_cast<float*>(in.Xp[par ^ 1] + i);
+    xp[d] = (float)xn;
+    if (d == 0) xp[3] = Rf;
+    if (left) atomicOr(in.status, ST_PARTICLE);
+    if (in.rec_state) {  // adjoint recording: the state this step hands to the next
+        double* q = in.rec_state + 16LL * i;
+        q[d] = xn;
+        q[3 + d] = L.Un;
+        q[12 + d] = An;
+        if (d == 0) q[15] = (double)L.cnt;
+    }
+    PRec& pr = in.prec_out[i];
+    pr.X[d] = xn;
+    pr.ref[d] = r.ref;
+    pr.frac[d] = r.frac;
+    pr.a[d] = r.a;
+    if (d == 0) record_radius(in, pr, L.rc, nt);
 }
 
 // ------------------------------------------------------------- the kernel --
@@ -499,220 +616,114 @@ __device__ bool grid_sync(GridBar* gb, int* status, unsigned long long limit_ns)
     return __syncthreads_and(ok) != 0;
 }
 
-// The totals of Eq. 22 of every particle from its velocity box, one block of
-// BS_THREADS per particle, launched between the fluid kernel and the particle
-// kernel: the threads take the box's entries (3D: only the rows that can reach
-// the sphere), turn every filled one (the nodes the particle owned in this
-// step's fluid kernel) into exact integer sums, and mark it empty again for
-// the next step.  The warps' totals are exact (integer reductions; 64-bit
-// sums by limbs) and so is their sum, so the totals do not depend on the order.
-constexpr int BS_THREADS = 128;  // 4 blocks per SM: 500 particles in one wave
-constexpr int BS_PER = 8;  // entries of a thread in flight at a time
-
-template <int D>
-__device__ __forceinline__ void box_block_sums(const InstDesc& in, int p, long long (*red)[NPV]) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int2 bi = in.boxinfo[p];
-    const int H = bi.y, side = 2 * H + 1;
-    const int nent = D == 2 ? side * side : side * side * side;  // < 2^31 for R <= 40
-    const int hmax = (H - 1) * (H - 1);  // owned nodes have |d| <= R + 1 <= H - 1
-    int icnt = 0, id[3] = {0, 0, 0}, idd[6] = {0, 0, 0, 0, 0, 0};
-    long long su[3] = {0, 0, 0}, sl[3] = {0, 0, 0};
-    const float nanv = __int_as_float(0x7fffffff);
-    for (int e0 = 0; e0 < nent; e0 += BS_THREADS * BS_PER) {
-        float4 u[BS_PER];
-        int dd[BS_PER][3];
-#pragma unroll
-        for (int j = 0; j < BS_PER; ++j) {
-            const int e = e0 + tid + BS_THREADS * j;
-            const int dx = e % side - H, dy = (e / side) % side - H, dz = D == 3 ? e / (side * side) - H : 0;
-            dd[j][0] = dx;
-            dd[j][1] = dy;
-            dd[j][2] = dz;
-            u[j] = make_float4(nanv, nanv, nanv, 0.f);
-            if (e < nent && (D == 2 || dy * dy + dz * dz <= hmax)) {
-                if (D == 2) {
-                    const float2 t = __ldcg(reinterpret_cast<const float2*>(in.ubox) + bi.x + e);
-                    u[j].x = t.x;
-                    u[j].y = t.y;
-                } else {
-                    u[j] = __ldcg(reinterpret_cast<const float4*>(in.ubox) + bi.x + e);
-                }
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < BS_PER; ++j) {
-            if (!(u[j].x == u[j].x)) continue;  // empty (NaN)
-            const int dx = dd[j][0], dy = dd[j][1], dz = dd[j][2];
-            const long long ux[3] = {to_fx32(u[j].x), to_fx32(u[j].y), D == 3 ? to_fx32(u[j].z) : 0};
-            icnt += 1;
-            id[0] += dx; id[1] += dy; id[2] += dz;
-            idd[0] += dx * dx; idd[1] += dy * dy; idd[2] += dz * dz;
-            idd[3] += dx * dy; idd[4] += dx * dz; idd[5] += dy * dz;
-            su[0] += ux[0]; su[1] += ux[1]; su[2] += ux[2];
-            sl[2] += (long long)dx * ux[1] - (long long)dy * ux[0];
-            if (D == 3) {
-                sl[0] += (long long)dy * ux[2] - (long long)dz * ux[1];
-                sl[1] += (long long)dz * ux[0] - (long long)dx * ux[2];
-            }
-            const long long e = bi.x + (long long)(e0 + tid + BS_THREADS * j);
-            if (D == 2) reinterpret_cast<float2*>(in.ubox)[e] = make_float2(nanv, nanv);
-            else reinterpret_cast<float4*>(in.ubox)[e] = make_float4(nanv, nanv, nanv, 0.f);
-        }
-    }
-    long long v[NPV];
-    v[0] = __reduce_add_sync(0xffffffffu, icnt);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) v[1 + k] = k < D ? (long long)__reduce_add_sync(0xffffffffu, id[k]) : 0;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        const bool need = D == 3 || k == 0 || k == 1 || k == 3;
-        v[4 + k] = need ? (long long)__reduce_add_sync(0xffffffffu, idd[k]) : 0;
-    }
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        v[10 + k] = k < D ? warp_sum_fx(su[k]) : 0;
-        v[13 + k] = (D == 3 || k == 2) ? warp_sum_fx(sl[k]) : 0;
-    }
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < NPV; ++k) red[warp][k] = v[k];
-}
-
-__global__ void __launch_bounds__(BS_THREADS, 4) k_box_sums(const InstDesc* __restrict__ insts,
-                                                       const PartRef* __restrict__ refs, int D) {
-    __shared__ long long red[BS_THREADS / 32][NPV];
-    __shared__ long long tot[NPV];
-    const PartRef r = refs[blockIdx.x];
-    if (r.inst < 0) return;  // padding entry (block-uniform)
-    const InstDesc& in = insts[r.inst];
-    if (threadIdx.x >= BS_THREADS - 4) {  // warm L1 with what the second pass reads
-        const int k = threadIdx.x - (BS_THREADS - 4);
-        const char* a = k < 2 ? reinterpret_cast<const char*>(in.prec + r.p) + 128 * k
-                              : (k == 2 ? reinterpret_cast<const char*>(in.U + 3 * r.p)
-                                        : reinterpret_cast<const char*>(in.pconst + PCONST_N * r.p));
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(a));
-    }
-    if (D == 2) box_block_sums<2>(in, r.p, red);
-    else box_block_sums<3>(in, r.p, red);
-    __syncthreads();
-    if (threadIdx.x < NPV) {
-        long long t = 0;
-        for (int w = 0; w < BS_THREADS / 32; ++w) t += red[w][threadIdx.x];
-        in.btot[(long long)r.p * NPV + threadIdx.x] = t;
-        tot[threadIdx.x] = t;
-    }
-    __syncthreads();
-    // the second pass of Eq. 22 for this particle: translation on warp 0,
-    // rotation on warp 1, one lane per component; the kernel boundary after
-    // it is the grid-wide barrier Algorithm 1 needs (every particle's U^n)
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane < 3) {
-        if (warp == 0) {
-            if (D == 2) finalize_translation<2>(in, r.p, tot, lane);
-            else finalize_translation<3>(in, r.p, tot, lane);
-        } else if (warp == 1) {
-            if (D == 2) finalize_rotation<2>(in, r.p, tot, lane);
-            else finalize_rotation<3>(in, r.p, tot, lane);
-        }
-    }
-}
-
-// Phase k (1..K): sub-step k of Algorithm 1, positions Xk[src] -> Xk[src ^ 1];
-// the block's warps find the pair forces (one particle each), one thread per
-// particle does the FP64 update.
-__device__ void phase_substep(const InstDesc& in, const PartRef* refs, int ntotal, int D, int gp0,
-                              int src, int K, int first, int last, const Shape& sh, float4* xs, float4* xs2,
-                              double (*sF)[6], AxisTiles (*sAT)[3]) {
+// Phase k (1..K): sub-step k of Algorithm 1 for the block's particles (slot s
+// is particle i0 + s; np of its instance), positions of buffer src -> src ^ 1
+// (the first from the state).  The block's warps find the pair forces (one
+// particle each); warp 0 does the FP64 update, one lane per particle component,
+// warp 1 the rotation, and warp 2 clears the totals that the next step adds to.
+template <bool FIRST>
+__device__ void phase_substep(const InstDesc& in, int i0, int D, int src, int par, int last, const Shape& sh,
+                              float4* xs, float4* xs2, double (*sF)[6], AxisTiles (*sAT)[3], Cand* sC) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const double h = in.hK;
-    const int gp = gp0 + warp;
-    const bool mine = warp < PB && gp < ntotal && refs[gp].inst >= 0;
-    const int i = mine ? refs[gp].p : 0;
-    double f1[3] = {0, 0, 0}, f2[3] = {0, 0, 0};
-    const float4* Xfb = reinterpret_cast<const float4*>(in.Xf) + (long long)src * in.np;
-    const float4* Xsb = reinterpret_cast<const float4*>(in.Xsf) + (long long)src * in.np;
-    float4 xi = make_float4(0.f, 0.f, 0.f, 0.f), xi2 = xi;
-    double cp = 0.0, idl = 0.0;
-    if (mine) {  // issued before the staging barrier, so the loads overlap it
-        xi = Xfb[i];
-        xi2 = Xsb[i];
-        cp = in.pconst[PCONST_N * i + PC_CPAIR];
-        idl = in.pconst[PCONST_N * i + PC_INVDELTA];
-    }
-    // warp 0: the operands of the update (one lane per particle component)
+    const int i = i0 + warp;
+    const bool mine = i < in.np;
+    // warps 0 and 1: particle slot and component of the lane
     const int usl = lane & (PB - 1), ud = lane / PB;
-    const bool uvalid = warp == 0 && ud < 3 && gp0 + usl < ntotal && refs[gp0 + usl].inst >= 0;
+    const bool uvalid = ud < 3 && i0 + usl < in.np;
     LaneIn li;
-    if (warp == 0) li = load_lane(in, uvalid ? refs[gp0 + usl].p : 0, ud, uvalid, src, first);
-    for (int j0 = 0; j0 < in.np; j0 += XCHUNK) {
-        const int nj = min(XCHUNK, in.np - j0);
-        // every load of the chunk in flight at once, then the shared stores
-        constexpr int PER = XCHUNK / 256;  // blockDim.x == 256
-        float4 ra[PER], rb[PER];
+    if (warp == 0) li = load_lane(in, i0 + usl, ud, uvalid, src, par, h, FIRST, D);
+    const bool pairs = in.np > 1;  // one particle: nothing to search
+    if (pairs) {
+        double f1[3] = {0, 0, 0}, f2[3] = {0, 0, 0};
+        const float4* Xfb = FIRST ? in.Xp[par] : reinterpret_cast<const float4*>(in.Xf) + (long long)src * in.np;
+        const float4* Xsb = reinterpret_cast<const float4*>(in.Xsf) + (long long)src * in.np;
+        float4 xi = make_float4(0.f, 0.f, 0.f, 0.f), xi2 = xi;
+        double cp = 0.0, idl = 0.0;
+        if (mine) {  // issued before the staging barrier, so the loads overlap it
+            xi = Xfb[i];
+            if (!FIRST) xi2 = Xsb[i];
+            cp = in.pconst[PCONST_N * i + PC_CPAIR];
+            idl = in.pconst[PCONST_N * i + PC_INVDELTA];
+        }
+        for (int j0 = 0; j0 < in.np; j0 += XCHUNK) {
+            const int nj = min(XCHUNK, in.np - j0);
+            // every load of the chunk in flight at once, then the shared stores
+            constexpr int PER = XCHUNK / 256;  // blockDim.x == 256
+            float4 ra[PER], rb[PER];
 #pragma unroll
-        for (int u = 0; u < PER; ++u) {
-            const int k = threadIdx.x + 256 * u;
-            if (k < nj) {
-                ra[u] = Xfb[j0 + k];
-                rb[u] = Xsb[j0 + k];
+            for (int u = 0; u < PER; ++u) {
+                const int k = threadIdx.x + 256 * u;
+                if (k < nj) {
+                    ra[u] = Xfb[j0 + k];
+                    if (!FIRST) rb[u] = Xsb[j0 + k];
+                }
             }
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < PER; ++u) {
+                const int k = threadIdx.x + 256 * u;
+                if (k < nj) {
+                    xs[k] = ra[u];
+                    if (!FIRST) xs2[k] = rb[u];
+                }
+            }
+            __syncthreads();
+            if (mine) pair_chunk<FIRST>(in, i, src, par, h, D, lane, xs, xs2, j0, nj, xi, xi2, cp, idl, f1, f2);
+        }
+        if (mine) {
+            double F1[3], F2[3];
+            gather_pairs(f1, f2, F1, F2);
+            if (lane == 0)
+                for (int d = 0; d < 3; ++d) {
+                    sF[warp][d] = F1[d];
+                    sF[warp][3 + d] = F2[d];
+                }
         }
         __syncthreads();
-#pragma unroll
-        for (int u = 0; u < PER; ++u) {
-            const int k = threadIdx.x + 256 * u;
-            if (k < nj) {
-                xs[k] = ra[u];
-                xs2[k] = rb[u];
-            }
-        }
-        __syncthreads();
-        if (mine) pair_chunk(in, i, src, h, lane, xs, xs2, j0, nj, xi, xi2, cp, idl, f1, f2);
     }
-    if (mine) {
-        double F1[3], F2[3];
-        gather_pairs(f1, f2, F1, F2);
-        if (lane == 0)
-            for (int d = 0; d < 3; ++d) {
-                sF[warp][d] = F1[d];
-                sF[warp][3 + d] = F2[d];
-            }
+    if (warp == 0) {
+        update_lane(in, i0 + usl, ud, usl, uvalid, pairs ? sF[usl] : nullptr, pairs ? sF[usl] + 3 : nullptr, src, par, h,
+                    FIRST, last, D, sh, sAT[usl], sC[usl], li);
+    } else if (warp == 1) {
+        if (uvalid) rotate_lane(in, i0 + usl, ud, par, FIRST, last, D);
+    } else if (FIRST && warp == 2) {
+        for (int k = lane; k < PB * NPV; k += 32)
+            if (i0 + k / NPV < in.np) in.tot[par ^ 1][(long long)NPV * i0 + k] = 0;
     }
-    __syncthreads();
-    if (warp == 0)  // one lane per (particle, component)
-        update_lane(in, uvalid ? refs[gp0 + usl].p : 0, ud, usl, uvalid, sF[usl], sF[usl] + 3, src, h, first, last,
-                    D, sh, sAT[usl], li);
 }
 
 // Particle part of one time step for the block's 8 particles (one instance),
-// phases first..last, phase k = sub-step k of Algorithm 1 (the projection of
-// Eq. 22 ran in k_box_sums); after the last sub-step the warps append their
+// phases first..last, phase k = sub-step k of Algorithm 1, the first after the
+// projection of Eq. 22; after the last sub-step the warps append their
 // particle to the next step's tile lists.  With more than one phase (K > 1)
 // the blocks meet at grid barriers between phases (the launch guarantees they
 // are all resident); with K = 1 there is no barrier.
 __global__ void __launch_bounds__(256, 1) k_particles(const InstDesc* __restrict__ insts,
-                                                   const PartRef* __restrict__ refs, int ntotal,
+                                                   const PartRef* __restrict__ refs, int ninst,
                                                    int D, int K, int first, int last, int lpar,
                                                    Shape sh, GridBar* gb, unsigned long long wait_ns) {
     __shared__ double sF[PB][6];
     __shared__ AxisTiles sAT[PB][3];
+    __shared__ Cand sC[PB];
     __shared__ float4 xs[XCHUNK];
     __shared__ float4 xs2[XCHUNK];
-    const int gp0 = blockIdx.x * PB;
     __shared__ __align__(16) InstDesc sdesc;
-    stage_desc(&sdesc, insts[refs[gp0].inst]);  // blocks never straddle instances
+    // blocks never straddle instances; one instance needs no look at the table
+    PartRef r0{0, (int)blockIdx.x * PB};
+    if (ninst > 1) r0 = refs[blockIdx.x * PB];
+    stage_desc(&sdesc, insts[r0.inst]);
     const InstDesc& in = sdesc;
+    const int par = lpar ^ 1, i0 = r0.p;
     for (int ph = first; ph <= last; ++ph) {
         if (ph > first && !grid_sync(gb, in.status, wait_ns)) return;
-        phase_substep(in, refs, ntotal, D, gp0, (ph - 1) & 1, K, ph == 1, ph == K, sh, xs, xs2, sF, sAT);
+        if (ph == 1) phase_substep<true>(in, i0, D, 0, par, K == 1, sh, xs, xs2, sF, sAT, sC);
+        else phase_substep<false>(in, i0, D, (ph - 1) & 1, par, ph == K, sh, xs, xs2, sF, sAT, sC);
     }
     if (last == K) {
         __syncthreads();  // records and tile ranges of the block's particles are ready
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        const int gp = gp0 + warp;
-        if (warp < PB && gp < ntotal && refs[gp].inst >= 0)
-            append_tiles(in, refs[gp].p, sAT[warp], lpar, lane, 32);
+        if (warp < PB && i0 + warp < in.np) append_tiles(in, i0 + warp, sAT[warp], sC[warp], lpar, lane, 32);
     }
 }
 
@@ -725,8 +736,8 @@ __global__ void k_publish(const InstDesc* __restrict__ insts, const PartRef* __r
     const PartRef r = refs[gp];
     if (r.inst < 0) return;
     AxisTiles at[3];
-    make_record(insts[r.inst], r.p, D, sh, at);
-    append_tiles(insts[r.inst], r.p, at, lpar, 0, 1);
+    const Cand cd = make_record(insts[r.inst], r.p, D, sh, at, lpar);
+    append_tiles(insts[r.inst], r.p, at, cd, lpar, 0, 1);
 }
 
 int particle_blocks_resident(int num_sms) {
@@ -737,22 +748,17 @@ int particle_blocks_resident(int num_sms) {
 
 // The particle part of a step: one launch with grid barriers when all blocks
 // fit on the GPU at once, else one launch per phase.
-cudaError_t launch_particles(const InstDesc* insts, const PartRef* refs, int ntotal, int D, int K,
+cudaError_t launch_particles(const InstDesc* insts, const PartRef* refs, int ntotal, int ninst, int D, int K,
                              int lpar, const Shape& sh, GridBar* gb, bool fused, cudaStream_t st,
                              long long wait_ns) {
     const int blocks = (ntotal + PB - 1) / PB;
     const unsigned long long lim = wait_ns < 0 ? PWAIT_NS : (unsigned long long)wait_ns;
     if (fused || K == 1) {
-        k_particles<<<blocks, 256, 0, st>>>(insts, refs, ntotal, D, K, 1, K, lpar, sh, gb, lim);
+        k_particles<<<blocks, 256, 0, st>>>(insts, refs, ninst, D, K, 1, K, lpar, sh, gb, lim);
         return cudaGetLastError();
     }
     for (int ph = 1; ph <= K; ++ph)
-        k_particles<<<blocks, 256, 0, st>>>(insts, refs, ntotal, D, K, ph, ph, lpar, sh, gb, lim);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_box_sums(const InstDesc* insts, const PartRef* refs, int ntotal, int D, cudaStream_t st) {
-    k_box_sums<<<ntotal, BS_THREADS, 0, st>>>(insts, refs, D);
+        k_particles<<<blocks, 256, 0, st>>>(insts, refs, ninst, D, K, ph, ph, lpar, sh, gb, lim);
     return cudaGetLastError();
 }
 
