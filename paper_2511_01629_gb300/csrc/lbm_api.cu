@@ -43,7 +43,7 @@ int fluid_direct_blocks_per_sm(int fp16, const Shape& sh);
 cudaError_t launch_fluid_direct(int fp16, const InstDesc* insts, const uint16_t* tile_inst, int ntiles, int par,
                                 const Shape& sh, int commit, cudaStream_t st);
 cudaError_t launch_adj_fluid(int Q, int fp16, const InstDesc* insts, const AdjFluid* afs,
-                             const uint16_t* tile_inst, int ntiles, int lam_mode, const Shape& sh,
+                             const uint16_t* tile_inst, int ninst, int ntiles, int lam_mode, const Shape& sh,
                              cudaStream_t st);
 cudaError_t launch_adj_particles(int D, const InstDesc* insts, const AdjPart* steps, const AdjBufs* bufs,
                                  int ninst, cudaStream_t st);
@@ -1394,11 +1394,10 @@ namespace {
 
 // Adjoint particle arrays of one instance inside one allocation.
 size_t adj_pbuf_doubles(int np, int K) {
-    const size_t n3 = 3 * (size_t)std::max(np, 1);
-    return 5 * n3 + (size_t)std::max(np, 1) + 1 + 4 * (size_t)std::max(np, 1) + 4 * (size_t)std::max(np, 1) +
-           n3 + (size_t)(K + 1) * n3 + 3 * (size_t)K * n3 + 5 * n3 + 8;
+    const size_t n1 = (size_t)std::max(np, 1), n3 = 3 * n1;
+    return 5 * n3 + n1 + 1 + 4 * n1 + 4 * n1 + adj_scratch((int)n1, K) + 8;
 }
-AdjBufs adj_bufs_layout(void* base, int np, int K) {
+AdjBufs adj_bufs_layout(void* base, int np) {
     double* q = static_cast<double*>(base);
     const size_t n1 = (size_t)std::max(np, 1), n3 = 3 * n1;
     AdjBufs b;
@@ -1411,16 +1410,7 @@ AdjBufs adj_bufs_layout(void* base, int np, int K) {
     b.alpha_b = q; q += 1;
     b.Abar = q; q += 4 * n1;
     b.coef = reinterpret_cast<float*>(q); q += 4 * n1;
-    b.Ubar = q; q += n3;
-    b.Xk = q; q += (size_t)(K + 1) * n3;
-    b.Xs = q; q += (size_t)K * n3;
-    b.F1 = q; q += (size_t)K * n3;
-    b.F2 = q; q += (size_t)K * n3;
-    b.Xkb = q; q += n3;
-    b.Xsb = q; q += n3;
-    b.v = q; q += n3;
-    b.Ubb = q; q += n3;
-    b.Wnb = q; q += n3;
+    b.scratch = q;
     return b;
 }
 
@@ -1529,7 +1519,7 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
     std::vector<long long> field_off(ni);
     for (int i = 0; i < ni; ++i) {
         Instance& I = ctx->inst[i];
-        ab[i] = adj_bufs_layout(A.ai[i].pbuf.ptr, I.np, K);
+        ab[i] = adj_bufs_layout(A.ai[i].pbuf.ptr, I.np);
         out_off[i] = nout;
         nout += 1 + 16LL * I.np;
         field_off[i] = foff;
@@ -1545,7 +1535,7 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
             f.fin = a.slot[kk].ptr;
             f.prec = P<PRec>(a.rprec) + n1 * kk;
             f.lcnt = P<int>(a.rlcnt) + (size_t)I.ntiles * kk;
-            f.lent = P<uint32_t>(a.rlent) + (size_t)I.ntiles * LIST_CAP * kk;
+            f.lrec = P<char>(a.rlrec) + (size_t)CAND_BYTES * I.ntiles * LIST_CAP * kk;
             f.lam_src = k == L ? (seed_field ? seed_field + field_off[i] : nullptr) : P<float>(a.fbar[(kk + 1) & 1]);
             f.lam_dst = P<float>(a.fbar[kk & 1]);
             f.coef = ab[i].coef;
@@ -1607,7 +1597,7 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
             const bool final_step = last && k == len - 1;
             const int mode = final_step ? (seed_field ? 1 : 2) : 0;
             CK(launch_adj_fluid(ctx->Q, ctx->fp16, dI, P<AdjFluid>(A.d_afl) + (size_t)(final_step ? L : k) * ni,
-                                P<uint16_t>(ctx->d_tile_inst), ctx->ntiles, mode, sh, st));
+                                P<uint16_t>(ctx->d_tile_inst), ni, ctx->ntiles, mode, sh, st));
         }
         return LBM_OK;
     };

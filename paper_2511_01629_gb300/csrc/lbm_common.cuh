@@ -1142,4 +1142,51 @@ __device__ __forceinline__ void pull_pre_all(const InstDesc& in, const S* __rest
     }
 }
 
+template <class S> __device__ __forceinline__ float load_one(const S* p, float s) {
+    return VecIO<S, 1 + (sizeof(S) == 2)>::load1(p, s);
+}
+__device__ __forceinline__ float2 load_pair(const float* p, float) { return __ldg(reinterpret_cast<const float2*>(p)); }
+__device__ __forceinline__ float2 load_pair(const __half* p, float s) {
+    const unsigned int t = __ldg(reinterpret_cast<const unsigned int*>(p));
+    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&t));
+    return make_float2(a.x * s, a.y * s);
+}
+
+// Populations of nodes x, x + 1 (x even) of a row whose y and z sources lie
+// inside the box; EDGE: the warp's nodes include x = 0 or reach x = nx - 1, so
+// the shifted loads of those nodes come from across the x face (bounce-back at
+// a wall, plus its term; the far column on a periodic axis).  Lanes past nx
+// read valid nodes, and their values are not stored.
+template <int Q, class S, bool EDGE>
+__device__ __forceinline__ void pull_pair(const InstDesc& in, const S* __restrict__ fin, int x, int y, int z, float2* f) {
+    using L = Lat<Q>;
+    const int nx = in.n[0], pitch = in.pitch, zs = in.n[1] * pitch, qs = (int)in.qstride;
+    const float sl = in.s_load;
+    const int own = z * zs + y * pitch;
+    const bool wall = !in.periodic[0];
+#pragma unroll
+    for (int q = 1; q < Q; ++q) {
+        const int cx = L::c(q, 0);
+        const int row = (q - 1) * qs + own - L::c(q, 2) * zs - L::c(q, 1) * pitch;
+        if (cx == 0) {
+            f[q - 1] = load_pair(fin + (row + (EDGE && x >= nx ? 0 : x)), sl);
+        } else if constexpr (!EDGE) {
+            f[q - 1] = make_float2(load_one(fin + (row + x - cx), sl), load_one(fin + (row + x + 1 - cx), sl));
+        } else {
+            float v[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int xe = min(x + e, nx - 1), xs = xe - cx;
+                const bool out = cx > 0 ? xs < 0 : xs >= nx;
+                const int face = cx > 0 ? 0 : 1;
+                const int off = !out ? row + xs : wall ? (L::opp(q) - 1) * qs + own + xe : row + (cx > 0 ? nx - 1 : 0);
+                const float term = __ldg(&in.wterm[0][face][q]);  // always: no load waits on a condition
+                const float w = load_one(fin + off, sl);
+                v[e] = out && wall ? w + term : w;
+            }
+            f[q - 1] = make_float2(v[0], v[1]);
+        }
+    }
+}
+
 }  // namespace lbmpen

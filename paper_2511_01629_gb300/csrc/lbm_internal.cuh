@@ -247,7 +247,7 @@ struct AdjFluid {
     const void* fin;         // populations entering step n (storage type, population layout)
     const PRec* prec;        // particle records of step n
     const int* lcnt;         // tile lists of step n
-    const uint32_t* lent;
+    const void* lrec;        // their candidate records (Cand)
     const float* lam_src;    // adjoint of the pre-collision populations of step n + 1
                              //   (population layout, FP32), or the field seed ([Q][N])
     float* lam_dst;          // adjoint of the pre-collision populations of step n
@@ -271,17 +271,11 @@ struct AdjBufs {
     double* alpha_b;         // [1]     d J / d alpha
     double* Abar;            // [np][4] (see AdjFluid)
     float* coef;             // [np][8]
-    double* Ubar;            // [np][3] scratch: (U^n + U^{n-1}) / 2
-    double* Xk;              // [K+1][np][3] sub-step positions
-    double* Xs;              // [K][np][3] predicted positions
-    double* F1;              // [K][np][3] collision force at Xk (C = 1: per unit C)
-    double* F2;              // [K][np][3] ... at Xs
-    double* Xkb;             // [np][3] adjoint of the current sub-step position
-    double* Xsb;             // [np][3]
-    double* v;               // [np][3] adjoint of the sub-step force sum
-    double* Ubb;             // [np][3] adjoint of Ubar
-    double* Wnb;             // [np][3] adjoint of W^n
+    double* scratch;         // adj_scratch(np, K) doubles of the particle sweep
 };
+// Doubles of the particle sweep's scratch: positions, predicted positions and
+// forces of K sub-steps, and six arrays of [np][3].
+__host__ __device__ inline size_t adj_scratch(int np, int K) { return 3 * (size_t)np * (3 * (size_t)K + 7); }
 
 // Particle index -> (instance, local index) for the per-particle kernels.
 struct PartRef {
