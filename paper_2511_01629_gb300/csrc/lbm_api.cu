@@ -39,9 +39,9 @@ cudaError_t launch_fluid_tma(int Q, int fp16, const InstDesc* insts, const void*
                              const uint16_t* tile_inst, int ntiles, int par, const Shape& sh,
                              int commit, int grid, int* tile_ctr, int stages, int ninst, cudaStream_t st);
 int direct_tile_width();
-int fluid_direct_blocks_per_sm(int fp16, const Shape& sh);
-cudaError_t launch_fluid_direct(int fp16, const InstDesc* insts, const uint16_t* tile_inst, int ntiles, int par,
-                                const Shape& sh, int commit, cudaStream_t st);
+int fluid_direct_blocks_per_sm(int Q, int fp16, const Shape& sh);
+cudaError_t launch_fluid_direct(int Q, int fp16, const InstDesc* insts, const uint16_t* tile_inst, int ninst, int ntiles,
+                                int par, const Shape& sh, int commit, cudaStream_t st);
 cudaError_t launch_adj_fluid(int Q, int fp16, const InstDesc* insts, const AdjFluid* afs,
                              const uint16_t* tile_inst, int ninst, int ntiles, int lam_mode, const Shape& sh,
                              cudaStream_t st);
@@ -476,11 +476,14 @@ int build_tmaps(lbm_ctx* ctx) {
     return LBM_OK;
 }
 
+// Whether a shape's fluid kernel stages tiles through shared memory (D2Q9).
+bool staged(const Shape& sh) { return sh.tma && sh.stages > 0; }
+
 // Tile grid, tile -> instance table and tile lists for a shape.
 int configure_shape(lbm_ctx* ctx, const Shape& sh_in) {
     Shape sh = sh_in;
     if (ctx->D == 2) sh.tz = 1;
-    sh.tw = !sh.tma ? 32 * sh.vec : ctx->D == 2 ? tma_tile_width(ctx->Q) : direct_tile_width();
+    sh.tw = !sh.tma ? 32 * sh.vec : staged(sh) ? tma_tile_width(ctx->Q) : direct_tile_width();
     ctx->shape = sh;
     const int T[3] = {sh.tw, sh.ty, sh.tz};
     int tile0 = 0;
@@ -511,35 +514,41 @@ int configure_shape(lbm_ctx* ctx, const Shape& sh_in) {
                        cudaMemcpyHostToDevice, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));
     const int occ = !sh.tma ? fluid_max_blocks_per_sm(ctx->Q, ctx->fp16, sh)
-                    : ctx->D == 2 ? fluid_tma_blocks_per_sm(ctx->Q, ctx->fp16, sh, sh.stages, (int)ctx->inst.size())
-                                  : fluid_direct_blocks_per_sm(ctx->fp16, sh);
+                    : staged(sh) ? fluid_tma_blocks_per_sm(ctx->Q, ctx->fp16, sh, sh.stages, (int)ctx->inst.size())
+                                 : fluid_direct_blocks_per_sm(ctx->Q, ctx->fp16, sh);
     if (occ < 1) return set_err(ctx, LBM_ERR_INVALID, "kernel shape does not fit on an SM%s");
     ctx->grid = occ * ctx->num_sms;
-    if (sh.tma && ctx->D == 2 && (rc = build_tmaps(ctx))) return rc;
+    if (staged(sh) && (rc = build_tmaps(ctx))) return rc;
     if ((rc = upload_descs(ctx))) return rc;
     invalidate_graphs(ctx);
     return republish(ctx);
 }
 
-Shape default_shape(int Q, int fp16) {
-    // TMA-staged pipeline, 2 stages: D2Q9 FP32 8 rows and 8 consumer warps
-    // (one box of all populations per tile, two blocks per SM); D2Q9 FP16 4
+Shape default_shape(int Q, int fp16, long long nodes) {
+    // Small D2Q9 grids: straight into registers, one block of 4 rows per 64-node
+    // tile.  2^18 nodes are one wave of such blocks (8 per SM); there the staged
+    // kernel's start (tables, work counter, ring) costs more than it gives:
+    // 100x200 10.3 us per step against 12.9, 200x800 (10 disks) 13.1 against 17.0,
+    // 300x1000 (20 disks) 16.7 against 17.7; above, 400x1600 17.4 against 14.9.
+    if (Q == 9 && nodes <= (1 << 18)) return Shape{fp16 ? 8 : 4, 4, 1, 4, 1, 1, 0, 64};
+    // Larger ones: TMA-staged pipeline, 2 stages: FP32 8 rows and 8 consumer
+    // warps (one box of all populations per tile, two blocks per SM); FP16 4
     // rows and 4 warps (four blocks per SM: 16 consumer warps, as for FP32,
-    // with tiles half as tall); D3Q19 4 warps (four blocks per SM fit in
-    // shared memory, against three with 3 stages)
+    // with tiles half as tall).  D3Q19: straight into registers.
     if (Q == 9) return fp16 ? Shape{8, 4, 1, 4, 1, 1, 2, 128} : Shape{4, 8, 1, 8, 1, 1, 2, 128};
-    return Shape{fp16 ? 4 : 2, 2, 2, 4, 1, 1, 2, 64};
+    return Shape{fp16 ? 4 : 2, 2, 2, 4, 1, 1, 0, 64};
 }
 
 // The fluid kernel over the instances of descriptor array insts (tensor maps
 // tmaps, D2Q9 staged path only), reading buffer par.
 int enqueue_fluid_on(lbm_ctx* ctx, const InstDesc* insts, const void* tmaps, int par, int commit, cudaStream_t st) {
     const Shape& sh = ctx->shape;
-    if (sh.tma && ctx->D == 2)
+    if (staged(sh))
         CK(launch_fluid_tma(ctx->Q, ctx->fp16, insts, tmaps, P<uint16_t>(ctx->d_tile_inst), ctx->ntiles, par, sh, commit,
                             ctx->grid, P<int>(ctx->d_tile_ctr), sh.stages, (int)ctx->inst.size(), st));
     else if (sh.tma)
-        CK(launch_fluid_direct(ctx->fp16, insts, P<uint16_t>(ctx->d_tile_inst), ctx->ntiles, par, sh, commit, st));
+        CK(launch_fluid_direct(ctx->Q, ctx->fp16, insts, P<uint16_t>(ctx->d_tile_inst), (int)ctx->inst.size(), ctx->ntiles,
+                               par, sh, commit, st));
     else
         CK(launch_fluid(ctx->Q, ctx->fp16, insts, P<uint16_t>(ctx->d_tile_inst), ctx->ntiles, par, sh, commit,
                         sh.persistent, ctx->grid, P<int>(ctx->d_tile_ctr), st));
@@ -728,7 +737,9 @@ int lbm_create_batch(const lbm_config* cfgs, int n, const lbm_allocator* alloc, 
         return LBM_ERR_CUDA;
     }
     ctx->inst.resize(n);
-    ctx->shape = default_shape(ctx->Q, ctx->fp16);
+    long long nodes = 0;
+    for (int i = 0; i < n; ++i) nodes += (long long)cfgs[i].n[0] * cfgs[i].n[1] * (ctx->D == 3 ? cfgs[i].n[2] : 1);
+    ctx->shape = default_shape(ctx->Q, ctx->fp16, nodes);
     const size_t ssz = ctx->fp16 ? 2 : 4;
     int rc = LBM_OK;
     for (int i = 0; i < n && rc == LBM_OK; ++i) {
@@ -1233,6 +1244,7 @@ int lbm_set_kernel_shape(lbm_ctx* ctx, int vec, int tile_rows, int warps) {
     s.tma = vec == 0;
     if (vec) s.vec = vec;
     s.warps = warps;
+    if (s.tma && ctx->D == 2 && s.stages == 0) s.stages = 2;
     if (s.tma && !tma_rows_ok(tile_rows))
         return set_err(ctx, LBM_ERR_INVALID, "TMA tiles hold 4 or 8 rows%s");
     if (ctx->D == 2) {
@@ -1269,7 +1281,8 @@ int lbm_autotune(lbm_ctx* ctx, int reps) {
                 }
     for (int rows : {4, 8})
         for (int warps : {4, 8})
-            for (int stages : {2, 3, 4}) {
+            for (int stages : {0, 2, 3, 4}) {  // 0: straight into registers (the only form in 3D)
+                if (ctx->D == 3 && stages > 0) continue;
                 Shape s{ctx->shape.vec, rows, 1, warps, 1, 1, stages, 0};
                 if (ctx->D == 3) {
                     s.tz = rows >= 4 ? 2 : 1;
@@ -1456,7 +1469,7 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
     // k + 1, its records go to record k (and k + 1 for the next step's input);
     // entry L is the publish of a segment's first state into record 0
     std::vector<InstDesc> rd((size_t)(L + 1) * ni);
-    const bool tma = sh.tma && ctx->D == 2;  // the fluid kernel reads through tensor maps
+    const bool tma = staged(sh);  // the fluid kernel reads through tensor maps
     std::vector<CUtensorMap> tm(tma ? (size_t)L * ni * 2 : 0);
     for (int k = 0; k <= L; ++k)
         for (int i = 0; i < ni; ++i) {

@@ -1,5 +1,5 @@
-// Fused stream-collide-penalize kernel for D3Q19: loads straight into
-// registers, one warp per 64-node row of a tile.
+// Fused stream-collide-penalize kernel that loads straight into registers, one
+// warp per 64-node row of a tile: D3Q19, and D2Q9 on small grids.
 //
 // Pull streaming reads every population value once, so staging a D3Q19 tile
 // through shared memory saves no traffic, and its tensor copies are small (18
@@ -8,11 +8,13 @@
 // lane takes two adjacent nodes: populations with c_x = 0 arrive by one
 // 8-byte (FP16: 4-byte) load, the others by two scalar loads of the shifted
 // pair; all 18 are in flight before the first is used, and enough warps are
-// resident to cover the latency.  Rows at a y or z face take pull_pre_all;
-// the x faces only change the address of an edge node's load.
-// 256 x 256 x 512, 8 spheres, the kernel alone: FP32 1.28 -> 0.905 ms (5.3 TB/s),
-// FP16 storage 1.28 -> 0.78 ms; 128 threads of 4 rows each against 8 rows per
-// 4 warps: 0.83 ms.
+// resident to cover the latency: 80 registers, 24 warps per SM (some 200 bytes of
+// spills, in the solid path) beat 128 registers and 16 warps (256 x 256 x 512, 8
+// spheres, per step: FP32 934 -> 812 us, 5.95 TB/s; FP16 151 x 133 x 203
+// 157 -> 135 us; 72 registers: 879 and 136).  Rows at a y or z face take
+// pull_pre_all; the x faces only change the address of an edge node's load.
+// On a small D2Q9 grid the kernel is bound by its chain of latencies, which is
+// shorter here than the staged kernel's (default_shape has the figures).
 #include "lbm_common.cuh"
 
 namespace lbmpen {
@@ -34,15 +36,15 @@ struct DescEnv {
 }  // namespace
 
 template <int Q, class S>
-__global__ void __launch_bounds__(256, 2) k_fluid_direct(const InstDesc* __restrict__ insts,
-                                                         const uint16_t* __restrict__ tile_inst, int par, Shape sh,
+__global__ void __launch_bounds__(256, Q == 9 ? 4 : 3) k_fluid_direct(const InstDesc* __restrict__ insts,
+                                                         const uint16_t* __restrict__ tile_inst, int ninst, int par, Shape sh,
                                                          int commit) {
     using L = Lat<Q>;
     constexpr int D = L::D;
     constexpr int QS = Q - 1;
     __shared__ Cand cand[LIST_CAP];
     const int t = blockIdx.x;
-    const InstDesc& in = insts[tile_inst[t]];
+    const InstDesc& in = insts[ninst > 1 ? (int)tile_inst[t] : 0];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int local = t - in.tile0;
     const int ntx = in.ntile[0], nty = in.ntile[1];
@@ -55,6 +57,8 @@ __global__ void __launch_bounds__(256, 2) k_fluid_direct(const InstDesc* __restr
     const float sload = in.s_load;
     const S* __restrict__ fin = static_cast<const S*>(in.f[par]);
     float2 f[QS];
+    dep_launch();
+    dep_wait();  // the populations and lists of the previous step
     auto pull_row = [&](int r) {  // false: the row lies beyond the box
         const int y = y0 + (r & (sh.ty - 1)), z = z0 + (r >> lty);
         if (r >= rows || y >= ny || z >= nz) return false;
@@ -104,18 +108,31 @@ __global__ void __launch_bounds__(256, 2) k_fluid_direct(const InstDesc* __restr
 
 int direct_tile_width() { return TW; }
 
-int fluid_direct_blocks_per_sm(int fp16, const Shape& sh) {
+template <int Q, class S>
+static int direct_blocks_t(const Shape& sh) {
     int nb = 0;
-    if (fp16) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_fluid_direct<19, __half>, 32 * sh.warps, 0);
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_fluid_direct<19, float>, 32 * sh.warps, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_fluid_direct<Q, S>, 32 * sh.warps, 0);
     return nb;
 }
+int fluid_direct_blocks_per_sm(int Q, int fp16, const Shape& sh) {
+    if (Q == 9) return fp16 ? direct_blocks_t<9, __half>(sh) : direct_blocks_t<9, float>(sh);
+    return fp16 ? direct_blocks_t<19, __half>(sh) : direct_blocks_t<19, float>(sh);
+}
 
-cudaError_t launch_fluid_direct(int fp16, const InstDesc* insts, const uint16_t* tile_inst, int ntiles, int par,
-                                const Shape& sh, int commit, cudaStream_t st) {
-    if (fp16) k_fluid_direct<19, __half><<<ntiles, 32 * sh.warps, 0, st>>>(insts, tile_inst, par, sh, commit);
-    else k_fluid_direct<19, float><<<ntiles, 32 * sh.warps, 0, st>>>(insts, tile_inst, par, sh, commit);
-    return cudaGetLastError();
+cudaError_t launch_fluid_direct(int Q, int fp16, const InstDesc* insts, const uint16_t* tile_inst, int ninst, int ntiles,
+                                int par, const Shape& sh, int commit, cudaStream_t st) {
+    cudaError_t e = cudaSuccess;
+    auto go = [&](auto kern) {
+        e = launch_dep(kern, dim3((unsigned)ntiles), 32 * sh.warps, 0, st, insts, tile_inst, ninst, par, sh, commit);
+    };
+    if (Q == 9) {
+        if (fp16) go(k_fluid_direct<9, __half>);
+        else go(k_fluid_direct<9, float>);
+    } else {
+        if (fp16) go(k_fluid_direct<19, __half>);
+        else go(k_fluid_direct<19, float>);
+    }
+    return e;
 }
 
 }  // namespace lbmpen

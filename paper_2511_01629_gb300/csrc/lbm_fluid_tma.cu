@@ -299,6 +299,8 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
     }
     for (int i = threadIdx.x; i < ntab; i += blockDim.x) make_tinst<Q>(tab[i], insts[i]);
     __syncthreads();
+    dep_launch();
+    dep_wait();  // the populations, lists and work counter of the previous step
 
     if (warp == 0) {
         // ---------------------------------------------------------- producer
@@ -644,10 +646,8 @@ static cudaError_t launch_tma_t(const InstDesc* insts, const void* tmaps, const 
                                 int ntiles, int par, const Shape& sh, int commit, int grid,
                                 int* tile_ctr, int stages, int ninst, cudaStream_t st) {
     const TmaLayout LY = tma_layout(Q, (int)sizeof(S), TW, ROWS, stages, ninst);
-    k_fluid_tma<Q, S, TW, ROWS><<<grid, 32 * (sh.warps + 1), LY.bytes, st>>>(
-        insts, static_cast<const CUtensorMap*>(tmaps), tile_inst, ntiles, par, sh, commit, tile_ctr,
-        stages, ninst);
-    return cudaGetLastError();
+    return launch_dep(k_fluid_tma<Q, S, TW, ROWS>, dim3((unsigned)grid), 32 * (sh.warps + 1), LY.bytes, st, insts,
+                      static_cast<const CUtensorMap*>(tmaps), tile_inst, ntiles, par, sh, commit, tile_ctr, stages, ninst);
 }
 
 int tma_tile_width(int Q) { return Q == 9 ? 128 : 64; }

@@ -285,4 +285,29 @@ struct PartRef {
 
 __host__ __device__ inline int tile_w(const Shape& s) { return s.tw; }
 
+// Programmatic dependent launch of the kernels of a step: the next kernel's
+// blocks may start while the previous kernel runs, and wait (dep_wait) before
+// they touch anything it writes; what comes before the wait reads only
+// what no kernel of a step writes (descriptors, constants).  dep_launch lets the
+// next kernel start.  Saves the launch gap and the prologue: 1.1 to 1.5 us a step
+// in graph replay (channel 100 x 200 14.6 -> 13.1 us, 500 disks FP32 62.6 -> 61.4).
+#ifdef __CUDACC__
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <class... P, class... A>
+inline cudaError_t launch_dep(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+#endif
+
 }  // namespace lbmpen

@@ -713,6 +713,8 @@ __global__ void __launch_bounds__(256, 1) k_particles(const InstDesc* __restrict
     PartRef r0{0, (int)blockIdx.x * PB};
     if (ninst > 1) r0 = refs[blockIdx.x * PB];
     stage_desc(&sdesc, insts[r0.inst]);
+    dep_wait();  // the totals of this step
+    dep_launch();
     const InstDesc& in = sdesc;
     const int par = lpar ^ 1, i0 = r0.p;
     for (int ph = first; ph <= last; ++ph) {
@@ -754,8 +756,7 @@ cudaError_t launch_particles(const InstDesc* insts, const PartRef* refs, int nto
     const int blocks = (ntotal + PB - 1) / PB;
     const unsigned long long lim = wait_ns < 0 ? PWAIT_NS : (unsigned long long)wait_ns;
     if (fused || K == 1) {
-        k_particles<<<blocks, 256, 0, st>>>(insts, refs, ninst, D, K, 1, K, lpar, sh, gb, lim);
-        return cudaGetLastError();
+        return launch_dep(k_particles, dim3((unsigned)blocks), 256, 0, st, insts, refs, ninst, D, K, 1, K, lpar, sh, gb, lim);
     }
     for (int ph = 1; ph <= K; ++ph)
         k_particles<<<blocks, 256, 0, st>>>(insts, refs, ninst, D, K, ph, ph, lpar, sh, gb, lim);
