@@ -57,8 +57,8 @@ __global__ void __launch_bounds__(256, Q == 9 ? 4 : 3) k_fluid_direct(const Inst
     const float sload = in.s_load;
     const S* __restrict__ fin = static_cast<const S*>(in.f[par]);
     float2 f[QS];
-    dep_launch();
     dep_wait();  // the populations and lists of the previous step
+    dep_launch();
     auto pull_row = [&](int r) {  // false: the row lies beyond the box
         const int y = y0 + (r & (sh.ty - 1)), z = z0 + (r >> lty);
         if (r >= rows || y >= ny || z >= nz) return false;

@@ -299,8 +299,8 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
     }
     for (int i = threadIdx.x; i < ntab; i += blockDim.x) make_tinst<Q>(tab[i], insts[i]);
     __syncthreads();
-    dep_launch();
     dep_wait();  // the populations, lists and work counter of the previous step
+    dep_launch();
 
     if (warp == 0) {
         // ---------------------------------------------------------- producer

@@ -62,29 +62,53 @@ __device__ __forceinline__ void pair_operands(const InstDesc& in, int j, int src
 // Pair part of Eq. 21 on particle i at two position sets: X^{k} (F1) and
 // X^{k} + h Ubar (F2).  The block's particles all belong to one instance;
 // its positions are staged in shared memory in chunks and the lanes split
-// them.  An FP32 filter leaves only pairs near the interaction range for the
-// FP64 evaluation, which follows the reference operation order.  The
-// predicted positions of the filter: staged (xs2) after the first sub-step; in the
-// first one taken from the totals, in FP32, for the few pairs within 2 of
-// range (a predicted position lies within |h Ubar| < sqrt(3)/2 of X^n, a larger
-// step is reported as ST_DISPLACEMENT).
-template <bool FIRST>
-__device__ void pair_chunk(const InstDesc& in, int i, int src, int par, double h, int D, int lane, const float4* xs,
-                           const float4* xs2, int j0, int nj, float4 xi, float4 xi2, double cp,
-                           double inv_delta, double* f1, double* f2) {
-    if (cp == 0.0) return;  // cp = C / eps_p of particle i
-    const float reach = xi.w + (float)in.delta + 0.01f;  // FP32 positions carry < 1e-3 error
-    const float nf[3] = {(float)in.n[0], (float)in.n[1], (float)in.n[2]};
-    const bool per[3] = {in.periodic[0] && in.n[0] > 1, in.periodic[1] && in.n[1] > 1,
-                         in.periodic[2] && in.n[2] > 1};
-    auto dist2 = [&](float4 a, float4 b) {
+// them: bit k of a lane's mask stands for particle j0 + lane + 32 k.  An FP32
+// filter (pair_mask) leaves the pairs within 2 of range at X^{k} (a predicted
+// position lies within |h Ubar| < sqrt(3)/2 of it, a larger step is reported
+// as ST_DISPLACEMENT); pair_forces evaluates in FP64, in the reference operation
+// order, those near the range at X^{k} or at the predicted positions.
+static_assert(XCHUNK <= 32 * 32, "a lane's pairs of a chunk fit a mask");
+struct PairGeo {
+    float n[3];
+    bool per[3];
+    __device__ __forceinline__ explicit PairGeo(const InstDesc& in) {
+        for (int d = 0; d < 3; ++d) {
+            n[d] = (float)in.n[d];
+            per[d] = in.periodic[d] && in.n[d] > 1;
+        }
+    }
+    __device__ __forceinline__ float dist2(float4 a, float4 b) const {
         float dv[3] = {a.x - b.x, a.y - b.y, a.z - b.z};
 #pragma unroll
         for (int d = 0; d < 3; ++d)
-            if (per[d]) dv[d] -= nf[d] * rintf(dv[d] / nf[d]);
+            if (per[d]) dv[d] -= n[d] * rintf(dv[d] / n[d]);
         return dv[0] * dv[0] + dv[1] * dv[1] + dv[2] * dv[2];
-    };
-    // X + h Ubar of a particle in FP32, from its totals (sums below 2^62: exact to FP32's last bit)
+    }
+};
+__device__ __forceinline__ float pair_reach(const InstDesc& in, float4 xi) {
+    return xi.w + (float)in.delta + 0.01f;  // FP32 positions carry < 1e-3 error
+}
+
+__device__ __forceinline__ unsigned pair_mask(const InstDesc& in, int i, int lane, const float4* xs, int j0, int nj, float4 xi) {
+    const PairGeo g(in);
+    const float reach = pair_reach(in, xi) + 2.0f;
+    unsigned m = 0;
+    for (int jj = lane, k = 0; jj < nj; jj += 32, ++k) {
+        const float4 b = xs[jj];
+        const float lim = reach + b.w;
+        if (j0 + jj != i && g.dist2(xi, b) <= lim * lim) m |= 1u << k;
+    }
+    return m;
+}
+
+template <bool FIRST>
+__device__ __noinline__ void pair_forces(const InstDesc& in, int i, int src, int par, double h, int D, int lane, const float4* xs,
+                            const float4* xs2, int j0, unsigned m, float4 xi, float4 xi2, double cp, double inv_delta,
+                            double* f1, double* f2) {
+    if (cp == 0.0) return;  // cp = C / eps_p of particle i
+    const PairGeo g(in);
+    const float reach = pair_reach(in, xi);
+    // X + h Ubar of a particle in FP32, from its totals (before the first sub-step)
     auto predicted = [&](int j, float4 x) {
         const long long* v = in.tot[par] + (long long)NPV * j;
         const float s = v[0] > 0 ? 9.094947017729282e-13f / (float)v[0] : 0.f;  // 2^-40 / count
@@ -95,14 +119,12 @@ __device__ void pair_chunk(const InstDesc& in, int i, int src, int par, double h
         if (D == 3) x.z += hh * ((float)v[12] * s + (float)ps.U[2]);
         return x;
     };
-    for (int jj = lane; jj < nj; jj += 32) {
-        const int j = j0 + jj;
-        if (j == i) continue;
+    for (; m; m &= m - 1) {
+        const int jj = lane + 32 * (__ffs(m) - 1), j = j0 + jj;
         const float4 b = xs[jj];
         const float lim = reach + b.w;
-        const float d2 = dist2(xi, b);
-        if (d2 > (lim + 2.0f) * (lim + 2.0f)) continue;  // out of range at both position sets
-        const float e2 = FIRST ? dist2(predicted(i, xi), predicted(j, b)) : dist2(xi2, xs2[jj]);
+        const float d2 = g.dist2(xi, b);
+        const float e2 = FIRST ? g.dist2(predicted(i, xi), predicted(j, b)) : g.dist2(xi2, xs2[jj]);
         const bool near[2] = {d2 <= lim * lim, e2 <= lim * lim};
         if (!near[0] && !near[1]) continue;
         const double Bi = in.pconst[PCONST_N * i + PC_B], Bj = in.pconst[PCONST_N * j + PC_B];
@@ -118,7 +140,7 @@ __device__ void pair_chunk(const InstDesc& in, int i, int src, int par, double h
                 const double xi_d = Xi[d] + sh * Ui[d];
                 const double xj_d = Xj[d] + sh * Uj[d];
                 dd[d] = xi_d - xj_d;
-                if (per[d]) {
+                if (g.per[d]) {
                     const double half = 0.5 * in.n[d];
                     if (dd[d] > half) dd[d] -= in.n[d];
                     else if (dd[d] < -half) dd[d] += in.n[d];
@@ -378,16 +400,15 @@ __device__ void append_tiles(const InstDesc& in, int p, const AxisTiles* at, Can
 // sub-step A^{n+1}, theta^{n+1}, U^{n-1} <- U^n and the record for the next
 // step.  Each lane evaluates the expressions of a serial loop over d.
 // The operands of update_lane, loaded in one batch before the pair search so
-// that their latency overlaps it; on the first sub-step the projection's
-// translation (Eq. 22) is part of it.
+// that their latency overlaps it (on the first sub-step before the fluid kernel
+// has ended; project_lane adds what its totals give).
 struct LaneIn {
     double X0, Ub, Un, invrhos, cw, idl, Ri, Bi, gfac, invc, Acor, ec, es;
     int cnt;
     RecConst rc;
 };
 
-__device__ __forceinline__ LaneIn load_lane(const InstDesc& in, int i, int d, bool valid, int src, int par, double h,
-                                            int first, int D) {
+__device__ __forceinline__ LaneIn load_lane(const InstDesc& in, int i, int d, bool valid, int src, int par, int first) {
     if (!valid) {  // in-range operands for the shuffle-only lanes
         i = 0;
         d = 0;
@@ -406,30 +427,9 @@ __device__ __forceinline__ LaneIn load_lane(const InstDesc& in, int i, int d, bo
     L.es = ps.es;
     L.rc = in.rconst[i];
     if (first) {
-        const long long* v = in.tot[par] + (long long)NPV * i;
-        const long long n = v[0], su = v[10 + d];
-        const double Uold = ps.U[d];
         L.X0 = ps.X[d];
+        L.Ub = ps.U[d];  // U^{n-1} until project_lane
         L.Acor = 0.0;
-        L.cnt = (int)n;
-        L.invc = 0.0;
-        L.Un = Uold;
-        L.Ub = 0.0;
-        if (n != 0) {
-            L.invc = rcp64((double)n);
-            L.Un = d < D ? finalize_u(su, L.invc) : 0.0;
-            L.Ub = d < D ? 0.5 * (L.Un + Uold) : 0.0;
-        }
-        if (valid) {
-            in.Un[j] = L.Un;
-            if (n == 0 && d == 0) atomicOr(in.status, ST_PARTICLE);
-            if (!(fabs(L.Ub) < 0.5)) atomicOr(in.status, ST_DISPLACEMENT);
-            if (d == 0) in.count[i] = (int)n;
-            if (in.K > 1) {  // the later sub-steps read these
-                in.Ubar[j] = L.Ub;
-                if (d == 0) in.invc[i] = L.invc;
-            }
-        }
     } else {
         L.X0 = in.Xk[(long long)src * in.np * 3 + j];
         L.Ub = in.Ubar[j];
@@ -441,12 +441,44 @@ __device__ __forceinline__ LaneIn load_lane(const InstDesc& in, int i, int d, bo
     return L;
 }
 
+// The translation of Eq. 22 into the operands of the first sub-step, from the
+// totals of this step.
+__device__ __forceinline__ void project_lane(const InstDesc& in, int i, int d, bool valid, int par, int D, LaneIn& L) {
+    if (!valid) {
+        i = 0;
+        d = 0;
+    }
+    const long long j = 3LL * i + d;
+    const long long* v = in.tot[par] + (long long)NPV * i;
+    const long long n = v[0], su = v[10 + d];
+    const double Uold = L.Ub;
+    L.cnt = (int)n;
+    L.invc = 0.0;
+    L.Un = Uold;
+    L.Ub = 0.0;
+    if (n != 0) {
+        L.invc = rcp64((double)n);
+        L.Un = d < D ? finalize_u(su, L.invc) : 0.0;
+        L.Ub = d < D ? 0.5 * (L.Un + Uold) : 0.0;
+    }
+    if (valid) {
+        in.Un[j] = L.Un;
+        if (n == 0 && d == 0) atomicOr(in.status, ST_PARTICLE);
+        if (!(fabs(L.Ub) < 0.5)) atomicOr(in.status, ST_DISPLACEMENT);
+        if (d == 0) in.count[i] = (int)n;
+        if (in.K > 1) {  // the later sub-steps read these
+            in.Ubar[j] = L.Ub;
+            if (d == 0) in.invc[i] = L.invc;
+        }
+    }
+}
+
 // Rotation of particle i, component d: W^n (first sub-step, Eq. 22) and, on
 // the last one, theta^{n+1} (reading: trapezoid of W) with the record's
 // orientation.  Runs on its own warp beside update_lane.
-__device__ __forceinline__ void rotate_lane(const InstDesc& in, int i, int d, int par, int first, int last, int D) {
+__device__ __forceinline__ void rotate_lane(const InstDesc& in, int i, int d, int par, int first, int last, int D,
+                                            double Th, double Wo) {
     const long long j = 3LL * i + d;
-    const double Th = in.theta[j], Wo = in.W[j];
     double Wn;
     if (first) {
         double* geo = in.adj_geo ? in.adj_geo + (long long)NPV * i : nullptr;
@@ -474,7 +506,7 @@ __device__ __forceinline__ void rotate_lane(const InstDesc& in, int i, int d, in
     }
 }
 
-__device__ void update_lane(const InstDesc& in, int i, int d, int sl, bool valid, const double* F1in,
+__device__ __forceinline__ void update_lane(const InstDesc& in, int i, int d, int sl, bool valid, const double* F1in,
                             const double* F2in, int src, int par, double h, int first, int last, int D,
                             const Shape& sh, AxisTiles* at, Cand& cd, const LaneIn& L) {
     if (!valid) {  // in-range operands for the shuffle-only lanes; nothing is stored
@@ -621,8 +653,11 @@ __device__ bool grid_sync(GridBar* gb, int* status, unsigned long long limit_ns)
 // (the first from the state).  The block's warps find the pair forces (one
 // particle each); warp 0 does the FP64 update, one lane per particle component,
 // warp 1 the rotation, and warp 2 clears the totals that the next step adds to.
+// The first phase runs up to its wait beside the fluid kernel: that kernel lets
+// this one start once the previous step's particle kernel has ended, so all but
+// the totals is there (state, positions, the pairs that may be in range).
 template <bool FIRST>
-__device__ void phase_substep(const InstDesc& in, int i0, int D, int src, int par, int last, const Shape& sh,
+__device__ __forceinline__ void phase_substep(const InstDesc& in, int i0, int D, int src, int par, int last, const Shape& sh,
                               float4* xs, float4* xs2, double (*sF)[6], AxisTiles (*sAT)[3], Cand* sC) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const double h = in.hK;
@@ -632,46 +667,66 @@ __device__ void phase_substep(const InstDesc& in, int i0, int D, int src, int pa
     const int usl = lane & (PB - 1), ud = lane / PB;
     const bool uvalid = ud < 3 && i0 + usl < in.np;
     LaneIn li;
-    if (warp == 0) li = load_lane(in, i0 + usl, ud, uvalid, src, par, h, FIRST, D);
+    double th = 0.0, wo = 0.0;
+    if (warp == 0) li = load_lane(in, i0 + usl, ud, uvalid, src, par, FIRST);
+    if (warp == 1 && uvalid) {
+        th = in.theta[3 * (i0 + usl) + ud];
+        wo = in.W[3 * (i0 + usl) + ud];
+    }
     const bool pairs = in.np > 1;  // one particle: nothing to search
+    const bool one = in.np <= XCHUNK;
+    const float4* Xfb = FIRST ? in.Xp[par] : reinterpret_cast<const float4*>(in.Xf) + (long long)src * in.np;
+    const float4* Xsb = reinterpret_cast<const float4*>(in.Xsf) + (long long)src * in.np;
+    float4 xi = make_float4(0.f, 0.f, 0.f, 0.f), xi2 = xi;
+    double cp = 0.0, idl = 0.0;
+    // the positions of a chunk into shared memory, every load in flight at
+    // once, and the pairs of the warp's particle that may be in range
+    auto chunk = [&](int j0) {
+        const int nj = min(XCHUNK, in.np - j0);
+        constexpr int PER = XCHUNK / 256;  // blockDim.x == 256
+        float4 ra[PER], rb[PER];
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int k = threadIdx.x + 256 * u;
+            if (k < nj) {
+                ra[u] = Xfb[j0 + k];
+                if (!FIRST) rb[u] = Xsb[j0 + k];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int k = threadIdx.x + 256 * u;
+            if (k < nj) {
+                xs[k] = ra[u];
+                if (!FIRST) xs2[k] = rb[u];
+            }
+        }
+        __syncthreads();
+        return mine ? pair_mask(in, i, lane, xs, j0, nj, xi) : 0u;
+    };
+    unsigned m = 0;
     if (pairs) {
-        double f1[3] = {0, 0, 0}, f2[3] = {0, 0, 0};
-        const float4* Xfb = FIRST ? in.Xp[par] : reinterpret_cast<const float4*>(in.Xf) + (long long)src * in.np;
-        const float4* Xsb = reinterpret_cast<const float4*>(in.Xsf) + (long long)src * in.np;
-        float4 xi = make_float4(0.f, 0.f, 0.f, 0.f), xi2 = xi;
-        double cp = 0.0, idl = 0.0;
         if (mine) {  // issued before the staging barrier, so the loads overlap it
             xi = Xfb[i];
             if (!FIRST) xi2 = Xsb[i];
             cp = in.pconst[PCONST_N * i + PC_CPAIR];
             idl = in.pconst[PCONST_N * i + PC_INVDELTA];
         }
+        if (one) m = chunk(0);
+    }
+    if (FIRST) {
+        dep_wait();  // the totals of this step
+        dep_launch();
+        if (warp == 0) project_lane(in, i0 + usl, ud, uvalid, par, D, li);
+    }
+    if (pairs) {
+        double f1[3] = {0, 0, 0}, f2[3] = {0, 0, 0};
         for (int j0 = 0; j0 < in.np; j0 += XCHUNK) {
-            const int nj = min(XCHUNK, in.np - j0);
-            // every load of the chunk in flight at once, then the shared stores
-            constexpr int PER = XCHUNK / 256;  // blockDim.x == 256
-            float4 ra[PER], rb[PER];
-#pragma unroll
-            for (int u = 0; u < PER; ++u) {
-                const int k = threadIdx.x + 256 * u;
-                if (k < nj) {
-                    ra[u] = Xfb[j0 + k];
-                    if (!FIRST) rb[u] = Xsb[j0 + k];
-                }
-            }
-            __syncthreads();
-#pragma unroll
-            for (int u = 0; u < PER; ++u) {
-                const int k = threadIdx.x + 256 * u;
-                if (k < nj) {
-                    xs[k] = ra[u];
-                    if (!FIRST) xs2[k] = rb[u];
-                }
-            }
-            __syncthreads();
-            if (mine) pair_chunk<FIRST>(in, i, src, par, h, D, lane, xs, xs2, j0, nj, xi, xi2, cp, idl, f1, f2);
+            if (!one) m = chunk(j0);
+            if (__any_sync(0xffffffffu, m != 0)) pair_forces<FIRST>(in, i, src, par, h, D, lane, xs, xs2, j0, m, xi, xi2, cp, idl, f1, f2);
         }
-        if (mine) {
+        if (mine) {  // (no lane found a pair: the sums are zero)
             double F1[3], F2[3];
             gather_pairs(f1, f2, F1, F2);
             if (lane == 0)
@@ -686,11 +741,17 @@ __device__ void phase_substep(const InstDesc& in, int i0, int D, int src, int pa
         update_lane(in, i0 + usl, ud, usl, uvalid, pairs ? sF[usl] : nullptr, pairs ? sF[usl] + 3 : nullptr, src, par, h,
                     FIRST, last, D, sh, sAT[usl], sC[usl], li);
     } else if (warp == 1) {
-        if (uvalid) rotate_lane(in, i0 + usl, ud, par, FIRST, last, D);
+        if (uvalid) rotate_lane(in, i0 + usl, ud, par, FIRST, last, D, th, wo);
     } else if (FIRST && warp == 2) {
         for (int k = lane; k < PB * NPV; k += 32)
             if (i0 + k / NPV < in.np) in.tot[par ^ 1][(long long)NPV * i0 + k] = 0;
     }
+}
+
+// The later sub-steps (K > 1), out of line: their registers stay out of the K = 1 path.
+__device__ __noinline__ void phase_later(const InstDesc& in, int i0, int D, int src, int par, int last, const Shape& sh,
+                                         float4* xs, float4* xs2, double (*sF)[6], AxisTiles (*sAT)[3], Cand* sC) {
+    phase_substep<false>(in, i0, D, src, par, last, sh, xs, xs2, sF, sAT, sC);
 }
 
 // Particle part of one time step for the block's 8 particles (one instance),
@@ -699,9 +760,9 @@ __device__ void phase_substep(const InstDesc& in, int i0, int D, int src, int pa
 // particle to the next step's tile lists.  With more than one phase (K > 1)
 // the blocks meet at grid barriers between phases (the launch guarantees they
 // are all resident); with K = 1 there is no barrier.
+template <int D>
 __global__ void __launch_bounds__(256, 1) k_particles(const InstDesc* __restrict__ insts,
-                                                   const PartRef* __restrict__ refs, int ninst,
-                                                   int D, int K, int first, int last, int lpar,
+                                                   const PartRef* __restrict__ refs, int ninst, int K, int first, int last, int lpar,
                                                    Shape sh, GridBar* gb, unsigned long long wait_ns) {
     __shared__ double sF[PB][6];
     __shared__ AxisTiles sAT[PB][3];
@@ -713,14 +774,12 @@ __global__ void __launch_bounds__(256, 1) k_particles(const InstDesc* __restrict
     PartRef r0{0, (int)blockIdx.x * PB};
     if (ninst > 1) r0 = refs[blockIdx.x * PB];
     stage_desc(&sdesc, insts[r0.inst]);
-    dep_wait();  // the totals of this step
-    dep_launch();
     const InstDesc& in = sdesc;
     const int par = lpar ^ 1, i0 = r0.p;
     for (int ph = first; ph <= last; ++ph) {
         if (ph > first && !grid_sync(gb, in.status, wait_ns)) return;
         if (ph == 1) phase_substep<true>(in, i0, D, 0, par, K == 1, sh, xs, xs2, sF, sAT, sC);
-        else phase_substep<false>(in, i0, D, (ph - 1) & 1, par, ph == K, sh, xs, xs2, sF, sAT, sC);
+        else phase_later(in, i0, D, (ph - 1) & 1, par, ph == K, sh, xs, xs2, sF, sAT, sC);
     }
     if (last == K) {
         __syncthreads();  // records and tile ranges of the block's particles are ready
@@ -744,7 +803,7 @@ __global__ void k_publish(const InstDesc* __restrict__ insts, const PartRef* __r
 
 int particle_blocks_resident(int num_sms) {
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_particles, 256, 0) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_particles<3>, 256, 0) != cudaSuccess) return 0;
     return nb * num_sms;
 }
 
@@ -755,11 +814,11 @@ cudaError_t launch_particles(const InstDesc* insts, const PartRef* refs, int nto
                              long long wait_ns) {
     const int blocks = (ntotal + PB - 1) / PB;
     const unsigned long long lim = wait_ns < 0 ? PWAIT_NS : (unsigned long long)wait_ns;
-    if (fused || K == 1) {
-        return launch_dep(k_particles, dim3((unsigned)blocks), 256, 0, st, insts, refs, ninst, D, K, 1, K, lpar, sh, gb, lim);
-    }
+    const auto kern = D == 2 ? k_particles<2> : k_particles<3>;
+    if (fused || K == 1)
+        return launch_dep(kern, dim3((unsigned)blocks), 256, 0, st, insts, refs, ninst, K, 1, K, lpar, sh, gb, lim);
     for (int ph = 1; ph <= K; ++ph)
-        k_particles<<<blocks, 256, 0, st>>>(insts, refs, ninst, D, K, ph, ph, lpar, sh, gb, lim);
+        kern<<<blocks, 256, 0, st>>>(insts, refs, ninst, K, ph, ph, lpar, sh, gb, lim);
     return cudaGetLastError();
 }
 
