@@ -748,22 +748,30 @@ __global__ void k_adj_finish(const InstDesc* __restrict__ insts, const AdjBufs* 
     }
 }
 
-// Copy the particle state between the context arrays and a [np][16] record.
-__global__ void k_adj_state(const InstDesc* __restrict__ insts, int inst, double* rec, int to_record) {
-    const InstDesc& in = insts[inst];
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= in.np) return;
-    double* r = rec + 16LL * p;
+// The particle state of checkpoint s, every instance in one launch (a block
+// each; one launch and three copies or clears per instance before).
+__global__ void __launch_bounds__(256) k_adj_state(const InstDesc* __restrict__ insts, const AdjSeg* __restrict__ seg,
+                                                   int s, AdjStateOp op) {
+    const InstDesc& in = insts[blockIdx.x];
+    const AdjSeg g = seg[blockIdx.x];
+    const int np = in.np;
+    double* rec = g.ckst + 16LL * np * s;
     double* arr[5] = {in.X, in.U, in.W, in.theta, in.A};
-    if (to_record) {
+    for (int p = threadIdx.x; p < np; p += blockDim.x) {
+        double* r = rec + 16LL * p;
+#pragma unroll
         for (int a = 0; a < 5; ++a)
-            for (int d = 0; d < 3; ++d) r[3 * a + d] = arr[a][3 * p + d];
-        r[15] = (double)in.count[p];
-    } else {
-        for (int a = 0; a < 5; ++a)
-            for (int d = 0; d < 3; ++d) arr[a][3 * p + d] = r[3 * a + d];
-        in.count[p] = (int)r[15];
+            for (int d = 0; d < 3; ++d) {
+                if (op == ADJ_SAVE) r[3 * a + d] = arr[a][3 * p + d];
+                else arr[a][3 * p + d] = r[3 * a + d];
+            }
+        if (op == ADJ_SAVE) r[15] = (double)in.count[p];
+        else in.count[p] = (int)r[15];
     }
+    if (op != ADJ_RESTART) return;
+    for (int k = threadIdx.x; k < 16 * np; k += blockDim.x) g.rstate[k] = rec[k];
+    for (int k = threadIdx.x; k < 2 * NPV * np; k += blockDim.x) g.tot[k] = 0;
+    for (int k = threadIdx.x; k < g.ntiles; k += blockDim.x) g.rlcnt[k] = 0;
 }
 
 // ------------------------------------------------------------- launchers --
@@ -810,10 +818,8 @@ cudaError_t launch_adj_pull_out(int Q, const InstDesc* insts, int inst, long lon
     return cudaGetLastError();
 }
 
-cudaError_t launch_adj_state(const InstDesc* insts, int inst, int np, double* rec, int to_record,
-                             cudaStream_t st) {
-    if (np <= 0) return cudaSuccess;
-    k_adj_state<<<(np + 127) / 128, 128, 0, st>>>(insts, inst, rec, to_record);
+cudaError_t launch_adj_state(const InstDesc* insts, const AdjSeg* seg, int ninst, int s, AdjStateOp op, cudaStream_t st) {
+    k_adj_state<<<ninst, 256, 0, st>>>(insts, seg, s, op);
     return cudaGetLastError();
 }
 

@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -51,8 +52,7 @@ cudaError_t launch_adj_finish(const InstDesc* insts, const AdjBufs* bufs, const 
                               double* out, int ninst, cudaStream_t st);
 cudaError_t launch_adj_pull_out(int Q, const InstDesc* insts, int inst, long long N, const float* lam,
                                 float* out, cudaStream_t st);
-cudaError_t launch_adj_state(const InstDesc* insts, int inst, int np, double* rec, int to_record,
-                             cudaStream_t st);
+cudaError_t launch_adj_state(const InstDesc* insts, const AdjSeg* seg, int ninst, int s, AdjStateOp op, cudaStream_t st);
 }  // namespace lbmpen
 
 using namespace lbmpen;
@@ -72,7 +72,9 @@ struct Instance {
     int np = 0, cap = 0;
     int ntile[3] = {1, 1, 1};
     int ntiles = 0, tile0 = 0;
+    int ref0 = 0;  // first entry of its particles in the particle table
     int maxk = 0;
+    DevBuf fslab, lslab, pslab;  // the allocations that hold the buffers below (slab_alloc)
     DevBuf f[2], prec, lcnt[2], lent[2], lrec[2], tot[2], tot_scratch, pst[2], Xp[2], X, U, W, Un, Wn, theta, A, R, ratio, count, Xk, pconst, Xsf, invc,
         Ubar, Xf, Acor, rconst;
     std::vector<double> hR;      // radii, semi-major axes of ellipses (validation)
@@ -83,9 +85,11 @@ struct Instance {
 // Adjoint recording of one instance: checkpoints of the forward pass and the
 // per-step records of the segment being recomputed.
 struct AdjInst {
-    std::vector<DevBuf> ckpt;   // [nseg] populations at the start of each segment
+    DevBuf ckpt;                // [nseg] populations at the start of each segment
     DevBuf ckst;                // [nseg + 1][np][16] particle state at segment starts, then the final one
-    std::vector<DevBuf> slot;   // [L + 1] populations entering each step of the segment
+    DevBuf slot;                // [L + 1] populations entering each step of the segment
+    size_t pitch = 0;           // bytes of one population buffer in ckpt and slot
+    DevBuf rslab;               // the allocation of the buffers below (slab_alloc)
     DevBuf rprec, rlcnt, rlent, rlrec, rgeo, rstate;  // [L + 1] records of each step
     DevBuf fbar[2];             // adjoint of the pre-collision populations (ping-pong)
     DevBuf pbuf;                // adjoint particle arrays (AdjBufs)
@@ -95,7 +99,7 @@ struct AdjCtx {
     bool ready = false;         // a recorded forward pass matches the current state
     int nsteps = 0, L = 0, nseg = 0;
     std::vector<AdjInst> ai;
-    DevBuf d_rdesc, d_rtmaps, d_afl, d_apt, d_abufs, d_out, d_out_off;
+    DevBuf d_rdesc, d_rtmaps, d_afl, d_apt, d_abufs, d_out, d_out_off, d_seg;
     cudaGraphExec_t seg_exec = nullptr;  // recompute + backward of one full segment
 };
 
@@ -175,6 +179,29 @@ void dfree(lbm_ctx* ctx, DevBuf& b) {
 }
 
 template <class T> T* P(const DevBuf& b) { return static_cast<T*>(b.ptr); }
+
+// Several buffers in one allocation (slab), each 256-byte aligned, in the order
+// given.  An allocator call costs several microseconds (a Python callback with
+// the torch allocator); one per buffer was most of the time that a context of
+// 64 instances took to build.  The parts are freed with the slab.
+struct Part {
+    DevBuf* buf;
+    size_t bytes;
+};
+int slab_alloc(lbm_ctx* ctx, DevBuf& slab, std::initializer_list<Part> parts) {
+    auto up = [](size_t b) { return (std::max<size_t>(b, 1) + 255) & ~(size_t)255; };
+    size_t total = 0;
+    for (const Part& p : parts) total += up(p.bytes);
+    const int rc = dalloc(ctx, slab, total);
+    if (rc) return rc;
+    char* q = static_cast<char*>(slab.ptr);
+    for (const Part& p : parts) {
+        p.buf->ptr = q;
+        p.buf->bytes = up(p.bytes);
+        q += up(p.bytes);
+    }
+    return LBM_OK;
+}
 
 int validate(const lbm_config* c, char* why, size_t nwhy) {
     auto bad = [&](const char* m) {
@@ -322,22 +349,27 @@ void invalidate_graphs(lbm_ctx* ctx) {
     }
 }
 
-int upload_descs(lbm_ctx* ctx) {
+// Descriptors of every instance, or of instance only (>= 0), and the particle table.
+int upload_descs(lbm_ctx* ctx, int only = -1) {
     std::vector<InstDesc> h;
-    for (auto& I : ctx->inst) h.push_back(make_desc(ctx, I));
-    int rc = dalloc(ctx, ctx->d_insts, sizeof(InstDesc) * h.size());
+    const int ni = (int)ctx->inst.size(), i0 = only < 0 ? 0 : only;
+    for (int i = i0; i < (only < 0 ? ni : only + 1); ++i) h.push_back(make_desc(ctx, ctx->inst[i]));
+    int rc = dalloc(ctx, ctx->d_insts, sizeof(InstDesc) * ni);
     if (rc) return rc;
-    CK(cudaMemcpyAsync(ctx->d_insts.ptr, h.data(), sizeof(InstDesc) * h.size(),
+    CK(cudaMemcpyAsync(P<InstDesc>(ctx->d_insts) + i0, h.data(), sizeof(InstDesc) * h.size(),
                        cudaMemcpyHostToDevice, ctx->st));
     // particle reference table for the per-particle kernels, padded per
     // instance to whole blocks of 8 so that no block straddles two instances
     std::vector<PartRef> refs;
-    for (int i = 0; i < (int)ctx->inst.size(); ++i) {
+    size_t cap = 0;
+    for (int i = 0; i < ni; ++i) {
+        ctx->inst[i].ref0 = (int)refs.size();
         for (int p = 0; p < ctx->inst[i].np; ++p) refs.push_back({i, p});
         while (refs.size() % 8) refs.push_back({-1, 0});
+        cap += ((size_t)ctx->inst[i].cap + 7) & ~(size_t)7;
     }
     ctx->np_total = (int)refs.size();
-    rc = dalloc(ctx, ctx->d_refs, sizeof(PartRef) * std::max<size_t>(refs.size(), 1));
+    rc = dalloc(ctx, ctx->d_refs, sizeof(PartRef) * std::max<size_t>(cap, 1));
     if (rc) return rc;
     if (!refs.empty())
         CK(cudaMemcpyAsync(ctx->d_refs.ptr, refs.data(), sizeof(PartRef) * refs.size(),
@@ -350,11 +382,10 @@ int upload_descs(lbm_ctx* ctx) {
 // gravity), C/eps_p and C/eps_w with C = (rho_s - rho_f)|g| (Eqs. 19-20),
 // 1/delta, 1/rho_s (the mass is rho_s times the node count), R and the
 // semi-minor axis B (B == R: disk or sphere).
-int upload_pconst(lbm_ctx* ctx, Instance& I) {
-    if (I.np == 0) return LBM_OK;
+void particle_constants(const Instance& I, std::vector<double>& pc, std::vector<RecConst>& rc) {
     const lbm_config& c = I.cfg;
     const double g = sqrt(c.g_grav[0] * c.g_grav[0] + c.g_grav[1] * c.g_grav[1] + c.g_grav[2] * c.g_grav[2]);
-    std::vector<double> pc(PCONST_N * (size_t)I.np, 0.0);
+    pc.assign(PCONST_N * (size_t)I.np, 0.0);
     for (int p = 0; p < I.np; ++p) {
         const double C = (I.hratio[p] - 1.0) * c.rho_f * g;
         double* q = pc.data() + PCONST_N * p;
@@ -366,13 +397,12 @@ int upload_pconst(lbm_ctx* ctx, Instance& I) {
         q[PC_R] = I.hR[p];
         q[PC_B] = I.hB[p];
     }
-    CK(cudaMemcpy(I.pconst.ptr, pc.data(), sizeof(double) * pc.size(), cudaMemcpyHostToDevice));
     // record fields that depend only on the size and shape: R^2 and B^2 as the
     // exact test of Eq. 9 takes them, and the float bands of its filter.  The
     // ellipse band: the float form (r.e / a)^2 + (r.e_perp / b)^2 carries a
     // relative error below ~1e-6 (1 + a/b) within the circumscribed circle,
     // and the band is ten times that.
-    std::vector<RecConst> rc((size_t)I.np);
+    rc.assign((size_t)I.np, RecConst{});
     for (int p = 0; p < I.np; ++p) {
         const double R = I.hR[p], B = I.hB[p];
         RecConst& r = rc[p];
@@ -390,20 +420,30 @@ int upload_pconst(lbm_ctx* ctx, Instance& I) {
         const int H = (int)ceil(R) + 2;
         r.rows2 = (H - 1) * (H - 1);
     }
+}
+int upload_pconst(lbm_ctx* ctx, Instance& I) {
+    if (I.np == 0) return LBM_OK;
+    std::vector<double> pc;
+    std::vector<RecConst> rc;
+    particle_constants(I, pc, rc);
+    CK(cudaMemcpy(I.pconst.ptr, pc.data(), sizeof(double) * pc.size(), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(I.rconst.ptr, rc.data(), sizeof(RecConst) * rc.size(), cudaMemcpyHostToDevice));
     return LBM_OK;
 }
 
 // Re-publish every particle into the tile lists of the current parity.
-int republish(lbm_ctx* ctx) {
-    for (auto& I : ctx->inst) {
-        if (I.np == 0) continue;
+// With only >= 0: instance only, whose particles changed; the others' lists hold.
+int republish(lbm_ctx* ctx, int only = -1) {
+    for (int i = 0; i < (int)ctx->inst.size(); ++i) {
+        Instance& I = ctx->inst[i];
+        if (I.np == 0 || (only >= 0 && i != only)) continue;
         CK(cudaMemsetAsync(I.lcnt[ctx->par].ptr, 0, sizeof(int) * I.ntiles, ctx->st));
         CK(cudaMemsetAsync(I.tot[ctx->par].ptr, 0, I.tot[ctx->par].bytes, ctx->st));
     }
-    if (ctx->np_total > 0)
-        CK(launch_publish(P<InstDesc>(ctx->d_insts), P<PartRef>(ctx->d_refs), ctx->np_total, ctx->D,
-                          ctx->par, ctx->shape, ctx->st));
+    const int r0 = only < 0 ? 0 : ctx->inst[only].ref0, n = only < 0 ? ctx->np_total : ctx->inst[only].np;
+    if (n > 0)
+        CK(launch_publish(P<InstDesc>(ctx->d_insts), P<PartRef>(ctx->d_refs) + r0, n, ctx->D, ctx->par, ctx->shape,
+                          ctx->st));
     return LBM_OK;
 }
 
@@ -499,13 +539,12 @@ int configure_shape(lbm_ctx* ctx, const Shape& sh_in) {
         tile0 += I.ntiles;
         tab.insert(tab.end(), (size_t)I.ntiles, (uint16_t)i);
         I.maxk = max_slots(I, ctx->D, ctx->shape);
-        int rc;
-        for (int b = 0; b < 2; ++b) {
-            if ((rc = dalloc(ctx, I.lcnt[b], sizeof(int) * I.ntiles))) return rc;
-            if ((rc = dalloc(ctx, I.lent[b], sizeof(uint32_t) * (size_t)I.ntiles * LIST_CAP))) return rc;
-            if ((rc = dalloc(ctx, I.lrec[b], (size_t)CAND_BYTES * I.ntiles * LIST_CAP))) return rc;
-            CK(cudaMemsetAsync(I.lcnt[b].ptr, 0, sizeof(int) * I.ntiles, ctx->st));
-        }
+        const size_t nc = sizeof(int) * I.ntiles, ne = sizeof(uint32_t) * (size_t)I.ntiles * LIST_CAP,
+                     nr = (size_t)CAND_BYTES * I.ntiles * LIST_CAP;
+        const int rc = slab_alloc(ctx, I.lslab, {{&I.lcnt[0], nc}, {&I.lcnt[1], nc}, {&I.lent[0], ne}, {&I.lent[1], ne},
+                                                 {&I.lrec[0], nr}, {&I.lrec[1], nr}});
+        if (rc) return rc;
+        CK(cudaMemsetAsync(I.lcnt[0].ptr, 0, I.lcnt[0].bytes + I.lcnt[1].bytes, ctx->st));
     }
     ctx->ntiles = tile0;
     int rc = dalloc(ctx, ctx->d_tile_inst, sizeof(uint16_t) * tab.size());
@@ -611,14 +650,10 @@ void adj_release(lbm_ctx* ctx) {
     AdjCtx& A = ctx->adj;
     adj_drop_graph(A);
     for (auto& a : A.ai) {
-        for (auto& b : a.ckpt) dfree(ctx, b);
-        for (auto& b : a.slot) dfree(ctx, b);
-        DevBuf* bufs[] = {&a.ckst, &a.rprec, &a.rlcnt, &a.rlent, &a.rlrec, &a.rgeo, &a.rstate, &a.fbar[0],
-                          &a.fbar[1], &a.pbuf, &a.tot, &a.pst, &a.Xp};
-        for (DevBuf* b : bufs) dfree(ctx, *b);
+        for (DevBuf* b : {&a.ckpt, &a.slot, &a.ckst, &a.rslab}) dfree(ctx, *b);
     }
     A.ai.clear();
-    DevBuf* bufs[] = {&A.d_rdesc, &A.d_rtmaps, &A.d_afl, &A.d_apt, &A.d_abufs, &A.d_out, &A.d_out_off};
+    DevBuf* bufs[] = {&A.d_rdesc, &A.d_rtmaps, &A.d_afl, &A.d_apt, &A.d_abufs, &A.d_out, &A.d_out_off, &A.d_seg};
     for (DevBuf* b : bufs) dfree(ctx, *b);
     A.ready = false;
 }
@@ -627,11 +662,7 @@ void destroy_all(lbm_ctx* ctx) {
     adj_release(ctx);
     invalidate_graphs(ctx);
     for (auto& I : ctx->inst) {
-        DevBuf* bufs[] = {&I.f[0], &I.f[1], &I.prec, &I.lcnt[0], &I.lcnt[1], &I.lent[0], &I.lent[1],
-                          &I.lrec[0], &I.lrec[1],
-                          &I.tot[0], &I.tot[1], &I.tot_scratch, &I.pst[0], &I.pst[1], &I.Xp[0], &I.Xp[1], &I.X, &I.U, &I.W, &I.Un, &I.Wn, &I.theta, &I.A, &I.R,
-                          &I.ratio, &I.count, &I.Xk, &I.Ubar, &I.Xf, &I.pconst, &I.Xsf, &I.invc, &I.Acor, &I.rconst};
-        for (DevBuf* b : bufs) dfree(ctx, *b);
+        for (DevBuf* b : {&I.fslab, &I.lslab, &I.pslab}) dfree(ctx, *b);
     }
     dfree(ctx, ctx->d_insts);
     dfree(ctx, ctx->d_tile_inst);
@@ -642,29 +673,20 @@ void destroy_all(lbm_ctx* ctx) {
     dfree(ctx, ctx->d_gridbar);
 }
 
+// The particle arrays of an instance.  X .. count come first, at one stride
+// (count is padded to it), so that they can be read back by one strided copy;
+// X .. rconst are everything that a first insertion of particles fills.
 int alloc_particles(lbm_ctx* ctx, Instance& I, int cap) {
-    DevBuf* v3[] = {&I.X, &I.U, &I.W, &I.Un, &I.Wn, &I.theta, &I.A, &I.Ubar, &I.Acor};
-    int rc;
-    const size_t c = (size_t)std::max(cap, 1);
-    for (DevBuf* b : v3)
-        if ((rc = dalloc(ctx, *b, sizeof(double) * 3 * c))) return rc;
-    if ((rc = dalloc(ctx, I.R, sizeof(double) * c))) return rc;
-    if ((rc = dalloc(ctx, I.ratio, sizeof(double) * c))) return rc;
-    if ((rc = dalloc(ctx, I.count, sizeof(int) * c))) return rc;
-    if ((rc = dalloc(ctx, I.prec, sizeof(PRec) * c))) return rc;
-    if ((rc = dalloc(ctx, I.Xk, sizeof(double) * 6 * c))) return rc;
-    if ((rc = dalloc(ctx, I.Xf, sizeof(float) * 8 * c))) return rc;
-    if ((rc = dalloc(ctx, I.pconst, sizeof(double) * PCONST_N * c))) return rc;
-    if ((rc = dalloc(ctx, I.rconst, sizeof(RecConst) * c))) return rc;
-    if ((rc = dalloc(ctx, I.invc, sizeof(double) * c))) return rc;
-    if ((rc = dalloc(ctx, I.Xsf, sizeof(float) * 8 * c))) return rc;
-    for (int b = 0; b < 2; ++b) {
-        if ((rc = dalloc(ctx, I.tot[b], sizeof(long long) * NPV * c))) return rc;
-        if ((rc = dalloc(ctx, I.pst[b], sizeof(PState) * c))) return rc;
-        if ((rc = dalloc(ctx, I.Xp[b], sizeof(float4) * c))) return rc;
-    }
-    if ((rc = dalloc(ctx, I.tot_scratch, sizeof(long long) * NPV * c))) return rc;
-    return LBM_OK;
+    const size_t c = (size_t)std::max(cap, 1), v = sizeof(double) * 3 * c;
+    return slab_alloc(ctx, I.pslab,
+                      {{&I.X, v}, {&I.U, v}, {&I.W, v}, {&I.theta, v}, {&I.A, v}, {&I.count, v}, {&I.Un, v}, {&I.Wn, v},
+                       {&I.R, sizeof(double) * c}, {&I.ratio, sizeof(double) * c},
+                       {&I.pconst, sizeof(double) * PCONST_N * c}, {&I.rconst, sizeof(RecConst) * c},
+                       {&I.Ubar, v}, {&I.Acor, v}, {&I.prec, sizeof(PRec) * c}, {&I.Xk, 2 * v},
+                       {&I.Xf, sizeof(float) * 8 * c}, {&I.Xsf, sizeof(float) * 8 * c}, {&I.invc, sizeof(double) * c},
+                       {&I.tot[0], sizeof(long long) * NPV * c}, {&I.tot[1], sizeof(long long) * NPV * c},
+                       {&I.tot_scratch, sizeof(long long) * NPV * c}, {&I.pst[0], sizeof(PState) * c},
+                       {&I.pst[1], sizeof(PState) * c}, {&I.Xp[0], sizeof(float4) * c}, {&I.Xp[1], sizeof(float4) * c}});
 }
 
 }  // namespace
@@ -751,11 +773,9 @@ int lbm_create_batch(const lbm_config* cfgs, int n, const lbm_allocator* alloc, 
         I.qstride = (long long)I.pitch * I.n[1] * I.n[2];
         I.cap = cfgs[i].max_particles;
         const size_t fb = ssz * (size_t)(ctx->Q - 1) * (size_t)I.qstride;
-        for (int b = 0; b < 2 && rc == LBM_OK; ++b) {
-            rc = dalloc(ctx, I.f[b], fb);
-            if (rc == LBM_OK && cudaMemsetAsync(I.f[b].ptr, 0, fb, ctx->st) != cudaSuccess)
-                rc = LBM_ERR_CUDA;
-        }
+        rc = slab_alloc(ctx, I.fslab, {{&I.f[0], fb}, {&I.f[1], fb}});
+        if (rc == LBM_OK && cudaMemsetAsync(I.fslab.ptr, 0, I.f[0].bytes + I.f[1].bytes, ctx->st) != cudaSuccess)
+            rc = LBM_ERR_CUDA;
         if (rc == LBM_OK) rc = alloc_particles(ctx, I, I.cap);
     }
     if (rc == LBM_OK) rc = dalloc(ctx, ctx->d_tile_ctr, sizeof(int) * 2);
@@ -838,31 +858,56 @@ static int add_particles_impl(lbm_ctx* ctx, int i, int n, const double* pos, con
                 for (int d = 0; d < 3; ++d) W[3 * k + d] = omega[3 * k + d];
         }
     }
-    const size_t o3 = sizeof(double) * 3 * I.np, b3 = sizeof(double) * 3 * n;
-    auto up = [&](DevBuf& b, const std::vector<double>& v) {
-        return cudaMemcpyAsync(static_cast<char*>(b.ptr) + o3, v.data(), b3, cudaMemcpyHostToDevice,
-                               ctx->st);
-    };
-    CK(up(I.X, X));
-    CK(up(I.U, U));
-    CK(up(I.W, W));
-    CK(up(I.Un, U));
-    CK(up(I.Wn, W));
-    CK(up(I.theta, T));
-    CK(up(I.A, Z));
-    CK(cudaMemcpyAsync(P<double>(I.R) + I.np, radius, sizeof(double) * n, cudaMemcpyHostToDevice, ctx->st));
-    CK(cudaMemcpyAsync(P<double>(I.ratio) + I.np, ratio, sizeof(double) * n, cudaMemcpyHostToDevice, ctx->st));
-    CK(cudaMemsetAsync(P<int>(I.count) + I.np, 0, sizeof(int) * n, ctx->st));
-    CK(cudaStreamSynchronize(ctx->st));
+    const int np0 = I.np;
     I.np += n;
     I.hR.insert(I.hR.end(), radius, radius + n);
     if (minor) I.hB.insert(I.hB.end(), minor, minor + n);
     else I.hB.insert(I.hB.end(), radius, radius + n);
     I.hratio.insert(I.hratio.end(), ratio, ratio + n);
-    if ((rc = upload_pconst(ctx, I))) return rc;
-    if ((rc = upload_descs(ctx))) return rc;
+    if (np0 == 0) {  // the first particles: their arrays as one image, X .. rconst
+        std::vector<double> pc;
+        std::vector<RecConst> rcs;
+        particle_constants(I, pc, rcs);
+        const char* base = P<char>(I.X);
+        std::vector<char> img((size_t)(P<char>(I.rconst) - base) + I.rconst.bytes, 0);
+        auto put = [&](const DevBuf& b, const void* src, size_t bytes) {
+            memcpy(img.data() + (static_cast<const char*>(b.ptr) - base), src, bytes);
+        };
+        const size_t b3 = sizeof(double) * 3 * n, b1 = sizeof(double) * n;
+        put(I.X, X.data(), b3);
+        put(I.U, U.data(), b3);
+        put(I.W, W.data(), b3);
+        put(I.Un, U.data(), b3);
+        put(I.Wn, W.data(), b3);
+        put(I.theta, T.data(), b3);
+        put(I.R, radius, b1);
+        put(I.ratio, ratio, b1);
+        put(I.pconst, pc.data(), sizeof(double) * pc.size());
+        put(I.rconst, rcs.data(), sizeof(RecConst) * rcs.size());
+        CK(cudaMemcpyAsync(I.X.ptr, img.data(), img.size(), cudaMemcpyHostToDevice, ctx->st));
+        CK(cudaStreamSynchronize(ctx->st));  // img goes out of scope
+    } else {
+        const size_t o3 = sizeof(double) * 3 * np0, b3 = sizeof(double) * 3 * n;
+        auto up = [&](DevBuf& b, const std::vector<double>& v) {
+            return cudaMemcpyAsync(static_cast<char*>(b.ptr) + o3, v.data(), b3, cudaMemcpyHostToDevice,
+                                   ctx->st);
+        };
+        CK(up(I.X, X));
+        CK(up(I.U, U));
+        CK(up(I.W, W));
+        CK(up(I.Un, U));
+        CK(up(I.Wn, W));
+        CK(up(I.theta, T));
+        CK(up(I.A, Z));
+        CK(cudaMemcpyAsync(P<double>(I.R) + np0, radius, sizeof(double) * n, cudaMemcpyHostToDevice, ctx->st));
+        CK(cudaMemcpyAsync(P<double>(I.ratio) + np0, ratio, sizeof(double) * n, cudaMemcpyHostToDevice, ctx->st));
+        CK(cudaMemsetAsync(P<int>(I.count) + np0, 0, sizeof(int) * n, ctx->st));
+        CK(cudaStreamSynchronize(ctx->st));
+        if ((rc = upload_pconst(ctx, I))) return rc;
+    }
+    if ((rc = upload_descs(ctx, i))) return rc;
     invalidate_graphs(ctx);
-    return republish(ctx);
+    return republish(ctx, i);
 }
 
 int lbm_add_particles(lbm_ctx* ctx, int i, int n, const double* pos, const double* radius,
@@ -1012,15 +1057,13 @@ int lbm_get_particles(lbm_ctx* ctx, int i, double* pos, double* vel, double* ome
     Instance& I = ctx->inst[i];
     const int n = I.np, D = ctx->D;
     if (n == 0) return LBM_OK;
-    std::vector<double> X(3 * n), U(3 * n), W(3 * n), T(3 * n), A(3 * n);
-    std::vector<int> C(n);
+    // X, U, W, theta, A and count lie at one stride (alloc_particles): one copy
+    const size_t b3 = sizeof(double) * 3 * n;
+    std::vector<double> all(6 * 3 * (size_t)n);
     CK(cudaStreamSynchronize(ctx->st));
-    CK(cudaMemcpy(X.data(), I.X.ptr, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(U.data(), I.U.ptr, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(W.data(), I.W.ptr, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(T.data(), I.theta.ptr, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(A.data(), I.A.ptr, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(C.data(), I.count.ptr, sizeof(int) * n, cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy2D(all.data(), b3, I.X.ptr, I.X.bytes, b3, 6, cudaMemcpyDeviceToHost));
+    const double *X = all.data(), *U = X + 3 * n, *W = U + 3 * n, *T = W + 3 * n, *A = T + 3 * n;
+    const int* C = reinterpret_cast<const int*>(A + 3 * n);
     for (int k = 0; k < n; ++k) {
         for (int d = 0; d < D; ++d) {
             if (pos) pos[k * D + d] = X[3 * k + d];
@@ -1344,6 +1387,22 @@ long long lbm_total_nodes(const lbm_ctx* ctx) {
 }
 
 // ------------------------------------------------------------- adjoint ---
+// Per-instance pointers of k_adj_state.
+static int adj_upload_seg(lbm_ctx* ctx) {
+    AdjCtx& A = ctx->adj;
+    std::vector<AdjSeg> sg;
+    for (size_t i = 0; i < ctx->inst.size(); ++i) {
+        AdjInst& a = A.ai[i];
+        sg.push_back(AdjSeg{P<double>(a.ckst), P<double>(a.rstate), P<long long>(a.tot), P<int>(a.rlcnt),
+                            ctx->inst[i].ntiles, 0});
+    }
+    const int rc = dalloc(ctx, A.d_seg, sizeof(AdjSeg) * sg.size());
+    if (rc) return rc;
+    CK(cudaMemcpyAsync(A.d_seg.ptr, sg.data(), sizeof(AdjSeg) * sg.size(), cudaMemcpyHostToDevice, ctx->st));
+    CK(cudaStreamSynchronize(ctx->st));  // sg goes out of scope
+    return LBM_OK;
+}
+
 // Forward pass with checkpoints: the populations and particle state at the
 // start of every segment of L steps (L = ceil(sqrt(nsteps)) by default), and
 // the final particle state.  The context advances by nsteps like lbm_step.
@@ -1374,28 +1433,23 @@ int lbm_adjoint_forward(lbm_ctx* ctx, int nsteps, int seg_len) {
         Instance& I = ctx->inst[i];
         AdjInst& a = A.ai[i];
         const size_t fb = ssz * (size_t)(ctx->Q - 1) * (size_t)I.qstride;
-        for (size_t s = nseg; s < a.ckpt.size(); ++s) dfree(ctx, a.ckpt[s]);
-        a.ckpt.resize(nseg);
-        for (int s = 0; s < nseg; ++s)
-            if ((rc = dalloc(ctx, a.ckpt[s], fb))) return rc;
+        a.pitch = (fb + 255) & ~(size_t)255;
+        if (a.ckpt.bytes > 2 * a.pitch * nseg) dfree(ctx, a.ckpt);  // a much longer earlier pass: give it back
+        if ((rc = dalloc(ctx, a.ckpt, a.pitch * nseg))) return rc;
         if ((rc = dalloc(ctx, a.ckst, sizeof(double) * 16 * (size_t)std::max(I.np, 1) * (nseg + 1)))) return rc;
     }
+    if ((rc = adj_upload_seg(ctx))) return rc;
     for (int s = 0; s < nseg; ++s) {
         for (int i = 0; i < ni; ++i) {
             Instance& I = ctx->inst[i];
             AdjInst& a = A.ai[i];
-            CK(cudaMemcpyAsync(a.ckpt[s].ptr, I.f[ctx->par].ptr, a.ckpt[s].bytes, cudaMemcpyDeviceToDevice,
-                               ctx->st));
-            CK(launch_adj_state(P<InstDesc>(ctx->d_insts), i, I.np, P<double>(a.ckst) + 16LL * I.np * s, 1,
-                                ctx->st));
+            CK(cudaMemcpyAsync(P<char>(a.ckpt) + a.pitch * s, I.f[ctx->par].ptr,
+                               ssz * (size_t)(ctx->Q - 1) * (size_t)I.qstride, cudaMemcpyDeviceToDevice, ctx->st));
         }
+        CK(launch_adj_state(P<InstDesc>(ctx->d_insts), P<AdjSeg>(A.d_seg), ni, s, ADJ_SAVE, ctx->st));
         if ((rc = step_impl(ctx, std::min(L, nsteps - s * L)))) return rc;
     }
-    for (int i = 0; i < ni; ++i) {
-        Instance& I = ctx->inst[i];
-        CK(launch_adj_state(P<InstDesc>(ctx->d_insts), i, I.np, P<double>(A.ai[i].ckst) + 16LL * I.np * nseg,
-                            1, ctx->st));
-    }
+    CK(launch_adj_state(P<InstDesc>(ctx->d_insts), P<AdjSeg>(A.d_seg), ni, nseg, ADJ_SAVE, ctx->st));
     A.nsteps = nsteps;
     A.L = L;
     A.nseg = nseg;
@@ -1446,25 +1500,20 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
         Instance& I = ctx->inst[i];
         AdjInst& a = A.ai[i];
         const size_t n1 = (size_t)std::max(I.np, 1);
-        const size_t fb = ssz * (size_t)(ctx->Q - 1) * (size_t)I.qstride;
-        for (size_t k = L + 1; k < a.slot.size(); ++k) dfree(ctx, a.slot[k]);
-        a.slot.resize(L + 1);
-        for (int k = 0; k <= L; ++k)
-            if ((rc = dalloc(ctx, a.slot[k], fb))) return rc;
-        if ((rc = dalloc(ctx, a.rprec, sizeof(PRec) * n1 * (L + 1))) ||
-            (rc = dalloc(ctx, a.rlcnt, sizeof(int) * (size_t)I.ntiles * (L + 1))) ||
-            (rc = dalloc(ctx, a.rlent, sizeof(uint32_t) * (size_t)I.ntiles * LIST_CAP * (L + 1))) ||
-            (rc = dalloc(ctx, a.rlrec, (size_t)CAND_BYTES * I.ntiles * LIST_CAP * (L + 1))) ||
-            (rc = dalloc(ctx, a.rgeo, sizeof(double) * NPV * n1 * (L + 1))) ||
-            (rc = dalloc(ctx, a.rstate, sizeof(double) * 16 * n1 * (L + 1))) ||
-            (rc = dalloc(ctx, a.fbar[0], sizeof(float) * (ctx->Q - 1) * (size_t)I.qstride)) ||
-            (rc = dalloc(ctx, a.fbar[1], sizeof(float) * (ctx->Q - 1) * (size_t)I.qstride)) ||
-            (rc = dalloc(ctx, a.tot, sizeof(long long) * NPV * n1 * 2)) ||
-            (rc = dalloc(ctx, a.pst, sizeof(PState) * n1 * 2)) || (rc = dalloc(ctx, a.Xp, sizeof(float4) * n1 * 2)) ||
-            (rc = dalloc(ctx, a.pbuf, sizeof(double) * adj_pbuf_doubles(I.np, K))))
-            return rc;
+        const size_t fbar = sizeof(float) * (ctx->Q - 1) * (size_t)I.qstride, l1 = (size_t)L + 1, nt = (size_t)I.ntiles;
+        if (a.slot.bytes > 2 * a.pitch * l1) dfree(ctx, a.slot);
+        if ((rc = dalloc(ctx, a.slot, a.pitch * l1))) return rc;
+        rc = slab_alloc(ctx, a.rslab,
+                        {{&a.rprec, sizeof(PRec) * n1 * l1}, {&a.rlcnt, sizeof(int) * nt * l1},
+                         {&a.rlent, sizeof(uint32_t) * nt * LIST_CAP * l1}, {&a.rlrec, (size_t)CAND_BYTES * nt * LIST_CAP * l1},
+                         {&a.rgeo, sizeof(double) * NPV * n1 * l1}, {&a.rstate, sizeof(double) * 16 * n1 * l1},
+                         {&a.fbar[0], fbar}, {&a.fbar[1], fbar}, {&a.tot, sizeof(long long) * NPV * n1 * 2},
+                         {&a.pst, sizeof(PState) * n1 * 2}, {&a.Xp, sizeof(float4) * n1 * 2},
+                         {&a.pbuf, sizeof(double) * adj_pbuf_doubles(I.np, K)}});
+        if (rc) return rc;
         CK(cudaMemsetAsync(a.pbuf.ptr, 0, a.pbuf.bytes, ctx->st));
     }
+    if ((rc = adj_upload_seg(ctx))) return rc;
     // descriptors of the recomputation: step k reads slot k and writes slot
     // k + 1, its records go to record k (and k + 1 for the next step's input);
     // entry L is the publish of a segment's first state into record 0
@@ -1493,8 +1542,8 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
                 d.list_rec[0] = lr;
             } else {
                 const int par = k & 1;
-                d.f[par] = a.slot[k].ptr;
-                d.f[par ^ 1] = a.slot[k + 1].ptr;
+                d.f[par] = P<char>(a.slot) + a.pitch * k;
+                d.f[par ^ 1] = P<char>(a.slot) + a.pitch * (k + 1);
                 d.prec = rp + n1 * k;
                 d.prec_out = rp + n1 * (k + 1);
                 d.list_cnt[par] = lc + (size_t)I.ntiles * k;
@@ -1506,8 +1555,8 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
                 d.adj_geo = P<double>(a.rgeo) + NPV * n1 * k;
                 d.rec_state = P<double>(a.rstate) + 16 * n1 * (k + 1);
                 if (tma) {
-                    if ((rc = encode_pop_map(ctx, I, a.slot[k].ptr, &tm[(size_t)k * ni * 2 + 2 * i + par]))) return rc;
-                    if ((rc = encode_pop_map(ctx, I, a.slot[k + 1].ptr, &tm[(size_t)k * ni * 2 + 2 * i + (par ^ 1)])))
+                    if ((rc = encode_pop_map(ctx, I, d.f[par], &tm[(size_t)k * ni * 2 + 2 * i + par]))) return rc;
+                    if ((rc = encode_pop_map(ctx, I, d.f[par ^ 1], &tm[(size_t)k * ni * 2 + 2 * i + (par ^ 1)])))
                         return rc;
                 }
             }
@@ -1545,7 +1594,7 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
             AdjInst& a = A.ai[i];
             const size_t n1 = (size_t)std::max(I.np, 1);
             AdjFluid f;
-            f.fin = a.slot[kk].ptr;
+            f.fin = P<char>(a.slot) + a.pitch * kk;
             f.prec = P<PRec>(a.rprec) + n1 * kk;
             f.lcnt = P<int>(a.rlcnt) + (size_t)I.ntiles * kk;
             f.lrec = P<char>(a.rlrec) + (size_t)CAND_BYTES * I.ntiles * LIST_CAP * kk;
@@ -1621,14 +1670,10 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
         for (int i = 0; i < ni; ++i) {
             Instance& I = ctx->inst[i];
             AdjInst& a = A.ai[i];
-            CK(cudaMemcpyAsync(a.slot[0].ptr, a.ckpt[s].ptr, a.ckpt[s].bytes, cudaMemcpyDeviceToDevice, ctx->st));
-            double* st = P<double>(a.ckst) + 16LL * I.np * s;
-            CK(launch_adj_state(dI, i, I.np, st, 0, ctx->st));
-            if (I.np)
-                CK(cudaMemcpyAsync(a.rstate.ptr, st, sizeof(double) * 16 * I.np, cudaMemcpyDeviceToDevice, ctx->st));
-            CK(cudaMemsetAsync(a.rlcnt.ptr, 0, sizeof(int) * I.ntiles, ctx->st));
-            CK(cudaMemsetAsync(a.tot.ptr, 0, a.tot.bytes, ctx->st));
+            CK(cudaMemcpyAsync(a.slot.ptr, P<char>(a.ckpt) + a.pitch * s, ssz * (size_t)(ctx->Q - 1) * (size_t)I.qstride,
+                               cudaMemcpyDeviceToDevice, ctx->st));
         }
+        CK(launch_adj_state(dI, P<AdjSeg>(A.d_seg), ni, s, ADJ_RESTART, ctx->st));
         if (ctx->np_total > 0)
             CK(launch_publish(dR + (size_t)L * ni, P<PartRef>(ctx->d_refs), ctx->np_total, ctx->D, 0, sh, ctx->st));
         if (s == nseg - 1) {
@@ -1658,10 +1703,7 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
             CK(launch_adj_pull_out(ctx->Q, dI, i, Nn, P<float>(A.ai[i].fbar[0]), grad_field + field_off[i], ctx->st));
         }
     // the context returns to the state after the forward pass
-    for (int i = 0; i < ni; ++i) {
-        Instance& I = ctx->inst[i];
-        CK(launch_adj_state(dI, i, I.np, P<double>(A.ai[i].ckst) + 16LL * I.np * nseg, 0, ctx->st));
-    }
+    CK(launch_adj_state(dI, P<AdjSeg>(A.d_seg), ni, nseg, ADJ_LOAD, ctx->st));
     CK(cudaMemcpyAsync(grad_particles, A.d_out.ptr, sizeof(double) * nout, cudaMemcpyDeviceToHost, ctx->st));
     return read_status(ctx);
 }

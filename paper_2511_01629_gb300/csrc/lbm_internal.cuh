@@ -277,6 +277,18 @@ struct AdjBufs {
 // forces of K sub-steps, and six arrays of [np][3].
 __host__ __device__ inline size_t adj_scratch(int np, int K) { return 3 * (size_t)np * (3 * (size_t)K + 7); }
 
+// What k_adj_state reads and writes of an instance, and the operation on the
+// particle state of checkpoint s: save it, load it, or load it and begin the
+// recomputation of segment s from it (record 0, empty lists and totals).
+struct AdjSeg {
+    double* ckst;            // [nseg + 1][np][16] states
+    double* rstate;          // [L + 1][np][16] the recomputation's records
+    long long* tot;          // [2][np][NPV] its totals
+    int* rlcnt;              // [ntiles] its list counts of step 0
+    int ntiles, pad;
+};
+enum AdjStateOp { ADJ_SAVE, ADJ_LOAD, ADJ_RESTART };
+
 // Particle index -> (instance, local index) for the per-particle kernels.
 struct PartRef {
     int inst;
