@@ -251,51 +251,58 @@ __device__ __forceinline__ void pull_lam_pair(const InstDesc& in, const float* _
 }  // namespace
 
 // ------------------------------------------------------------ fluid sweep --
-constexpr int ADJ_WARPS = 4;  // warps per block; a tile of more rows takes several blocks
+constexpr int ADJ_WARPS = 4;   // warps per block
+constexpr int ADJ_BLOCKS = 5;  // resident blocks per SM in 2D (launch bounds)
 
 // lam_mode: 0 = pull the adjoint of step n + 1, 1 = read a field seed [Q][N]
 // (the adjoint of the final post-collision populations), 2 = zero.
-// One block per tile of the forward kernel's shape (its candidate lists are
-// per tile), one warp per tile row at a time; a lane takes two adjacent nodes
-// of a 64-node segment, all of their populations and adjoints in flight
-// before the first is used (8-byte loads where c_x = 0), and stores 8-byte
-// pairs.  HBM-bound: two reads and a write per population.
-// 16 boxes of 400 x 1600, FP32: about 285 us a step before (one node per lane,
-// scalar arithmetic over all velocities, the candidates before the loads), 212 now
-// (983 MB); one box: 32 -> 24 us.
+// A block takes a tile of the forward kernel's shape (the candidate lists are
+// per tile) or a part of one, a warp a 64-node segment of a row at a time; a
+// lane takes two adjacent nodes, all of their populations and adjoints in
+// flight before the first is used (8-byte loads where c_x = 0), and stores
+// 8-byte pairs.  The candidates are read where they are: copying them to shared
+// memory behind a barrier first cost one box of 400 x 1600 11 % of its backward
+// pass.  HBM-bound: two reads and a write per population.  16 boxes of 400 x
+// 1600, FP32: about 285 us a step before (one node per lane, scalar arithmetic
+// over all velocities, the candidates before the loads), 212 now (983 MB, 4.6
+// TB/s; what is left is load latency, at 20 warps per SM).
+// Warps that stride over all segments (760 blocks) took 22.4 ms for the 16 boxes.
 template <int Q, class S>
-__global__ void __launch_bounds__(32 * ADJ_WARPS, Q == 9 ? 5 : 3) k_adj_fluid(const InstDesc* __restrict__ insts,
-                                                   const AdjFluid* __restrict__ afs,
-                                                   const uint16_t* __restrict__ tile_inst, int ninst, int lam_mode,
-                                                   Shape sh) {
+__global__ void __launch_bounds__(32 * ADJ_WARPS, Q == 9 ? ADJ_BLOCKS : 3) k_adj_fluid(
+    const InstDesc* __restrict__ insts, const AdjFluid* __restrict__ afs, const uint16_t* __restrict__ tile_inst, int ninst,
+    int lam_mode, Shape sh) {
     using L = Lat<Q>;
     constexpr int D = L::D;
     constexpr int QS = Q - 1;
-    __shared__ Cand cand[LIST_CAP];
+    const int lane = threadIdx.x & 31;
+    const int tw = sh.tw, rows = sh.ty * sh.tz, segs = (tw + 63) >> 6;
     const int t = blockIdx.x;
     const int ii = ninst > 1 ? (int)tile_inst[t] : 0;
     const InstDesc& in = insts[ii];
     const AdjFluid& af = afs[ii];
     const int local = t - in.tile0;
-    const int tw = sh.tw;
     const int ntx = in.ntile[0], nty = in.ntile[1];
     const int rest = local / ntx;
     const int x0 = (local - rest * ntx) * tw, y0 = (rest % nty) * sh.ty, z0 = (rest / nty) * sh.tz;
     const int nx = in.n[0], ny = in.n[1], nz = in.n[2];
     const int pitch = in.pitch;
     const int qs = (int)in.qstride;  // (Q - 1) * qstride < 2^31 (validated at creation)
-    const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) + (blockDim.x >> 5) * blockIdx.y;
-    const int nwarps = (blockDim.x >> 5) * gridDim.y;  // warps of the tile
     const S* __restrict__ fin = static_cast<const S*>(af.fin);
     const float* __restrict__ lsrc = af.lam_src;
     float* __restrict__ ldst = af.lam_dst;
-    const int w = min(tw, nx - x0);
-    const int nseg = (w + 63) >> 6;
-    const int rows = sh.ty * sh.tz;
-    float2 f[QS], lam[QS];
-    // unit k of this warp: segment k % nseg of row warp + nwarps (k / nseg)
-    auto pull = [&](int y, int z, int xb) {
-        const int x = xb + 2 * lane;
+    const int ncand = in.np > 0 ? min(af.lcnt[local], LIST_CAP) : 0;
+    const Cand* cand = static_cast<const Cand*>(af.lrec) + (long long)local * LIST_CAP;
+    Geo geo = make_geo(in);
+    geo.prec = af.prec;
+    const CollK ck = make_collk<Q>(make_collp(in));
+    const float gd[3] = {in.gdrive[0], in.gdrive[1], in.gdrive[2]};
+    const bool free = gd[0] == 0.f && gd[1] == 0.f && gd[2] == 0.f;
+    for (int rs = (threadIdx.x >> 5) + ADJ_WARPS * blockIdx.y; rs < rows * segs; rs += ADJ_WARPS * gridDim.y) {
+        const int r = rs / segs, sg = rs - r * segs;
+        const int y = y0 + r % sh.ty, z = z0 + r / sh.ty, xb = x0 + 64 * sg;
+        if (xb >= nx || y >= ny || z >= nz) continue;  // warp-uniform: beyond the box
+        const int x = xb + 2 * lane, wseg = min(64, min(tw - 64 * sg, nx - xb));
+        float2 f[QS], lam[QS];
         const int xc0 = min(x, nx - 1), xc1 = min(x + 1, nx - 1);  // lanes past the row read valid nodes
         const bool row_in = y >= 1 && y + 1 < ny && (D == 2 || (z >= 1 && z + 1 < nz));
         const bool edge = xb == 0 || xb + 64 >= nx;
@@ -328,34 +335,6 @@ __global__ void __launch_bounds__(32 * ADJ_WARPS, Q == 9 ? 5 : 3) k_adj_fluid(co
 #pragma unroll
             for (int q = 0; q < QS; ++q) lam[q] = bc2(0.f);
         }
-    };
-    auto inside = [&](int r) {  // row r of the tile lies in the box
-        return r < rows && y0 + r % sh.ty < ny && z0 + r / sh.ty < nz;
-    };
-    int r = warp, sg = 0;
-    while (r < rows && !inside(r)) r += nwarps;
-    int ncand = 0;
-    Geo geo = make_geo(in);
-    geo.prec = af.prec;
-    const CollK ck = make_collk<Q>(make_collp(in));
-    const float gd[3] = {in.gdrive[0], in.gdrive[1], in.gdrive[2]};
-    const bool free = gd[0] == 0.f && gd[1] == 0.f && gd[2] == 0.f;
-    for (bool first = true;; first = false) {
-        const int y = y0 + r % sh.ty, z = z0 + r / sh.ty, xb = x0 + 64 * sg, x = xb + 2 * lane;
-        const bool have = r < rows;
-        if (have) pull(y, z, xb);
-        if (first) {  // the candidates arrive beside the first segment's values
-            if (in.np > 0) {
-                ncand = min(af.lcnt[local], LIST_CAP);
-                const uint4* src =
-                    reinterpret_cast<const uint4*>(static_cast<const Cand*>(af.lrec) + (long long)local * LIST_CAP);
-                for (int c = threadIdx.x; c < ncand * (CAND_BYTES / 16); c += blockDim.x)
-                    reinterpret_cast<uint4*>(cand)[c] = src[c];
-            }
-            __syncthreads();
-        }
-        if (!have) break;
-        const int wseg = min(64, w - 64 * sg);
         const bool v0 = 2 * lane < wseg, v1 = 2 * lane + 1 < wseg;
         const int xyz0[3] = {x, y, z}, xyz1[3] = {x + 1, y, z};
         int own0 = -1, own1 = -1, sl0 = -1, sl1 = -1;
@@ -415,11 +394,6 @@ __global__ void __launch_bounds__(32 * ADJ_WARPS, Q == 9 ? 5 : 3) k_adj_fluid(co
         } else if (v0) {
 #pragma unroll
             for (int q = 0; q < QS; ++q) out[q * qs] = lam[q].x;
-        }
-        if (++sg == nseg) {  // the warp's next segment
-            sg = 0;
-            do r += nwarps;
-            while (r < rows && !inside(r));
         }
         // per-particle sums of the adjoint acceleration and alpha derivative
         if (!any) continue;
@@ -778,15 +752,14 @@ __global__ void __launch_bounds__(256) k_adj_state(const InstDesc* __restrict__ 
 cudaError_t launch_adj_fluid(int Q, int fp16, const InstDesc* insts, const AdjFluid* afs,
                              const uint16_t* tile_inst, int ninst, int ntiles, int lam_mode, const Shape& sh,
                              cudaStream_t st) {
-    const int rows = sh.ty * sh.tz;
-    // A warp takes a row at a time.  With few tiles a tall tile goes to several
-    // blocks, a row per warp; with two waves of tiles or more one block takes all
-    // of it and starts up once (16 x 400 x 1600: 48 steps 21.4 against 22.4 ms with
-    // two; one 400 x 1600 box, 240 steps: 14.6 against 13.8 ms).
-    const bool many = ntiles >= 2 * 5 * 152;
-    const dim3 grid((unsigned)ntiles, many ? 1u : (unsigned)((rows + ADJ_WARPS - 1) / ADJ_WARPS));
-    const int threads = 32 * (rows < ADJ_WARPS ? rows : ADJ_WARPS);
-    auto go = [&](auto kern) { kern<<<grid, threads, 0, st>>>(insts, afs, tile_inst, ninst, lam_mode, sh); };
+    const int units = sh.ty * sh.tz * ((sh.tw + 63) / 64), per = (units + ADJ_WARPS - 1) / ADJ_WARPS;
+    // With few tiles every segment goes to a warp of its own; with two waves of
+    // tiles or more one block takes a whole tile and starts up once (backward pass,
+    // 1 / 2 / 4 blocks per tile: one 400 x 1600 box, 240 steps 13.4 / 12.2 / 11.9 ms;
+    // 16 of them, 48 steps 19.7 / 20.7 / 22.9 ms).
+    const bool many = ntiles >= 2 * ADJ_BLOCKS * 152;
+    const dim3 grid((unsigned)ntiles, many ? 1u : (unsigned)per);
+    auto go = [&](auto kern) { kern<<<grid, 32 * ADJ_WARPS, 0, st>>>(insts, afs, tile_inst, ninst, lam_mode, sh); };
     if (Q == 9) {
         if (fp16) go(k_adj_fluid<9, __half>);
         else go(k_adj_fluid<9, float>);
