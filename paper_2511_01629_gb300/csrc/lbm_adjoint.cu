@@ -224,26 +224,31 @@ __device__ __forceinline__ void pull_lam_pair(const InstDesc& in, const float* _
                                               float2* l) {
     using L = Lat<Q>;
     const int nx = in.n[0], pitch = in.pitch, zs = in.n[1] * pitch, qs = (int)in.qstride;
-    const int own = z * zs + y * pitch;
-    const bool wall = !in.periodic[0];
+    const int own = z * zs + y * pitch, xl = EDGE ? min(x, (nx - 1) & ~1) : x;
+    auto row_of = [&](int q) { return (q - 1) * qs + own + L::c(q, 2) * zs + L::c(q, 1) * pitch; };
 #pragma unroll
     for (int q = 1; q < Q; ++q) {
-        const int cx = L::c(q, 0);
-        const int row = (q - 1) * qs + own + L::c(q, 2) * zs + L::c(q, 1) * pitch;
-        if (cx == 0) {
-            l[q - 1] = __ldg(reinterpret_cast<const float2*>(ls + (row + (EDGE && x >= nx ? 0 : x))));
-        } else if constexpr (!EDGE) {
-            l[q - 1] = make_float2(__ldg(ls + (row + x + cx)), __ldg(ls + (row + x + 1 + cx)));
-        } else {
-            float v[2];
+        const int cx = L::c(q, 0), at = row_of(q) + xl;
+        if (cx == 0) l[q - 1] = __ldg(reinterpret_cast<const float2*>(ls + at));
+        else l[q - 1] = make_float2(__ldg(ls + (at + cx)), __ldg(ls + (at + 1 + cx)));
+    }
+    if constexpr (EDGE) {
+        const bool wall = !in.periodic[0], lo = x == 0, hi0 = x == nx - 1, hi1 = x + 1 == nx - 1;
+        float v[Q];
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int xe = min(x + e, nx - 1), xd = xe + cx;
-                const bool out = cx < 0 ? xd < 0 : xd >= nx;
-                const int off = !out ? row + xd : wall ? (L::opp(q) - 1) * qs + own + xe : row + (cx < 0 ? nx - 1 : 0);
-                v[e] = __ldg(ls + off);
-            }
-            l[q - 1] = make_float2(v[0], v[1]);
+        for (int q = 1; q < Q; ++q) {
+            const int cx = L::c(q, 0);
+            if (cx == 0) continue;
+            const int off = wall ? (L::opp(q) - 1) * qs + own + (cx < 0 ? 0 : nx - 1) : row_of(q) + (cx < 0 ? nx - 1 : 0);
+            v[q] = 0.f;
+            if (cx < 0 ? lo : hi0 || hi1) v[q] = __ldg(ls + off);
+        }
+#pragma unroll
+        for (int q = 1; q < Q; ++q) {
+            const int cx = L::c(q, 0);
+            if (cx == 0) continue;
+            if (cx < 0 ? lo : hi0) l[q - 1].x = v[q];
+            if (cx > 0 && hi1) l[q - 1].y = v[q];
         }
     }
 }
