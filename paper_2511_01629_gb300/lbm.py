@@ -373,7 +373,9 @@ class LBM:
 
     def step_timed(self, n):
         """n steps launched one by one with CUDA events around each kernel:
-        mean ms per step of (fluid kernel, box sums, particle kernel)."""
+        mean ms per step of (fluid kernel, the interval of two events with
+        nothing between them, where a kernel for the sums of Eq. 22 used to be,
+        particle kernel)."""
         t = (C.c_float * 3)()
         self._check(lib().lbm_step_timed(self._h, int(n), C.byref(t, 0), C.byref(t, 4), C.byref(t, 8)))
         return float(t[0]), float(t[1]), float(t[2])
