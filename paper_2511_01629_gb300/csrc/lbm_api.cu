@@ -460,40 +460,20 @@ PFN_cuTensorMapEncodeTiled_v12000 tmap_encoder() {
     return fn;
 }
 
-// Tensor map of one population buffer: the stored populations as a
-// [Q-1][nz][ny][pitch] tensor (x innermost, dim = nx so that boxes read
-// zeros beyond the last node).  D2Q9 boxes hold every population of a tile
-// with one halo row on each side, (tile width + 2 halo) x (ty + 2) x (Q - 1),
-// so a tile takes one copy; D3Q19 boxes hold one population's source rows,
-// (tile width + 2 halo) x ty x tz.
+// Tensor map of one D2Q9 population buffer: the stored populations as a
+// [Q-1][ny][pitch] tensor (x innermost, dim = nx so that boxes read zeros beyond
+// the last node).  A box holds every population of a tile with one halo row on
+// each side, (tile width + 2 halo) x (ty + 2) x (Q - 1), so a tile takes one copy.
 int encode_pop_map(lbm_ctx* ctx, const Instance& I, void* ptr, CUtensorMap* out) {
     auto enc = tmap_encoder();
     if (!enc) return set_err(ctx, LBM_ERR_CUDA, "cuTensorMapEncodeTiled is not available%s");
     const size_t ss = ctx->fp16 ? 2 : 4;
     const int halo = 16 / (int)ss;
-    cuuint64_t dims[4], strides[3];
-    cuuint32_t box[4], es[4] = {1, 1, 1, 1};
-    cuuint32_t rank;
-    dims[0] = (cuuint64_t)I.n[0];
-    dims[1] = (cuuint64_t)I.n[1];
-    strides[0] = (cuuint64_t)I.pitch * ss;
-    box[0] = (cuuint32_t)(ctx->shape.tw + 2 * halo);
-    box[1] = (cuuint32_t)ctx->shape.ty;
-    if (ctx->D == 2) {  // one box per tile: every population, rows y0 - 1 .. y0 + ty
-        rank = 3;
-        dims[2] = (cuuint64_t)(ctx->Q - 1);
-        strides[1] = (cuuint64_t)I.pitch * I.n[1] * ss;
-        box[1] = (cuuint32_t)(ctx->shape.ty + 2);
-        box[2] = (cuuint32_t)(ctx->Q - 1);
-    } else {
-        rank = 4;
-        dims[2] = (cuuint64_t)I.n[2];
-        dims[3] = (cuuint64_t)(ctx->Q - 1);
-        strides[1] = (cuuint64_t)I.pitch * I.n[1] * ss;
-        strides[2] = (cuuint64_t)I.pitch * I.n[1] * I.n[2] * ss;
-        box[2] = (cuuint32_t)ctx->shape.tz;
-        box[3] = 1;
-    }
+    const cuuint32_t rank = 3, es[3] = {1, 1, 1};
+    const cuuint64_t dims[3] = {(cuuint64_t)I.n[0], (cuuint64_t)I.n[1], (cuuint64_t)(ctx->Q - 1)};
+    const cuuint64_t strides[2] = {(cuuint64_t)I.pitch * ss, (cuuint64_t)I.pitch * I.n[1] * ss};
+    const cuuint32_t box[3] = {(cuuint32_t)(ctx->shape.tw + 2 * halo), (cuuint32_t)(ctx->shape.ty + 2),
+                               (cuuint32_t)(ctx->Q - 1)};
     CUresult r = enc(out, ctx->fp16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, rank,
                      ptr, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);

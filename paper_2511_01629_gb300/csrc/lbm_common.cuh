@@ -707,17 +707,10 @@ __device__ __forceinline__ void collide(float* f, const float* a, bool solid, co
     *p_out = p2.x;
 }
 
-// Fixed-point image round(u * 2^FXBITS) of a velocity component, rounded to
-// the nearest integer (ties to even): the scaling by a power of two is exact,
-// so the conversion is the only rounding.  The value is clamped to |u| < 1/2;
-// a larger or non-finite velocity is reported as divergence by the caller.
-__device__ __forceinline__ long long to_fx(float u) {
-    u = fminf(fmaxf(u, -0.49999997f), 0.49999997f);
-    return __float2ll_rn(u * 1099511627776.0f);  // u * 2^40 is exact; round to nearest even
-}
-
-// The same round(u * 2^FXBITS) by two 32-bit conversions (the 64-bit one
-// issues at the FP64 rate on this GPU): x = u 2^40 is exact, t = trunc(x 2^-20)
+// Fixed-point image round(u * 2^FXBITS) of a velocity component (ties to even),
+// |u| clamped below 1/2 (a larger or non-finite one is reported as divergence by
+// the caller), by two 32-bit conversions (the 64-bit one issues at the FP64 rate
+// on this GPU): x = u 2^40 is exact, t = trunc(x 2^-20)
 // fits in 20 bits, x - t 2^20 is exact (a multiple of ulp(x) below 2^20 in
 // magnitude, so at most 24 significant bits), and since t 2^20 is an even
 // integer, rne(x) = t 2^20 + rne(x - t 2^20), ties included.
@@ -741,12 +734,6 @@ __device__ __forceinline__ long long warp_sum_fx(long long v) {
     const long long s1 = (long long)__reduce_add_sync(0xffffffffu, l1);
     const long long s2 = (long long)__reduce_add_sync(0xffffffffu, l2);
     return s0 + s1 * (1LL << 21) + s2 * (1LL << 42);
-}
-
-__device__ __forceinline__ long long warp_sum_ll(long long v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
 }
 
 // round(u * 2^FXBITS) of two velocities as hi * 2^20 + lo (|hi| <= 2^19,
@@ -1066,45 +1053,11 @@ __device__ __forceinline__ double finalize_rotation(const long long* v, const do
     return Wo;
 }
 
-// Where population q of node (x, y, z) pulls from (Eq. 10, left side): the
-// element of the previous post-collision buffer, and the term added to it.
-// Across a periodic face the source wraps; across a wall (the first wall axis
-// in the order x, y, z) the node's own opposite population bounces back, plus
-// the moving-wall term 2 w_q (c_q . u_w) / cs^2.
-template <int Q, class S>
-__device__ __forceinline__ const S* pull_source(const InstDesc& in, const S* fin, int q, int x, int y, int z,
-                                                float* add) {
-    using L = Lat<Q>;
-    const int c[3] = {L::c(q, 0), L::c(q, 1), L::c(q, 2)};
-    int src[3] = {x - c[0], y - c[1], z - c[2]};
-    int axis = -1, face = 0;
-    for (int d = 0; d < 3; ++d) {
-        if (src[d] < 0 || src[d] >= in.n[d]) {
-            if (in.periodic[d]) src[d] = src[d] < 0 ? src[d] + in.n[d] : src[d] - in.n[d];
-            else if (axis < 0) { axis = d; face = src[d] < 0 ? 0 : 1; }
-        }
-    }
-    if (axis >= 0) {
-        *add = in.wterm[axis][face][q];
-        const long long off = ((long long)z * in.n[1] + y) * in.pitch + x;
-        return fin + (long long)(L::opp(q) - 1) * in.qstride + off;
-    }
-    *add = 0.f;
-    const long long off = ((long long)src[2] * in.n[1] + src[1]) * in.pitch + src[0];
-    return fin + (long long)(q - 1) * in.qstride + off;
-}
-
-template <int Q, class S>
-__device__ __noinline__ float pull_scalar(const InstDesc& in, const S* fin, int q, int x, int y, int z) {
-    float add;
-    const S* p = pull_source<Q, S>(in, fin, q, x, y, z, &add);
-    return VecIO<S, 1 + (sizeof(S) == 2)>::load1(p, in.s_load) + add;
-}
-
-// Pre-collision population q at node (x, y, z): pull_scalar for a
-// compile-time q, with bounce-back and the wall term where x - c_q lies beyond
-// a wall (the first such axis names the wall).  Selects instead of branches, so that the lanes of a warp
-// on a face stay together.
+// Pre-collision population q (compile-time) at node (x, y, z) (Eq. 10, left
+// side): across a periodic face the source wraps; across a wall (the first
+// wall axis in the order x, y, z) the node's own opposite population bounces
+// back, plus the moving-wall term 2 w_q (c_q . u_w) / cs^2.  Selects instead of
+// branches, so that the lanes of a warp on a face stay together.
 template <int Q, class S, int q>
 __device__ __forceinline__ float pull_pre_any(const InstDesc& in, const S* __restrict__ fin, int x, int y, int z,
                                               int qs) {

@@ -1,11 +1,10 @@
-// TMA-pipelined variant of the fused stream-collide-penalize kernel.
+// TMA-pipelined variant of the fused stream-collide-penalize kernel (D2Q9).
 //
 // Persistent blocks of one producer warp and NC consumer warps.  The producer
 // takes tiles from a work counter (successive claims alternate between the
 // two ends of the tile range) and fills a ring of shared-memory stages: the
-// tile's populations by cp.async.bulk.tensor (D2Q9: one box of every
-// population over the tile rows and one halo row on each side; D3Q19: one
-// box per population over its source rows y - c_y, z - c_z), 32*k nodes wide
+// tile's populations by cp.async.bulk.tensor (one box of every population
+// over the tile rows and one halo row on each side), 32*k nodes wide
 // plus a 16-byte halo on both sides so that every box starts on a 16-byte
 // boundary, and the tile's candidate particles by one bulk copy of the
 // records the particle kernel listed for the tile.  Everything else the
@@ -79,14 +78,6 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, i
         "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
         " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar))
-        : "memory");
-}
-__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, int c0, int c1, int c2,
-                                            int c3, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(smem_u32(bar))
         : "memory");
 }
 
@@ -262,6 +253,7 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
                                                    int par, Shape sh, int commit, int* tile_ctr,
                                                    int stages, int ninst) {
     using L = Lat<Q>;
+    static_assert(Q == 9, "D3Q19 takes k_fluid_direct");
     constexpr int D = L::D;
     constexpr int QS = Q - 1;
     constexpr int H = 16 / (int)sizeof(S);
@@ -420,16 +412,8 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
             if (lane == 0) {
                 const CUtensorMap* map = tmaps + 2 * a.ii + par;
                 unsigned char* dst = smem + s * LY.stage;
-                if (Q == 9) {
-                    mbar_expect_tx(&full[s], (uint32_t)(QS * LY.bw * (rows + 2) * (int)sizeof(S) + CAND_BYTES * ncand));
-                    tma_load_3d(dst, map, a.x0 - H, a.y0 - 1, 0, &full[s]);
-                } else {
-                    mbar_expect_tx(&full[s], (uint32_t)(QS * LY.bw * rows * (int)sizeof(S) + CAND_BYTES * ncand));
-#pragma unroll 1
-                    for (int q = 1; q < Q; ++q)
-                        tma_load_4d(dst + (q - 1) * LY.slab, map, a.x0 - H, a.y0 - d3q19_c(q, 1),
-                                    a.z0 - d3q19_c(q, 2), q - 1, &full[s]);
-                }
+                mbar_expect_tx(&full[s], (uint32_t)(QS * LY.bw * (rows + 2) * (int)sizeof(S) + CAND_BYTES * ncand));
+                tma_load_3d(dst, map, a.x0 - H, a.y0 - 1, 0, &full[s]);
                 if (ncand > 0) {
                     const Cand* lr = ninst <= TI_MAX ? tab[a.ii].lrec[par]
                                                      : static_cast<const Cand*>(insts[a.ii].list_rec[par]);
