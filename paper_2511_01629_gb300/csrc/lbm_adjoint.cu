@@ -193,7 +193,7 @@ struct NodeAdj {
 // beyond a wall (the population bounced back at x).
 template <int Q, int q>
 __device__ __forceinline__ float pull_lam_any(const InstDesc& in, const float* __restrict__ lam, int x, int y, int z,
-                                              int qs) {
+                                              long long qs) {
     using L = Lat<Q>;
     constexpr int c[3] = {L::c(q, 0), L::c(q, 1), L::c(q, 2)};
     int dst[3] = {x + c[0], y + c[1], z + c[2]};
@@ -206,11 +206,11 @@ __device__ __forceinline__ float pull_lam_any(const InstDesc& in, const float* _
         else if (out) wall = true;
     }
     const int node = (z * in.n[1] + y) * in.pitch + x;
-    const int off = wall ? (L::opp(q) - 1) * qs + node : (q - 1) * qs + (dst[2] * in.n[1] + dst[1]) * in.pitch + dst[0];
-    return __ldg(lam + off);
+    return __ldg(wall ? pop(lam, L::opp(q), qs) + node : pop(lam, q, qs) + ((dst[2] * in.n[1] + dst[1]) * in.pitch + dst[0]));
 }
 template <int Q, int q = 1>
-__device__ __forceinline__ void pull_lam_all(const InstDesc& in, const float* ls, int x, int y, int z, int qs, float* l) {
+__device__ __forceinline__ void pull_lam_all(const InstDesc& in, const float* ls, int x, int y, int z, long long qs,
+                                             float* l) {
     if constexpr (q < Q) {
         l[q - 1] = pull_lam_any<Q, q>(in, ls, x, y, z, qs);
         pull_lam_all<Q, q + 1>(in, ls, x, y, z, qs, l);
@@ -223,14 +223,16 @@ template <int Q, bool EDGE>
 __device__ __forceinline__ void pull_lam_pair(const InstDesc& in, const float* __restrict__ ls, int x, int y, int z,
                                               float2* l) {
     using L = Lat<Q>;
-    const int nx = in.n[0], pitch = in.pitch, zs = in.n[1] * pitch, qs = (int)in.qstride;
+    const int nx = in.n[0], pitch = in.pitch, zs = in.n[1] * pitch;
+    const long long qs = in.qstride;
     const int own = z * zs + y * pitch, xl = EDGE ? min(x, (nx - 1) & ~1) : x;
-    auto row_of = [&](int q) { return (q - 1) * qs + own + L::c(q, 2) * zs + L::c(q, 1) * pitch; };
+    auto row_of = [&](int q) { return own + L::c(q, 2) * zs + L::c(q, 1) * pitch; };  // within population q
 #pragma unroll
     for (int q = 1; q < Q; ++q) {
         const int cx = L::c(q, 0), at = row_of(q) + xl;
-        if (cx == 0) l[q - 1] = __ldg(reinterpret_cast<const float2*>(ls + at));
-        else l[q - 1] = make_float2(__ldg(ls + (at + cx)), __ldg(ls + (at + 1 + cx)));
+        const float* lq = pop(ls, q, qs);
+        if (cx == 0) l[q - 1] = __ldg(reinterpret_cast<const float2*>(lq + at));
+        else l[q - 1] = make_float2(__ldg(lq + (at + cx)), __ldg(lq + (at + 1 + cx)));
     }
     if constexpr (EDGE) {
         const bool wall = !in.periodic[0], lo = x == 0, hi0 = x == nx - 1, hi1 = x + 1 == nx - 1;
@@ -239,9 +241,10 @@ __device__ __forceinline__ void pull_lam_pair(const InstDesc& in, const float* _
         for (int q = 1; q < Q; ++q) {
             const int cx = L::c(q, 0);
             if (cx == 0) continue;
-            const int off = wall ? (L::opp(q) - 1) * qs + own + (cx < 0 ? 0 : nx - 1) : row_of(q) + (cx < 0 ? nx - 1 : 0);
+            const float* from = wall ? pop(ls, L::opp(q), qs) + (own + (cx < 0 ? 0 : nx - 1))
+                                     : pop(ls, q, qs) + (row_of(q) + (cx < 0 ? nx - 1 : 0));
             v[q] = 0.f;
-            if (cx < 0 ? lo : hi0 || hi1) v[q] = __ldg(ls + off);
+            if (cx < 0 ? lo : hi0 || hi1) v[q] = __ldg(from);
         }
 #pragma unroll
         for (int q = 1; q < Q; ++q) {
@@ -291,7 +294,7 @@ __global__ void __launch_bounds__(32 * ADJ_WARPS, Q == 9 ? ADJ_BLOCKS : 3) k_adj
     const int x0 = (local - rest * ntx) * tw, y0 = (rest % nty) * sh.ty, z0 = (rest / nty) * sh.tz;
     const int nx = in.n[0], ny = in.n[1], nz = in.n[2];
     const int pitch = in.pitch;
-    const int qs = (int)in.qstride;  // (Q - 1) * qstride < 2^31 (validated at creation)
+    const long long qs = in.qstride;
     const S* __restrict__ fin = static_cast<const S*>(af.fin);
     const float* __restrict__ lsrc = af.lam_src;
     float* __restrict__ ldst = af.lam_dst;
@@ -395,10 +398,10 @@ __global__ void __launch_bounds__(32 * ADJ_WARPS, Q == 9 ? ADJ_BLOCKS : 3) k_adj
         float* out = ldst + ((z * ny + y) * pitch + x);
         if (v1) {
 #pragma unroll
-            for (int q = 0; q < QS; ++q) *reinterpret_cast<float2*>(out + q * qs) = lam[q];
+            for (int q = 1; q < Q; ++q) *reinterpret_cast<float2*>(pop(out, q, qs)) = lam[q - 1];
         } else if (v0) {
 #pragma unroll
-            for (int q = 0; q < QS; ++q) out[q * qs] = lam[q].x;
+            for (int q = 1; q < Q; ++q) *pop(out, q, qs) = lam[q - 1].x;
         }
         // per-particle sums of the adjoint acceleration and alpha derivative
         if (!any) continue;
@@ -439,7 +442,7 @@ __global__ void k_adj_pull_out(const InstDesc* __restrict__ insts, int inst, con
     const int x = (int)(i % in.n[0]), y = (int)((i / in.n[0]) % in.n[1]),
               z = (int)(i / ((long long)in.n[0] * in.n[1]));
     float v[Q - 1];
-    pull_lam_all<Q>(in, lam, x, y, z, (int)in.qstride, v);
+    pull_lam_all<Q>(in, lam, x, y, z, in.qstride, v);
     out[i] = 0.f;
 #pragma unroll
     for (int q = 1; q < Q; ++q) out[(long long)q * N + i] = v[q - 1];

@@ -1053,14 +1053,23 @@ __device__ __forceinline__ double finalize_rotation(const long long* v, const do
     return Wo;
 }
 
-// Pre-collision population q (compile-time) at node (x, y, z) (Eq. 10, left
-// side): across a periodic face the source wraps; across a wall (the first
-// wall axis in the order x, y, z) the node's own opposite population bounces
-// back, plus the moving-wall term 2 w_q (c_q . u_w) / cs^2.  Selects instead of
-// branches, so that the lanes of a warp on a face stay together.
-template <int Q, class S, int q>
-__device__ __forceinline__ float pull_pre_any(const InstDesc& in, const S* __restrict__ fin, int x, int y, int z,
-                                              int qs) {
+// Population q of a buffer whose populations lie qs elements apart.  The whole
+// buffer of a D3Q19 box that lbm_create accepts can hold more than 2^31
+// elements (x rows are padded to 32 nodes: 100 x 1000 x 1000 has 18 qs = 2.3e9,
+// 2 x 7200 x 7200 3.0e10), so the base of a population is a 64-bit offset; one
+// population holds fewer (qs <= 1.7e9), so offsets within it are 32-bit.
+template <class P>
+__host__ __device__ __forceinline__ P* pop(P* f, int q, long long qs) { return f + (q - 1) * qs; }
+
+// Where population q (compile-time) of node (x, y, z) comes from (Eq. 10, left
+// side): offset off within population q, or across a wall (the first wall
+// axis in the order x, y, z: axis >= 0) within the opposite one, the node's own
+// that bounces back.  Across a periodic face the source wraps.
+struct PullSrc {
+    int off, axis, face;
+};
+template <int Q, int q>
+__host__ __device__ __forceinline__ PullSrc pull_source(const InstDesc& in, int x, int y, int z) {
     using L = Lat<Q>;
     constexpr int c[3] = {L::c(q, 0), L::c(q, 1), L::c(q, 2)};
     int src[3] = {x - c[0], y - c[1], z - c[2]};
@@ -1075,20 +1084,28 @@ __device__ __forceinline__ float pull_pre_any(const InstDesc& in, const S* __res
             face = src[d] < 0 ? 0 : 1;
         }
     }
-    const int node = (z * in.n[1] + y) * in.pitch + x;
-    const int off = axis >= 0 ? (L::opp(q) - 1) * qs + node
-                              : (q - 1) * qs + (src[2] * in.n[1] + src[1]) * in.pitch + src[0];
+    return PullSrc{axis >= 0 ? (z * in.n[1] + y) * in.pitch + x : (src[2] * in.n[1] + src[1]) * in.pitch + src[0], axis, face};
+}
+
+// Pre-collision population q at node (x, y, z): what it pulls, plus across a
+// wall the moving-wall term 2 w_q (c_q . u_w) / cs^2.  Selects instead of
+// branches, so that the lanes of a warp on a face stay together.
+template <int Q, class S, int q>
+__device__ __forceinline__ float pull_pre_any(const InstDesc& in, const S* __restrict__ fin, int x, int y, int z,
+                                              long long qs) {
+    const PullSrc s = pull_source<Q, q>(in, x, y, z);
     // the wall term is loaded whether it is needed or not: a load under a
     // condition would hold back the next population's (one memory latency each)
-    const float term = __ldg(&in.wterm[axis >= 0 ? axis : 0][face][q]);
-    const float v = VecIO<S, 1 + (sizeof(S) == 2)>::load1(fin + off, in.s_load);
-    return axis >= 0 ? v + term : v;
+    const float term = __ldg(&in.wterm[s.axis >= 0 ? s.axis : 0][s.face][q]);
+    const S* from = s.axis >= 0 ? pop(fin, Lat<Q>::opp(q), qs) : pop(fin, q, qs);
+    const float v = VecIO<S, 1 + (sizeof(S) == 2)>::load1(from + s.off, in.s_load);
+    return s.axis >= 0 ? v + term : v;
 }
 
 // All populations of a node by pull_pre_any (independent loads in flight).
 template <int Q, class S, int q = 1>
-__device__ __forceinline__ void pull_pre_all(const InstDesc& in, const S* __restrict__ fin, int x, int y, int z, int qs,
-                                             float* f) {
+__device__ __forceinline__ void pull_pre_all(const InstDesc& in, const S* __restrict__ fin, int x, int y, int z,
+                                             long long qs, float* f) {
     if constexpr (q < Q) {
         f[q - 1] = pull_pre_any<Q, S, q>(in, fin, x, y, z, qs);
         pull_pre_all<Q, S, q + 1>(in, fin, x, y, z, qs, f);
@@ -1118,15 +1135,17 @@ __device__ __forceinline__ float2 load_pair(const __half* p, float s) {
 template <int Q, class S, bool EDGE>
 __device__ __forceinline__ void pull_pair(const InstDesc& in, const S* __restrict__ fin, int x, int y, int z, float2* f) {
     using L = Lat<Q>;
-    const int nx = in.n[0], pitch = in.pitch, zs = in.n[1] * pitch, qs = (int)in.qstride;
+    const int nx = in.n[0], pitch = in.pitch, zs = in.n[1] * pitch;
+    const long long qs = in.qstride;
     const float sl = in.s_load;
     const int own = z * zs + y * pitch, xl = EDGE ? min(x, (nx - 1) & ~1) : x;
-    auto row_of = [&](int q) { return (q - 1) * qs + own - L::c(q, 2) * zs - L::c(q, 1) * pitch; };
+    auto row_of = [&](int q) { return own - L::c(q, 2) * zs - L::c(q, 1) * pitch; };  // within population q
 #pragma unroll
     for (int q = 1; q < Q; ++q) {
         const int cx = L::c(q, 0), at = row_of(q) + xl;
-        if (cx == 0) f[q - 1] = load_pair(fin + at, sl);
-        else f[q - 1] = make_float2(load_one(fin + (at - cx), sl), load_one(fin + (at + 1 - cx), sl));
+        const S* fq = pop(fin, q, qs);
+        if (cx == 0) f[q - 1] = load_pair(fq + at, sl);
+        else f[q - 1] = make_float2(load_one(fq + (at - cx), sl), load_one(fq + (at + 1 - cx), sl));
     }
     if constexpr (EDGE) {
         const bool wall = !in.periodic[0], lo = x == 0, hi0 = x == nx - 1, hi1 = x + 1 == nx - 1;
@@ -1135,9 +1154,10 @@ __device__ __forceinline__ void pull_pair(const InstDesc& in, const S* __restric
         for (int q = 1; q < Q; ++q) {
             const int cx = L::c(q, 0);
             if (cx == 0) continue;
-            const int off = wall ? (L::opp(q) - 1) * qs + own + (cx > 0 ? 0 : nx - 1) : row_of(q) + (cx > 0 ? nx - 1 : 0);
+            const S* from = wall ? pop(fin, L::opp(q), qs) + (own + (cx > 0 ? 0 : nx - 1))
+                                 : pop(fin, q, qs) + (row_of(q) + (cx > 0 ? nx - 1 : 0));
             v[q] = 0.f;
-            if (cx > 0 ? lo : hi0 || hi1) v[q] = load_one(fin + off, sl);
+            if (cx > 0 ? lo : hi0 || hi1) v[q] = load_one(from, sl);
             t[q] = __ldg(&in.wterm[0][cx > 0 ? 0 : 1][q]);
         }
 #pragma unroll

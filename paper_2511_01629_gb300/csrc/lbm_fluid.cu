@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(256, Q == 9 ? 4 : 2) k_fields(const InstDesc* 
     const int row = (int)(w / (unsigned)nseg);
     const int y = row % ny, z = row / ny;
     const long long N = (long long)nx * ny * nz;
-    const int qs = (int)in.qstride;  // (Q - 1) * qstride < 2^31 (validated at creation)
+    const long long qs = in.qstride;
     const S* __restrict__ fin = static_cast<const S*>(in.f[par]);
     const float sl = in.s_load;
     const bool row_in = y >= 1 && y + 1 < ny && (D == 2 || (z >= 1 && z + 1 < nz));
@@ -337,11 +337,11 @@ __global__ void __launch_bounds__(256, Q == 9 ? 4 : 2) k_fields(const InstDesc* 
         if (xc >= nx) break;
         const int x = min(xc + lane, nx - 1);  // lanes past the row read a valid node and write nothing
         if (row_in && xc >= 1 && xc + 32 < nx) {
-            const S* base = fin + (row * pitch + x);
+            const int at = row * pitch + x;
 #pragma unroll
             for (int q = 1; q < Q; ++q)
                 f[k][q - 1] = VecIO<S, 1 + (sizeof(S) == 2)>::load1(
-                    base + ((q - 1) * qs - (L::c(q, 2) * ny + L::c(q, 1)) * pitch - L::c(q, 0)), sl);
+                    pop(fin, q, qs) + (at - (L::c(q, 2) * ny + L::c(q, 1)) * pitch - L::c(q, 0)), sl);
         } else {
             pull_pre_all<Q, S>(in, fin, x, y, z, qs, f[k]);
         }

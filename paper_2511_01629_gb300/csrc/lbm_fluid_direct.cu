@@ -67,10 +67,10 @@ __global__ void __launch_bounds__(256, Q == 9 ? 4 : 3) k_fluid_direct(const Inst
             else pull_pair<Q, S, false>(in, fin, x, y, z, f);
         } else {
             float g[QS];
-            pull_pre_all<Q, S>(in, fin, min(x, nx - 1), y, z, (int)in.qstride, g);
+            pull_pre_all<Q, S>(in, fin, min(x, nx - 1), y, z, in.qstride, g);
 #pragma unroll
             for (int q = 0; q < QS; ++q) f[q].x = g[q];
-            pull_pre_all<Q, S>(in, fin, min(x + 1, nx - 1), y, z, (int)in.qstride, g);
+            pull_pre_all<Q, S>(in, fin, min(x + 1, nx - 1), y, z, in.qstride, g);
 #pragma unroll
             for (int q = 0; q < QS; ++q) f[q].y = g[q];
         }
