@@ -1087,39 +1087,39 @@ __host__ __device__ __forceinline__ PullSrc pull_source(const InstDesc& in, int 
     return PullSrc{axis >= 0 ? (z * in.n[1] + y) * in.pitch + x : (src[2] * in.n[1] + src[1]) * in.pitch + src[0], axis, face};
 }
 
+// One population value, or two of adjacent nodes, by plain (coherent) loads: the
+// fluid kernels may be resident while the step before writes them (dep_wait).
+__device__ __forceinline__ float load_one(const float* p, float) { return *p; }
+__device__ __forceinline__ float load_one(const __half* p, float s) { return __half2float(*p) * s; }
+__device__ __forceinline__ float2 load_pair(const float* p, float) { return *reinterpret_cast<const float2*>(p); }
+__device__ __forceinline__ float2 load_pair(const __half* p, float s) {
+    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(p));
+    return make_float2(a.x * s, a.y * s);
+}
+
 // Pre-collision population q at node (x, y, z): what it pulls, plus across a
 // wall the moving-wall term 2 w_q (c_q . u_w) / cs^2.  Selects instead of
 // branches, so that the lanes of a warp on a face stay together.
 template <int Q, class S, int q>
-__device__ __forceinline__ float pull_pre_any(const InstDesc& in, const S* __restrict__ fin, int x, int y, int z,
+__device__ __forceinline__ float pull_pre_any(const InstDesc& in, const S* fin, int x, int y, int z,
                                               long long qs) {
     const PullSrc s = pull_source<Q, q>(in, x, y, z);
     // the wall term is loaded whether it is needed or not: a load under a
     // condition would hold back the next population's (one memory latency each)
     const float term = __ldg(&in.wterm[s.axis >= 0 ? s.axis : 0][s.face][q]);
     const S* from = s.axis >= 0 ? pop(fin, Lat<Q>::opp(q), qs) : pop(fin, q, qs);
-    const float v = VecIO<S, 1 + (sizeof(S) == 2)>::load1(from + s.off, in.s_load);
+    const float v = load_one(from + s.off, in.s_load);
     return s.axis >= 0 ? v + term : v;
 }
 
 // All populations of a node by pull_pre_any (independent loads in flight).
 template <int Q, class S, int q = 1>
-__device__ __forceinline__ void pull_pre_all(const InstDesc& in, const S* __restrict__ fin, int x, int y, int z,
+__device__ __forceinline__ void pull_pre_all(const InstDesc& in, const S* fin, int x, int y, int z,
                                              long long qs, float* f) {
     if constexpr (q < Q) {
         f[q - 1] = pull_pre_any<Q, S, q>(in, fin, x, y, z, qs);
         pull_pre_all<Q, S, q + 1>(in, fin, x, y, z, qs, f);
     }
-}
-
-template <class S> __device__ __forceinline__ float load_one(const S* p, float s) {
-    return VecIO<S, 1 + (sizeof(S) == 2)>::load1(p, s);
-}
-__device__ __forceinline__ float2 load_pair(const float* p, float) { return __ldg(reinterpret_cast<const float2*>(p)); }
-__device__ __forceinline__ float2 load_pair(const __half* p, float s) {
-    const unsigned int t = __ldg(reinterpret_cast<const unsigned int*>(p));
-    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&t));
-    return make_float2(a.x * s, a.y * s);
 }
 
 // Populations of nodes x, x + 1 (x even) of a row whose y and z sources lie
@@ -1133,7 +1133,7 @@ __device__ __forceinline__ float2 load_pair(const __half* p, float s) {
 // 200 instructions a row (backward pass of 16 boxes of 400 x 1600: 19.7 -> 18.1
 // ms; the forward kernels, bound elsewhere, did not change).
 template <int Q, class S, bool EDGE>
-__device__ __forceinline__ void pull_pair(const InstDesc& in, const S* __restrict__ fin, int x, int y, int z, float2* f) {
+__device__ __forceinline__ void pull_pair(const InstDesc& in, const S* fin, int x, int y, int z, float2* f) {
     using L = Lat<Q>;
     const int nx = in.n[0], pitch = in.pitch, zs = in.n[1] * pitch;
     const long long qs = in.qstride;

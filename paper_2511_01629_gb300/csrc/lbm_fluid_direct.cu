@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(256, Q == 9 ? 4 : 3) k_fluid_direct(const Inst
     const int x = x0 + 2 * lane;
     const bool edge = x0 == 0 || x0 + TW >= nx;
     const float sload = in.s_load;
-    const S* __restrict__ fin = static_cast<const S*>(in.f[par]);
+    const S* fin = static_cast<const S*>(in.f[par]);
     float2 f[QS];
     dep_wait();  // the populations and lists of the previous step
     dep_launch();

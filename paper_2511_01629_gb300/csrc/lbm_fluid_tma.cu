@@ -296,6 +296,9 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
 
     if (warp == 0) {
         // ---------------------------------------------------------- producer
+        // the lists and populations were written by plain stores; the copies below
+        // read them through the async proxy
+        if (lane == 0) asm volatile("fence.proxy.async.global;" ::: "memory");
         // Tiles come from a work counter; claims alternate between the two
         // ends of the tile range (the slower y-face rows come first).  Two
         // claims are in flight, and everything the next tile needs from

@@ -299,13 +299,31 @@ __host__ __device__ inline int tile_w(const Shape& s) { return s.tw; }
 
 // Programmatic dependent launch of the kernels of a step: the next kernel's
 // blocks may start while the previous kernel runs, and wait (dep_wait) before
-// they touch anything it writes; what comes before the wait reads only
-// what no kernel of a step writes (descriptors, constants).  dep_launch lets the
-// next kernel start.  Saves the launch gap and the prologue: 1.1 to 1.5 us a step
+// they touch anything it writes.  Before the wait a kernel reads what no kernel
+// of a step writes (descriptors, constants), and the particle kernel also the
+// state that the previous step's particle kernel wrote: that one has ended
+// (the fluid kernel between them waited for it before it let this one start),
+// but what it wrote is promised only to a kernel that waits, so these
+// loads (ld_l2) go past L1 to where every ended kernel's stores are.  Populations
+// are read after the wait by plain loads, not through the read-only
+// path, which asks for data that nobody writes while the kernel is resident
+// (without particles the step before still writes them until the wait ends).
+// dep_launch lets the next kernel start.  Saves the launch gap and the prologue: 1.1 to 1.5 us a step
 // in graph replay (channel 100 x 200 14.6 -> 13.1 us, 500 disks FP32 62.6 -> 61.4).
 #ifdef __CUDACC__
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ double ld_l2(const double* p) {
+    double v;
+    asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(v) : "l"(__cvta_generic_to_global(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ float4 ld_l2(const float4* p) {
+    float4 v;
+    asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(__cvta_generic_to_global(p)) : "memory");
+    return v;
+}
 template <class... P, class... A>
 inline cudaError_t launch_dep(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
     cudaLaunchConfig_t cfg = {};

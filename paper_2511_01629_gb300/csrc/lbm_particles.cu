@@ -416,6 +416,12 @@ __device__ __forceinline__ LaneIn load_lane(const InstDesc& in, int i, int d, bo
     const long long j = 3LL * i + d;
     LaneIn L;
     const PState& ps = in.pst[par][i];
+    L.ec = ld_l2(&ps.ec);  // orientation theta^n of this step's record
+    L.es = ld_l2(&ps.es);
+    if (first) {
+        L.X0 = ld_l2(ps.X + d);
+        L.Ub = ld_l2(ps.U + d);  // U^{n-1} until project_lane
+    }
     const double* pc = in.pconst + PCONST_N * i;
     L.invrhos = pc[PC_INVRHOS];
     L.cw = pc[PC_CWALL];
@@ -423,12 +429,8 @@ __device__ __forceinline__ LaneIn load_lane(const InstDesc& in, int i, int d, bo
     L.Ri = pc[PC_R];
     L.Bi = pc[PC_B];
     L.gfac = pc[PC_GFAC];
-    L.ec = ps.ec;  // orientation theta^n of this step's record
-    L.es = ps.es;
     L.rc = in.rconst[i];
     if (first) {
-        L.X0 = ps.X[d];
-        L.Ub = ps.U[d];  // U^{n-1} until project_lane
         L.Acor = 0.0;
     } else {
         L.X0 = in.Xk[(long long)src * in.np * 3 + j];
@@ -655,7 +657,8 @@ __device__ bool grid_sync(GridBar* gb, int* status, unsigned long long limit_ns)
 // warp 1 the rotation, and warp 2 clears the totals that the next step adds to.
 // The first phase runs up to its wait beside the fluid kernel: that kernel lets
 // this one start once the previous step's particle kernel has ended, so all but
-// the totals is there (state, positions, the pairs that may be in range).
+// the totals is there (state, positions, the pairs that may be in range; read
+// by ld_l2).
 template <bool FIRST>
 __device__ __forceinline__ void phase_substep(const InstDesc& in, int i0, int D, int src, int par, int last, const Shape& sh,
                               float4* xs, float4* xs2, double (*sF)[6], AxisTiles (*sAT)[3], Cand* sC) {
@@ -670,8 +673,8 @@ __device__ __forceinline__ void phase_substep(const InstDesc& in, int i0, int D,
     double th = 0.0, wo = 0.0;
     if (warp == 0) li = load_lane(in, i0 + usl, ud, uvalid, src, par, FIRST);
     if (warp == 1 && uvalid) {
-        th = in.theta[3 * (i0 + usl) + ud];
-        wo = in.W[3 * (i0 + usl) + ud];
+        th = ld_l2(in.theta + 3 * (i0 + usl) + ud);
+        wo = ld_l2(in.W + 3 * (i0 + usl) + ud);
     }
     const bool pairs = in.np > 1;  // one particle: nothing to search
     const bool one = in.np <= XCHUNK;
@@ -689,7 +692,7 @@ __device__ __forceinline__ void phase_substep(const InstDesc& in, int i0, int D,
         for (int u = 0; u < PER; ++u) {
             const int k = threadIdx.x + 256 * u;
             if (k < nj) {
-                ra[u] = Xfb[j0 + k];
+                ra[u] = FIRST ? ld_l2(Xfb + j0 + k) : Xfb[j0 + k];
                 if (!FIRST) rb[u] = Xsb[j0 + k];
             }
         }
@@ -708,7 +711,7 @@ __device__ __forceinline__ void phase_substep(const InstDesc& in, int i0, int D,
     unsigned m = 0;
     if (pairs) {
         if (mine) {  // issued before the staging barrier, so the loads overlap it
-            xi = Xfb[i];
+            xi = FIRST ? ld_l2(Xfb + i) : Xfb[i];
             if (!FIRST) xi2 = Xsb[i];
             cp = in.pconst[PCONST_N * i + PC_CPAIR];
             idl = in.pconst[PCONST_N * i + PC_INVDELTA];
