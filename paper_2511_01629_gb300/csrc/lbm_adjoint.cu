@@ -236,13 +236,14 @@ __device__ __forceinline__ void pull_lam_pair(const InstDesc& in, const float* _
     }
     if constexpr (EDGE) {
         const bool wall = !in.periodic[0], lo = x == 0, hi0 = x == nx - 1, hi1 = x + 1 == nx - 1;
+        const long long wq = wall ? qs : 0;  // see pull_pair
         float v[Q];
 #pragma unroll
         for (int q = 1; q < Q; ++q) {
             const int cx = L::c(q, 0);
             if (cx == 0) continue;
-            const float* from = wall ? pop(ls, L::opp(q), qs) + (own + (cx < 0 ? 0 : nx - 1))
-                                     : pop(ls, q, qs) + (row_of(q) + (cx < 0 ? nx - 1 : 0));
+            const float* from = pop(ls, q, qs) + (L::opp(q) - q) * wq +
+                                (wall ? own + (cx < 0 ? 0 : nx - 1) : row_of(q) + (cx < 0 ? nx - 1 : 0));
             v[q] = 0.f;
             if (cx < 0 ? lo : hi0 || hi1) v[q] = __ldg(from);
         }

@@ -1140,22 +1140,26 @@ __device__ __forceinline__ void pull_pair(const InstDesc& in, const S* fin, int 
     const float sl = in.s_load;
     const int own = z * zs + y * pitch, xl = EDGE ? min(x, (nx - 1) & ~1) : x;
     auto row_of = [&](int q) { return own - L::c(q, 2) * zs - L::c(q, 1) * pitch; };  // within population q
+    const S* fq = fin + (own + xl);
 #pragma unroll
-    for (int q = 1; q < Q; ++q) {
-        const int cx = L::c(q, 0), at = row_of(q) + xl;
-        const S* fq = pop(fin, q, qs);
-        if (cx == 0) f[q - 1] = load_pair(fq + at, sl);
-        else f[q - 1] = make_float2(load_one(fq + (at - cx), sl), load_one(fq + (at + 1 - cx), sl));
+    for (int q = 1; q < Q; ++q, fq += qs) {
+        const int cx = L::c(q, 0), sh = -L::c(q, 2) * zs - L::c(q, 1) * pitch;
+        if (cx == 0) f[q - 1] = load_pair(fq + sh, sl);
+        else f[q - 1] = make_float2(load_one(fq + sh - cx, sl), load_one(fq + sh + (1 - cx), sl));
     }
     if constexpr (EDGE) {
         const bool wall = !in.periodic[0], lo = x == 0, hi0 = x == nx - 1, hi1 = x + 1 == nx - 1;
+        // at a wall population opp(q) = q + (opp - q): one 64-bit select for all of them.
+        // Selecting each pointer cost 256 x 256 x 512 FP16 656 us a step, this 620 (616
+        // with 32-bit addresses, which do not reach all of a large box)
+        const long long wq = wall ? qs : 0;
         float v[Q], t[Q];
 #pragma unroll
         for (int q = 1; q < Q; ++q) {
             const int cx = L::c(q, 0);
             if (cx == 0) continue;
-            const S* from = wall ? pop(fin, L::opp(q), qs) + (own + (cx > 0 ? 0 : nx - 1))
-                                 : pop(fin, q, qs) + (row_of(q) + (cx > 0 ? nx - 1 : 0));
+            const S* from = pop(fin, q, qs) + (L::opp(q) - q) * wq +
+                            (wall ? own + (cx > 0 ? 0 : nx - 1) : row_of(q) + (cx > 0 ? nx - 1 : 0));
             v[q] = 0.f;
             if (cx > 0 ? lo : hi0 || hi1) v[q] = load_one(from, sl);
             t[q] = __ldg(&in.wterm[0][cx > 0 ? 0 : 1][q]);
