@@ -140,8 +140,10 @@ __global__ void __launch_bounds__(NA_BLOCK) k_na_accumulate(NaGrid g, const floa
     if (ok_radius) {
         const float xf[3] = {(float)Xp[0], (float)Xp[1], (float)Xp[2]};
         for (int j = threadIdx.x; j < p; j += NA_BLOCK) {
-            // FP32 first: coordinates below 2^20 carry an error below 0.1, so a
-            // pair 1 beyond reach along a non-periodic axis cannot overlap
+            // FP32 first: on an axis of up to 2^20 nodes the coordinates of two
+            // particles that share a node carry an error below 0.1 each, so a pair 1
+            // beyond reach along a non-periodic axis cannot overlap.  Longer axes
+            // (from 2^25 nodes the error exceeds the margin) leave it to FP64 below.
             const double Rj = R[j];
             const float reachf = (float)Rj + (float)Rp + 3.0f;
             bool far = false;
@@ -149,7 +151,7 @@ __global__ void __launch_bounds__(NA_BLOCK) k_na_accumulate(NaGrid g, const floa
 #pragma unroll
             for (int d = 0; d < D; ++d) {
                 Xj[d] = X[j * D + d];
-                far |= !g.per[d] && fabsf((float)Xj[d] - xf[d]) > reachf;
+                far |= !g.per[d] && g.n[d] <= (1 << 20) && fabsf((float)Xj[d] - xf[d]) > reachf;
             }
             if (far) continue;
             double d2 = 0.0;
