@@ -24,6 +24,7 @@
 // returns.
 #include <cuda.h>
 
+#include <mutex>
 #include <type_traits>
 
 #include "lbm_common.cuh"
@@ -644,12 +645,20 @@ bool tma_rows_ok(int rows) { return rows == 4 || rows == 8; }
 template <int Q, class S, int TW, int ROWS>
 static int tma_blocks_t(const Shape& sh, int stages, int ninst) {
     const TmaLayout LY = tma_layout(Q, (int)sizeof(S), TW, ROWS, stages, ninst);
-    if (cudaFuncSetAttribute(k_fluid_tma<Q, S, TW, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             LY.bytes) != cudaSuccess)
-        return 0;
+    auto* const kern = k_fluid_tma<Q, S, TW, ROWS>;
+    {
+        // the limit belongs to the kernel, not to a context: only raised, so that a
+        // context with fewer instances or stages leaves the others' launches valid
+        static std::mutex m;
+        std::lock_guard<std::mutex> lock(m);
+        cudaFuncAttributes at;
+        if (cudaFuncGetAttributes(&at, kern) != cudaSuccess) return 0;
+        if (at.maxDynamicSharedSizeBytes < LY.bytes &&
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, LY.bytes) != cudaSuccess)
+            return 0;
+    }
     int nb = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_fluid_tma<Q, S, TW, ROWS>, 32 * (sh.warps + 1),
-                                                  LY.bytes);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, 32 * (sh.warps + 1), LY.bytes);
     return nb;
 }
 
