@@ -204,15 +204,19 @@ int lbm_set_graphs(lbm_ctx* ctx, int steps_per_graph); /* 0 = plain launches */
 /* Time each fluid-kernel shape on the current state and keep the fastest.
  * The state is not changed.  reps: timed launches per shape. */
 int lbm_autotune(lbm_ctx* ctx, int reps);
-/* Fluid-kernel shape.  vec = 0 is the default path: for D2Q9 the TMA-staged pipeline (one producer warp
- * filling a ring of shared-memory stages by tensor copies, `warps` consumer
- * warps, tile rows 4 or 8); vec = 1/2/4 (FP32) or 2/4/8 (FP16) is the
- * register path with vec nodes per thread and `warps` warps per block.
- * A new context starts in the TMA pipeline with a 2-stage ring: D2Q9 FP32
- * with 8 rows and 8 warps, D2Q9 FP16 and D3Q19 with 4 rows and 4 warps.
- * lbm_set_kernel_shape keeps the current ring depth; lbm_autotune may change
- * it.  D3Q19 has no staged pipeline: there vec = 0 is the direct kernel (one
- * warp per 64-node row, loads straight into registers) over the same tiles. */
+/* Fluid-kernel shape: what lbm_kernel_shape reports, lbm_set_kernel_shape takes.
+ *   vec = 0   D2Q9: the TMA-staged pipeline (one producer warp filling a ring of
+ *             shared-memory stages by tensor copies, `warps` consumer warps, tiles of
+ *             4 or 8 rows); D3Q19: the direct kernel (one warp per 64-node row,
+ *             loads straight into registers, tiles of 4 or 8 rows);
+ *   vec = -1  D2Q9 only: the direct kernel (as vec = 0 of D3Q19);
+ *   vec = 1/2/4 (FP32) or 2/4/8 (FP16): the register path with vec nodes per
+ *             thread and `warps` warps per block.
+ * A new context starts, D2Q9, in the direct kernel with 4 rows and 4 warps when its
+ * instances hold at most 2^18 nodes together, and otherwise in the staged
+ * pipeline with a 2-stage ring (FP32 8 rows and 8 warps, FP16 4 and 4); D3Q19 in
+ * the direct kernel with 4 rows and 4 warps.  A change of shape within the
+ * staged pipeline keeps the ring depth; lbm_autotune may change it. */
 int lbm_kernel_shape(const lbm_ctx* ctx, int* vec, int* tile_rows, int* warps);
 int lbm_set_kernel_shape(lbm_ctx* ctx, int vec, int tile_rows, int warps);
 /* Bound on each wait of the particle kernel at its grid-wide barrier between

@@ -1246,7 +1246,8 @@ int lbm_set_particle_wait_limit(lbm_ctx* ctx, double seconds) {
 
 int lbm_kernel_shape(const lbm_ctx* ctx, int* vec, int* tile_rows, int* warps) {
     if (!ctx) return LBM_ERR_INVALID;
-    if (vec) *vec = ctx->shape.tma ? 0 : ctx->shape.vec;
+    // -1: the direct kernel where the staged one is the other choice (D2Q9)
+    if (vec) *vec = !ctx->shape.tma ? ctx->shape.vec : ctx->D == 2 && ctx->shape.stages == 0 ? -1 : 0;
     if (tile_rows) *tile_rows = ctx->shape.ty * ctx->shape.tz;
     if (warps) *warps = ctx->shape.warps;
     return LBM_OK;
@@ -1259,13 +1260,18 @@ static bool shape_ok(const lbm_ctx* ctx, int vec) {
 int lbm_set_kernel_shape(lbm_ctx* ctx, int vec, int tile_rows, int warps) {
     int rc = check_ctx(ctx);
     if (rc) return rc;
-    if ((vec != 0 && !shape_ok(ctx, vec)) || tile_rows < 1 || tile_rows > 64 || warps < 1 || warps > 8)
+    const bool direct2d = vec == -1 && ctx->D == 2;
+    if ((vec != 0 && !direct2d && !shape_ok(ctx, vec)) || tile_rows < 1 || tile_rows > 64 || warps < 1 || warps > 8)
         return set_err(ctx, LBM_ERR_INVALID, "unsupported kernel shape%s");
+    int now[3];
+    lbm_kernel_shape(ctx, now, now + 1, now + 2);
+    if (vec == now[0] && tile_rows == now[1] && warps == now[2]) return LBM_OK;
     Shape s = ctx->shape;
-    s.tma = vec == 0;
-    if (vec) s.vec = vec;
+    s.tma = vec <= 0;
+    if (vec > 0) s.vec = vec;
     s.warps = warps;
-    if (s.tma && ctx->D == 2 && s.stages == 0) s.stages = 2;
+    if (direct2d) s.stages = 0;
+    else if (s.tma && ctx->D == 2 && s.stages == 0) s.stages = 2;
     if (s.tma && !tma_rows_ok(tile_rows))
         return set_err(ctx, LBM_ERR_INVALID, "TMA tiles hold 4 or 8 rows%s");
     if (ctx->D == 2) {

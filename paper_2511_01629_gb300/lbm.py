@@ -345,6 +345,9 @@ class LBM:
         self._check(lib().lbm_autotune(self._h, int(reps)))
 
     def kernel_shape(self):
+        """(vec, tile rows, warps) of the fluid kernel, as set_kernel_shape takes
+        them: vec 0 is the staged kernel (D3Q19: the direct one), -1 the direct
+        kernel of D2Q9, others the register path."""
         v, r, w = C.c_int(), C.c_int(), C.c_int()
         lib().lbm_kernel_shape(self._h, C.byref(v), C.byref(r), C.byref(w))
         return v.value, r.value, w.value
