@@ -760,13 +760,13 @@ __global__ void __launch_bounds__(256) k_adj_state(const InstDesc* __restrict__ 
 // ------------------------------------------------------------- launchers --
 cudaError_t launch_adj_fluid(int Q, int fp16, const InstDesc* insts, const AdjFluid* afs,
                              const uint16_t* tile_inst, int ninst, int ntiles, int lam_mode, const Shape& sh,
-                             cudaStream_t st) {
+                             int num_sms, cudaStream_t st) {
     const int units = sh.ty * sh.tz * ((sh.tw + 63) / 64), per = (units + ADJ_WARPS - 1) / ADJ_WARPS;
     // With few tiles every segment goes to a warp of its own; with two waves of
     // tiles or more one block takes a whole tile and starts up once (backward pass,
     // 1 / 2 / 4 blocks per tile: one 400 x 1600 box, 240 steps 13.4 / 12.2 / 11.9 ms;
     // 16 of them, 48 steps 19.7 / 20.7 / 22.9 ms).
-    const bool many = ntiles >= 2 * ADJ_BLOCKS * 152;
+    const bool many = ntiles >= 2 * ADJ_BLOCKS * num_sms;
     const dim3 grid((unsigned)ntiles, many ? 1u : (unsigned)per);
     auto go = [&](auto kern) { kern<<<grid, 32 * ADJ_WARPS, 0, st>>>(insts, afs, tile_inst, ninst, lam_mode, sh); };
     if (Q == 9) {

@@ -27,16 +27,16 @@ cudaError_t launch_pack(int Q, int fp16, const InstDesc* insts, int inst, long l
                         const float* src, cudaStream_t st);
 cudaError_t launch_unpack(int Q, int fp16, const InstDesc* insts, int inst, long long N, int par,
                           float* dst, cudaStream_t st);
-int particle_blocks_resident(int num_sms);
+int particle_blocks_resident(int D, int num_sms);
 cudaError_t launch_particles(const InstDesc* insts, const PartRef* refs, int ntotal, int ninst, int D, int K,
                              int lpar, const Shape& sh, GridBar* gb, bool fused, cudaStream_t st,
                              long long wait_ns);
 cudaError_t launch_publish(const InstDesc* insts, const PartRef* refs, int ntotal, int D, int lpar,
                            const Shape& sh, cudaStream_t st);
-int tma_tile_width(int Q);
+int tma_tile_width();
 bool tma_rows_ok(int rows);
-int fluid_tma_blocks_per_sm(int Q, int fp16, const Shape& sh, int stages, int ninst);
-cudaError_t launch_fluid_tma(int Q, int fp16, const InstDesc* insts, const void* tmaps,
+int fluid_tma_blocks_per_sm(int fp16, const Shape& sh, int stages, int ninst);
+cudaError_t launch_fluid_tma(int fp16, const InstDesc* insts, const void* tmaps,
                              const uint16_t* tile_inst, int ntiles, int par, const Shape& sh,
                              int commit, int grid, int* tile_ctr, int stages, int ninst, cudaStream_t st);
 int direct_tile_width();
@@ -45,7 +45,7 @@ cudaError_t launch_fluid_direct(int Q, int fp16, const InstDesc* insts, const ui
                                 int par, const Shape& sh, int commit, cudaStream_t st);
 cudaError_t launch_adj_fluid(int Q, int fp16, const InstDesc* insts, const AdjFluid* afs,
                              const uint16_t* tile_inst, int ninst, int ntiles, int lam_mode, const Shape& sh,
-                             cudaStream_t st);
+                             int num_sms, cudaStream_t st);
 cudaError_t launch_adj_particles(int D, const InstDesc* insts, const AdjPart* steps, const AdjBufs* bufs,
                                  int ninst, cudaStream_t st);
 cudaError_t launch_adj_finish(const InstDesc* insts, const AdjBufs* bufs, const long long* out_off,
@@ -268,7 +268,6 @@ InstDesc make_desc(lbm_ctx* ctx, const Instance& I) {
     d.tile0 = I.tile0;
     d.np = I.np;
     d.maxk = I.maxk;
-    d.tau_inv = (float)(1.0 / c.tau);
     d.keep = (float)(1.0 - 1.0 / c.tau);
     d.fpref = (float)(1.0 - 1.0 / (2.0 * c.tau));
     d.alpha = (float)c.alpha;
@@ -501,7 +500,7 @@ bool staged(const Shape& sh) { return sh.tma && sh.stages > 0; }
 int configure_shape(lbm_ctx* ctx, const Shape& sh_in) {
     Shape sh = sh_in;
     if (ctx->D == 2) sh.tz = 1;
-    sh.tw = !sh.tma ? 32 * sh.vec : staged(sh) ? tma_tile_width(ctx->Q) : direct_tile_width();
+    sh.tw = !sh.tma ? 32 * sh.vec : staged(sh) ? tma_tile_width() : direct_tile_width();
     ctx->shape = sh;
     const int T[3] = {sh.tw, sh.ty, sh.tz};
     int tile0 = 0;
@@ -531,7 +530,7 @@ int configure_shape(lbm_ctx* ctx, const Shape& sh_in) {
                        cudaMemcpyHostToDevice, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));
     const int occ = !sh.tma ? fluid_max_blocks_per_sm(ctx->Q, ctx->fp16, sh)
-                    : staged(sh) ? fluid_tma_blocks_per_sm(ctx->Q, ctx->fp16, sh, sh.stages, (int)ctx->inst.size())
+                    : staged(sh) ? fluid_tma_blocks_per_sm(ctx->fp16, sh, sh.stages, (int)ctx->inst.size())
                                  : fluid_direct_blocks_per_sm(ctx->Q, ctx->fp16, sh);
     if (occ < 1) return set_err(ctx, LBM_ERR_INVALID, "kernel shape does not fit on an SM%s");
     ctx->grid = occ * ctx->num_sms;
@@ -561,7 +560,7 @@ Shape default_shape(int Q, int fp16, long long nodes) {
 int enqueue_fluid_on(lbm_ctx* ctx, const InstDesc* insts, const void* tmaps, int par, int commit, cudaStream_t st) {
     const Shape& sh = ctx->shape;
     if (staged(sh))
-        CK(launch_fluid_tma(ctx->Q, ctx->fp16, insts, tmaps, P<uint16_t>(ctx->d_tile_inst), ctx->ntiles, par, sh, commit,
+        CK(launch_fluid_tma(ctx->fp16, insts, tmaps, P<uint16_t>(ctx->d_tile_inst), ctx->ntiles, par, sh, commit,
                             ctx->grid, P<int>(ctx->d_tile_ctr), sh.stages, (int)ctx->inst.size(), st));
     else if (sh.tma)
         CK(launch_fluid_direct(ctx->Q, ctx->fp16, insts, P<uint16_t>(ctx->d_tile_inst), (int)ctx->inst.size(), ctx->ntiles,
@@ -582,7 +581,7 @@ int enqueue_step(lbm_ctx* ctx, cudaStream_t st) {
     if (rc) return rc;
     if (ctx->np_total > 0) {
         const int K = ctx->inst[0].cfg.K;
-        const bool fused = (ctx->np_total + 7) / 8 <= particle_blocks_resident(ctx->num_sms);
+        const bool fused = (ctx->np_total + 7) / 8 <= particle_blocks_resident(ctx->D, ctx->num_sms);
         CK(launch_particles(P<InstDesc>(ctx->d_insts), P<PartRef>(ctx->d_refs), ctx->np_total,
                             (int)ctx->inst.size(), ctx->D, K, ctx->par ^ 1, ctx->shape, P<GridBar>(ctx->d_gridbar), fused, st,
                             ctx->wait_ns));
@@ -978,7 +977,7 @@ int lbm_step_timed(lbm_ctx* ctx, int nsteps, float* ms_fluid, float* ms_box, flo
         // events' own interval
         if (rc == LBM_OK && e == cudaSuccess) e = cudaEventRecord(q[2], ctx->st);
         if (parts && rc == LBM_OK && e == cudaSuccess) {
-            const bool fused = (ctx->np_total + 7) / 8 <= particle_blocks_resident(ctx->num_sms);
+            const bool fused = (ctx->np_total + 7) / 8 <= particle_blocks_resident(ctx->D, ctx->num_sms);
             e = launch_particles(P<InstDesc>(ctx->d_insts), P<PartRef>(ctx->d_refs), ctx->np_total,
                                  (int)ctx->inst.size(), ctx->D, ctx->inst[0].cfg.K, ctx->par ^ 1, ctx->shape, P<GridBar>(ctx->d_gridbar), fused,
                                  ctx->st, ctx->wait_ns);
@@ -1362,7 +1361,7 @@ int lbm_autotune(lbm_ctx* ctx, int reps) {
 int lbm_launches_per_step(const lbm_ctx* ctx) {
     if (!ctx) return 0;
     if (ctx->np_total == 0) return 1;
-    const bool fused = (ctx->np_total + 7) / 8 <= particle_blocks_resident(ctx->num_sms);
+    const bool fused = (ctx->np_total + 7) / 8 <= particle_blocks_resident(ctx->D, ctx->num_sms);
     return 1 + (fused ? 1 : ctx->inst[0].cfg.K);  // fluid, particles
 }
 
@@ -1627,7 +1626,7 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
     }
     const InstDesc* dI = P<InstDesc>(ctx->d_insts);
     const InstDesc* dR = P<InstDesc>(A.d_rdesc);
-    const bool fused = (ctx->np_total + 7) / 8 <= particle_blocks_resident(ctx->num_sms);
+    const bool fused = (ctx->np_total + 7) / 8 <= particle_blocks_resident(ctx->D, ctx->num_sms);
     // recomputation of a segment of len steps into the slots and records, then
     // the backward sweep through it (k = len - 1 .. 0); last: the segment holds
     // the final step of the run, whose adjoint comes from the seed
@@ -1648,7 +1647,7 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* seed_particles, const float
             const bool final_step = last && k == len - 1;
             const int mode = final_step ? (seed_field ? 1 : 2) : 0;
             CK(launch_adj_fluid(ctx->Q, ctx->fp16, dI, P<AdjFluid>(A.d_afl) + (size_t)(final_step ? L : k) * ni,
-                                P<uint16_t>(ctx->d_tile_inst), ni, ctx->ntiles, mode, sh, st));
+                                P<uint16_t>(ctx->d_tile_inst), ni, ctx->ntiles, mode, sh, ctx->num_sms, st));
         }
         return LBM_OK;
     };

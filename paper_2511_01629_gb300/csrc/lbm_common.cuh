@@ -531,20 +531,6 @@ __device__ __forceinline__ void moments2(const float2* f, float2& s, float2* m) 
     }
 }
 
-// Scalar moments (the adjoint's forward recomputation): the same sums.
-template <int Q>
-__device__ __forceinline__ void moments(const float* f, float& s, float* m) {
-    float2 f2v[Q - 1];
-#pragma unroll
-    for (int q = 0; q < Q - 1; ++q) f2v[q] = bc2(f[q]);
-    float2 s2, m2[3];
-    moments2<Q>(f2v, s2, m2);
-    s = s2.x;
-    m[0] = m2[0].x;
-    m[1] = m2[1].x;
-    m[2] = m2[2].x;
-}
-
 // Two nodes: f holds the stored populations q = 1..Q-1 (index q-1) after
 // streaming; on return it holds f*.  u and p of Eq. 15 are returned.  solid
 // flags the halves on which the penalty acts.
@@ -686,24 +672,6 @@ __device__ __forceinline__ void collide2_t1_scaled(float2* f, const float2* a, b
     } else {
         collide_pair2_t1<Q, 1, false>(f, u, a, base, nua, ks, nullptr, bc2(0.f), false, false);
     }
-}
-
-// One node (both halves of the packed arithmetic carry it): the same bits
-// as collide2 gives that node.
-template <int Q>
-__device__ __forceinline__ void collide(float* f, const float* a, bool solid, const CollK& k, float* u_out,
-                                        float* p_out) {
-    float2 f2v[Q - 1], a2[3], u2[3], p2;
-#pragma unroll
-    for (int q = 0; q < Q - 1; ++q) f2v[q] = bc2(f[q]);
-#pragma unroll
-    for (int d = 0; d < 3; ++d) a2[d] = bc2(a[d]);
-    collide2<Q>(f2v, a2, solid, solid, k, u2, &p2);
-#pragma unroll
-    for (int q = 0; q < Q - 1; ++q) f[q] = f2v[q].x;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) u_out[d] = u2[d].x;
-    *p_out = p2.x;
 }
 
 // Fixed-point image round(u * 2^FXBITS) of a velocity component (ties to even),

@@ -15,9 +15,9 @@
 // mbarrier; each consumer lane pulls two adjacent nodes' populations from
 // shared memory at x - c_x, collides them with packed FP32x2 arithmetic,
 // stores them to HBM with 8-byte coalesced stores, and adds the velocities
-// of solid nodes to their particle's sums of Eq. 22.  Rows whose source lies beyond a y or z face
-// gather those populations from HBM directly, as the register-path kernel
-// does.
+// of solid nodes to their particle's sums of Eq. 22.  At a y wall a node's own
+// opposite populations, staged too, come back; the rows at a periodic y face
+// gather theirs from the previous buffer directly.
 //
 // Every mbarrier wait is bounded in time; on expiry the kernel records a
 // timeout in the status word, waits (bounded) for the copies it issued and
@@ -99,6 +99,11 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
+constexpr int Q = 9;  // D3Q19 takes k_fluid_direct
+using L = Lat<Q>;
+// Populations with c_x = +1 (equally, -1): the ones an x-edge node pulls
+// across its face.
+__host__ __device__ constexpr int edge_pops() { return 3; }
 constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;  // 2 s
 
 // The constants of one instance that a tile needs, copied once per block
@@ -112,17 +117,16 @@ struct __align__(16) TInst {
     int* lcnt[2];              // tile list counts per parity
     const Cand* lrec[2];       // candidate records per parity
     long long qstride;
-    int tile0, ntx, nty, pitch, np, maxk;
+    int tile0, ntx, pitch, np;
     int n[3], per[3];
     float gdrive[3], sload, sstore, keep, fpref, alpha;
     int free;                  // no body force: fluid nodes take collide2_free
-    float ewt[2][5];           // moving-wall term of the populations an x-edge node pulls
+    float ewt[2][edge_pops()];  // moving-wall term of the populations an x-edge node pulls
                                //   across the low (0) / high (1) x face
 };
 constexpr int TI_MAX = 64;
 constexpr int TI_WORDS = (int)(sizeof(TInst) / 16);
 
-template <int Q>
 __device__ __forceinline__ void make_tinst(TInst& t, const InstDesc& in) {
     for (int b = 0; b < 2; ++b) {
         t.f[b] = in.f[b];
@@ -137,10 +141,8 @@ __device__ __forceinline__ void make_tinst(TInst& t, const InstDesc& in) {
     t.qstride = in.qstride;
     t.tile0 = in.tile0;
     t.ntx = in.ntile[0];
-    t.nty = in.ntile[1];
     t.pitch = in.pitch;
     t.np = in.np;
-    t.maxk = in.maxk;
     for (int d = 0; d < 3; ++d) {
         t.n[d] = in.n[d];
         t.per[d] = in.periodic[d];
@@ -153,11 +155,11 @@ __device__ __forceinline__ void make_tinst(TInst& t, const InstDesc& in) {
     t.alpha = in.alpha;
     t.free = in.gdrive[0] == 0.f && in.gdrive[1] == 0.f && in.gdrive[2] == 0.f;
     for (int face = 0; face < 2; ++face)
-        for (int k = 0; k < 5; ++k) t.ewt[face][k] = 0.f;
+        for (int k = 0; k < edge_pops(); ++k) t.ewt[face][k] = 0.f;
     for (int face = 0; face < 2; ++face) {  // face 0 is pulled across by c_x = +1, face 1 by c_x = -1
         const int ecx = face == 0 ? 1 : -1;
         for (int k = 0, q = 1; q < Q; ++q)
-            if (Lat<Q>::c(q, 0) == ecx) t.ewt[face][k++] = in.wterm[0][face][q];
+            if (L::c(q, 0) == ecx) t.ewt[face][k++] = in.wterm[0][face][q];
     }
 }
 
@@ -178,7 +180,7 @@ struct __align__(16) StageHdr {
     int tile;   // global tile index, -1 = no more work
     int ncand;
     int inst;
-    int x0, y0, z0;
+    int x0, y0;
     int ex;     // bit 0: the tile holds x = 0, bit 1: it holds x = nx - 1 (the values
                 //   these nodes pull across the face are staged, side by side)
 };
@@ -187,9 +189,9 @@ struct __align__(16) StageHdr {
 // registers; its list count and the values its x-edge nodes pull across the
 // faces in flight to the shared prefetch buffer (cp.async) while the producer
 // waits for a free stage.
-constexpr int EDGE_ITERS = 3;  // edge values per lane: 2 sides x 8 rows x 5 populations at most
+constexpr int EDGE_ITERS = 2;  // edge values per lane: 2 sides x 8 rows x 3 populations at most
 struct TileAhead {
-    int t, ii, local, x0, y0, z0, ex, np;
+    int t, ii, local, x0, y0, ex, np;
     float sload;
     float add[EDGE_ITERS];
     int hsel;  // FP16: bit j set = value j is the upper half of its 4-byte word
@@ -202,33 +204,23 @@ constexpr int PRE_CNT = 32 * EDGE_ITERS;
 // Geometry of the shared-memory ring, identical on host and device.
 struct TmaLayout {
     int bw;          // box width (nodes) = tile width + 2 halo
-    int slab;        // bytes of one population box, rounded to 128
     int stage;       // bytes of all populations of one stage
     int pops_bytes;  // stages * stage
     int hdr_off, cand_off, edge_off, tab_off, pre_off, bar_off, bytes;
 };
 
-// Populations with c_x = +1 (equally, -1): the ones an x-edge node pulls
-// across its face.
-__host__ __device__ constexpr int edge_pops(int Q) { return Q == 9 ? 3 : 5; }
-
-__host__ __device__ inline TmaLayout tma_layout(int Q, int ssize, int tw, int rows, int stages, int ninst) {
+__host__ __device__ inline TmaLayout tma_layout(int ssize, int tw, int rows, int stages, int ninst) {
     TmaLayout L;
     const int halo = 16 / ssize;
     const int ntab = ninst < TI_MAX ? ninst : TI_MAX;
     L.bw = tw + 2 * halo;
-    if (Q == 9) {  // one box per tile: all populations, rows y0 - 1 .. y0 + rows, densely packed
-        L.slab = L.bw * (rows + 2) * ssize;
-        L.stage = ((Q - 1) * L.slab + 127) & ~127;
-    } else {       // one box per population, rows y0 - c_y .., each slab 128-byte aligned
-        L.slab = ((L.bw * rows * ssize) + 127) & ~127;
-        L.stage = (Q - 1) * L.slab;
-    }
+    // one box per tile: all populations, rows y0 - 1 .. y0 + rows, densely packed
+    L.stage = ((Q - 1) * L.bw * (rows + 2) * ssize + 127) & ~127;
     L.pops_bytes = stages * L.stage;
     L.hdr_off = L.pops_bytes;
     L.cand_off = L.hdr_off + (int)sizeof(StageHdr) * stages;  // 16-byte aligned (bulk copies)
     L.edge_off = L.cand_off + CAND_BYTES * LIST_CAP * stages;
-    L.tab_off = (L.edge_off + (int)sizeof(float) * 2 * rows * edge_pops(Q) * stages + 15) & ~15;
+    L.tab_off = (L.edge_off + (int)sizeof(float) * 2 * rows * edge_pops() * stages + 15) & ~15;
     L.pre_off = L.tab_off + (int)sizeof(TInst) * ntab;
     L.bar_off = L.pre_off + 4 * 2 * PRE_WORDS;
     L.bytes = L.bar_off + 16 * stages + 128;  // + alignment slack of the base
@@ -236,9 +228,7 @@ __host__ __device__ inline TmaLayout tma_layout(int Q, int ssize, int tw, int ro
 }
 
 // The k-th population (0-based) with c_x == ecx.
-template <int Q>
 __device__ __forceinline__ int edge_pop(int ecx, int k) {
-    using L = Lat<Q>;
     int q = 1;
     for (int m = 0, qq = 1; qq < Q; ++qq)
         if (L::c(qq, 0) == ecx && m++ == k) q = qq;
@@ -247,15 +237,12 @@ __device__ __forceinline__ int edge_pop(int ecx, int k) {
 
 // Register budget: two blocks of 9 warps per SM; each lane collides two
 // nodes at a time.
-template <int Q, class S, int TW, int ROWS>
+template <class S, int TW, int ROWS>
 __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict__ insts,
                                                    const CUtensorMap* __restrict__ tmaps,
                                                    const uint16_t* __restrict__ tile_inst, int ntiles,
                                                    int par, Shape sh, int commit, int* tile_ctr,
                                                    int stages, int ninst) {
-    using L = Lat<Q>;
-    static_assert(Q == 9, "D3Q19 takes k_fluid_direct");
-    constexpr int D = L::D;
     constexpr int QS = Q - 1;
     constexpr int H = 16 / (int)sizeof(S);
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -263,26 +250,21 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
     // array itself: a pointer rebuilt from an integer would lose its address
     // space, and every access through it would become a generic load.
     unsigned char* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
-    constexpr int rows = ROWS;  // == sh.ty * sh.tz
+    constexpr int rows = ROWS;  // == sh.ty
     constexpr int BW = TW + 2 * H;
-    // elements between populations in a stage, and the row offset of population
-    // q's source row y - c_y: D2Q9 boxes span rows y0 - 1 .. y0 + rows (one copy
-    // per tile), D3Q19 boxes start at the source rows (one copy per population)
-    constexpr int SLAB = Q == 9 ? BW * (ROWS + 2)
-                                : ((BW * ROWS * (int)sizeof(S)) + 127) / 128 * 128 / (int)sizeof(S);
-    const TmaLayout LY = tma_layout(Q, (int)sizeof(S), TW, rows, stages, ninst);
+    constexpr int SLAB = BW * (ROWS + 2);  // elements between populations in a stage
+    const TmaLayout LY = tma_layout((int)sizeof(S), TW, rows, stages, ninst);
     StageHdr* hdr = reinterpret_cast<StageHdr*>(smem + LY.hdr_off);
     Cand* cands = reinterpret_cast<Cand*>(smem + LY.cand_off);
     float* edgev = reinterpret_cast<float*>(smem + LY.edge_off);  // [stages][side][rows][QE]
     TInst* tab = reinterpret_cast<TInst*>(smem + LY.tab_off);
     uint32_t* pre = reinterpret_cast<uint32_t*>(smem + LY.pre_off);  // [2][PRE_WORDS]
-    constexpr int QE = edge_pops(Q);
+    constexpr int QE = edge_pops();
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + LY.bar_off);
     uint64_t* empty = full + stages;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nc = (blockDim.x >> 5) - 1;  // consumer warps
     const int ntab = ninst < TI_MAX ? ninst : TI_MAX;
-    const int lty = __ffs(sh.ty) - 1;  // tile rows along y: a power of two
     if (threadIdx.x == 0) {
         for (int s = 0; s < stages; ++s) {
             mbar_init(&full[s], 1);
@@ -290,7 +272,7 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int i = threadIdx.x; i < ntab; i += blockDim.x) make_tinst<Q>(tab[i], insts[i]);
+    for (int i = threadIdx.x; i < ntab; i += blockDim.x) make_tinst(tab[i], insts[i]);
     __syncthreads();
     dep_wait();  // the populations, lists and work counter of the previous step
     dep_launch();
@@ -337,16 +319,12 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
             const bool tb = ninst <= TI_MAX;
             const int tile0 = tb ? tab[a.ii].tile0 : in.tile0;
             const int ntx = tb ? tab[a.ii].ntx : in.ntile[0];
-            const int nty = tb ? tab[a.ii].nty : in.ntile[1];
-            const int n[3] = {tb ? tab[a.ii].n[0] : in.n[0], tb ? tab[a.ii].n[1] : in.n[1],
-                              tb ? tab[a.ii].n[2] : in.n[2]};
+            const int n[2] = {tb ? tab[a.ii].n[0] : in.n[0], tb ? tab[a.ii].n[1] : in.n[1]};
             a.np = tb ? tab[a.ii].np : in.np;
             a.sload = tb ? tab[a.ii].sload : in.s_load;
             a.local = t - tile0;
             a.x0 = (a.local % ntx) * TW;
-            const int rest = a.local / ntx;
-            a.y0 = (rest % nty) * sh.ty;
-            a.z0 = (rest / nty) * sh.tz;
+            a.y0 = a.local / ntx * rows;
             if (lane == 0) {
                 if (a.np > 0) cp_async4(pb + PRE_CNT, (tb ? tab[a.ii].lcnt[par] : in.list_cnt[par]) + a.local);
                 else pb[PRE_CNT] = 0u;
@@ -368,17 +346,14 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
                     if (!((a.ex >> side) & 1)) continue;
                     const int r = (l - side * rows * QE) / QE, k = (l - side * rows * QE) % QE;
                     const int ecx = side ? -1 : 1, xe = side ? n[0] - 1 : 0;
-                    const int q = edge_pop<Q>(ecx, k);
-                    const int y = a.y0 + (r & (sh.ty - 1)), z = a.z0 + (r >> lty);
-                    const int ys = y - L::c(q, 1), zs = z - L::c(q, 2);
+                    const int q = edge_pop(ecx, k);
+                    const int y = a.y0 + r, ys = y - L::c(q, 1);
                     const S* src = nullptr;
                     if (!xper) {  // bounce-back at the x wall
-                        if (y < n[1] && z < n[2])
-                            src = fin + (long long)(L::opp(q) - 1) * qstr + ((long long)z * n[1] + y) * pitch + xe;
+                        if (y < n[1]) src = pop(fin, L::opp(q), qstr) + (y * pitch + xe);
                         a.add[j] = tb ? tab[a.ii].ewt[side][k] : in.wterm[0][side][q];
-                    } else if (y < n[1] && z < n[2] && ys >= 0 && ys < n[1] && zs >= 0 && zs < n[2]) {
-                        const int xs = side ? 0 : n[0] - 1;  // periodic wrap
-                        src = fin + (long long)(q - 1) * qstr + ((long long)zs * n[1] + ys) * pitch + xs;
+                    } else if (y < n[1] && ys >= 0 && ys < n[1]) {
+                        src = pop(fin, q, qstr) + (ys * pitch + (side ? 0 : n[0] - 1));  // periodic wrap
                     }
                     if (src) {
                         const uintptr_t ad = reinterpret_cast<uintptr_t>(src);
@@ -430,7 +405,7 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
                 if (lane < TI_WORDS)
                     reinterpret_cast<uint4*>(&h.ti)[lane] = reinterpret_cast<const uint4*>(&tab[a.ii])[lane];
             } else if (lane == 0) {
-                make_tinst<Q>(h.ti, insts[a.ii]);
+                make_tinst(h.ti, insts[a.ii]);
             }
             if (a.ex) {
                 float* ev = edgev + s * 2 * rows * QE;
@@ -455,7 +430,6 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
                 h.inst = a.ii;
                 h.x0 = a.x0;
                 h.y0 = a.y0;
-                h.z0 = a.z0;
                 h.ncand = ncand;
                 h.ex = a.ex;
                 if (commit && a.np > 0)  // this tile's list of the next step starts empty
@@ -502,17 +476,17 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
         const StageHdr& h = hdr[s];
         const int ncand = h.ncand;
         const Cand* cand = cands + s * LIST_CAP;
-        const int nx = h.ti.n[0], ny = h.ti.n[1], nz = h.ti.n[2];
+        const int nx = h.ti.n[0], ny = h.ti.n[1];
         const float sload = h.ti.sload;
         const CollK ck = make_collk<Q>(CollP{h.ti.keep, h.ti.fpref, h.ti.alpha});
-        const int x0 = h.x0, y0 = h.y0, z0 = h.z0;
+        const int x0 = h.x0, y0 = h.y0;
         const S* stage = reinterpret_cast<const S*>(smem + s * LY.stage);
         const int ex = h.ex;
         const bool free = h.ti.free != 0;
         const TileEnv env{h.ti, h.ti.tot[commit ? par : 2]};
         const float* ev = edgev + s * 2 * rows * QE;
         bool bad = false;
-        // FOLD (D2Q9, FP16 storage at tau = 1): the populations stay at the
+        // FOLD (FP16 storage at tau = 1): the populations stay at the
         // storage scale from the stage to the store (collide2_t1_scaled)
         auto tile_rows = [&](auto fold_tag) {
             constexpr bool FOLD = decltype(fold_tag)::value;
@@ -527,19 +501,18 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
                 }
             }
             for (int r = cw; r < rows; r += nc) {
-                const int y = y0 + (r & (sh.ty - 1)), z = z0 + (r >> lty);
-                if (y >= ny || z >= nz) continue;
-                // every source row lies inside the box (and so in the stage), or (D2Q9)
-                // beyond a y wall: then the node's own opposite population, staged
-                // too, comes back
+                const int y = y0 + r;
+                if (y >= ny) break;
+                // every source row lies inside the box (and so in the stage), or beyond
+                // a y wall: then the node's own opposite population, staged too,
+                // comes back
                 const bool lo_y = y < 1, hi_y = y + 1 >= ny;
-                const bool rowfast = D == 2 ? !(lo_y || hi_y) || !h.ti.per[1]
-                                            : !(lo_y || hi_y) && z >= 1 && z + 1 < nz;
+                const bool rowfast = !(lo_y || hi_y) || !h.ti.per[1];
                 const S* rowbase = stage + r * BW + H;
                 // element of population q's source row in the stage, relative to rowbase
-                auto qoff = [&](int q) { return (q - 1) * SLAB + (Q == 9 ? (1 - L::c(q, 1)) * BW : 0); };
-                auto beyond_y = [&](int q) { return D == 2 && (L::c(q, 1) > 0 ? lo_y : L::c(q, 1) < 0 && hi_y); };
-                S* outrow = static_cast<S*>(const_cast<void*>(h.ti.f[par ^ 1])) + ((long long)z * ny + y) * h.ti.pitch;
+                auto qoff = [&](int q) { return (q - 1) * SLAB + (1 - L::c(q, 1)) * BW; };
+                auto beyond_y = [&](int q) { return L::c(q, 1) > 0 ? lo_y : L::c(q, 1) < 0 && hi_y; };
+                S* outrow = static_cast<S*>(const_cast<void*>(h.ti.f[par ^ 1])) + y * h.ti.pitch;
                 // two adjacent nodes per lane: packed FP32x2 arithmetic, 8-byte stores
                 for (int j = 0; j < TW / 64; ++j) {
                     const int lx = j * 64 + 2 * lane;
@@ -560,7 +533,7 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
                                                            to_float_scaled(src[1], sload));
                             }
                         }
-                        if (D == 2 && (lo_y || hi_y)) {  // bounce-back at the y walls (Eq. 10)
+                        if (lo_y || hi_y) {  // bounce-back at the y walls (Eq. 10)
 #pragma unroll
                             for (int q = 1; q < Q; ++q) {
                                 const int cy = L::c(q, 1);
@@ -600,23 +573,23 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
                             }
                         }
                     } else {
-                        // a row at a y or z face: every population straight from the
+                        // a row at a periodic y face: every population straight from the
                         // previous buffer (L2 holds it), all loads in flight
                         const S* fin = static_cast<const S*>(h.ti.f[par]);
                         float g[QS];
-                        pull_pre_all<Q, S>(insts[h.inst], fin, min(x, nx - 1), y, z, h.ti.qstride, g);
+                        pull_pre_all<Q, S>(insts[h.inst], fin, min(x, nx - 1), y, 0, h.ti.qstride, g);
 #pragma unroll
                         for (int q = 0; q < QS; ++q) f[q].x = FOLD ? g[q] * sstore : g[q];
-                        pull_pre_all<Q, S>(insts[h.inst], fin, min(x + 1, nx - 1), y, z, h.ti.qstride, g);
+                        pull_pre_all<Q, S>(insts[h.inst], fin, min(x + 1, nx - 1), y, 0, h.ti.qstride, g);
 #pragma unroll
                         for (int q = 0; q < QS; ++q) f[q].y = FOLD ? g[q] * sstore : g[q];
                     }
                     bad |= finish_pair<Q, S, FOLD>(env, f, FOLD ? cks : ck, sload, sstore, free, cand, ncand,
-                                                   x0 + j * 64, x, y, z, lane, outrow + x, (int)h.ti.qstride);
+                                                   x0 + j * 64, x, y, 0, lane, outrow + x, (int)h.ti.qstride);
                 }
             }
         };
-        if constexpr (sizeof(S) == 2 && Q == 9) {  // (D3Q19 would spill more)
+        if constexpr (sizeof(S) == 2) {
             if (ck.keep == 0.f) tile_rows(std::true_type{});
             else tile_rows(std::false_type{});
         } else {
@@ -629,23 +602,23 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
 }
 
 // ------------------------------------------------------------- host side ---
-template <int Q, class S, int TW, int ROWS>
+template <class S, int TW, int ROWS>
 static cudaError_t launch_tma_t(const InstDesc* insts, const void* tmaps, const uint16_t* tile_inst,
                                 int ntiles, int par, const Shape& sh, int commit, int grid,
                                 int* tile_ctr, int stages, int ninst, cudaStream_t st) {
-    const TmaLayout LY = tma_layout(Q, (int)sizeof(S), TW, ROWS, stages, ninst);
-    return launch_dep(k_fluid_tma<Q, S, TW, ROWS>, dim3((unsigned)grid), 32 * (sh.warps + 1), LY.bytes, st, insts,
+    const TmaLayout LY = tma_layout((int)sizeof(S), TW, ROWS, stages, ninst);
+    return launch_dep(k_fluid_tma<S, TW, ROWS>, dim3((unsigned)grid), 32 * (sh.warps + 1), LY.bytes, st, insts,
                       static_cast<const CUtensorMap*>(tmaps), tile_inst, ntiles, par, sh, commit, tile_ctr, stages, ninst);
 }
 
-int tma_tile_width(int Q) { return Q == 9 ? 128 : 64; }
+int tma_tile_width() { return 128; }
 
 bool tma_rows_ok(int rows) { return rows == 4 || rows == 8; }
 
-template <int Q, class S, int TW, int ROWS>
+template <class S, int TW, int ROWS>
 static int tma_blocks_t(const Shape& sh, int stages, int ninst) {
-    const TmaLayout LY = tma_layout(Q, (int)sizeof(S), TW, ROWS, stages, ninst);
-    auto* const kern = k_fluid_tma<Q, S, TW, ROWS>;
+    const TmaLayout LY = tma_layout((int)sizeof(S), TW, ROWS, stages, ninst);
+    auto* const kern = k_fluid_tma<S, TW, ROWS>;
     {
         // the limit belongs to the kernel, not to a context: only raised, so that a
         // context with fewer instances or stages leaves the others' launches valid
@@ -662,28 +635,26 @@ static int tma_blocks_t(const Shape& sh, int stages, int ninst) {
     return nb;
 }
 
-#define LBM_TMA_DISPATCH(CALL)                                       \
-    {                                                                \
-        const int rows = sh.ty;                                      \
-        if (Q == 9 && !fp16 && rows == 4) return CALL(9, float, 128, 4);  \
-        if (Q == 9 && !fp16 && rows == 8) return CALL(9, float, 128, 8);  \
-        if (Q == 9 && fp16 && rows == 4) return CALL(9, __half, 128, 4);  \
-        if (Q == 9 && fp16 && rows == 8) return CALL(9, __half, 128, 8);  \
+#define LBM_TMA_DISPATCH(CALL)                              \
+    {                                                       \
+        if (!fp16 && sh.ty == 4) return CALL(float, 128, 4);  \
+        if (!fp16 && sh.ty == 8) return CALL(float, 128, 8);  \
+        if (fp16 && sh.ty == 4) return CALL(__half, 128, 4);  \
+        if (fp16 && sh.ty == 8) return CALL(__half, 128, 8);  \
     }
 
-int fluid_tma_blocks_per_sm(int Q, int fp16, const Shape& sh, int stages, int ninst) {
-#define LBM_BLK(QQ, SS, TT, RR) tma_blocks_t<QQ, SS, TT, RR>(sh, stages, ninst)
+int fluid_tma_blocks_per_sm(int fp16, const Shape& sh, int stages, int ninst) {
+#define LBM_BLK(SS, TT, RR) tma_blocks_t<SS, TT, RR>(sh, stages, ninst)
     LBM_TMA_DISPATCH(LBM_BLK)
 #undef LBM_BLK
     return 0;
 }
 
-cudaError_t launch_fluid_tma(int Q, int fp16, const InstDesc* insts, const void* tmaps,
+cudaError_t launch_fluid_tma(int fp16, const InstDesc* insts, const void* tmaps,
                              const uint16_t* tile_inst, int ntiles, int par, const Shape& sh,
                              int commit, int grid, int* tile_ctr, int stages, int ninst, cudaStream_t st) {
-#define LBM_LAUNCH(QQ, SS, TT, RR)                                                                    \
-    launch_tma_t<QQ, SS, TT, RR>(insts, tmaps, tile_inst, ntiles, par, sh, commit, grid, tile_ctr, stages, \
-                                 ninst, st)
+#define LBM_LAUNCH(SS, TT, RR)                                                                             \
+    launch_tma_t<SS, TT, RR>(insts, tmaps, tile_inst, ntiles, par, sh, commit, grid, tile_ctr, stages, ninst, st)
     LBM_TMA_DISPATCH(LBM_LAUNCH)
 #undef LBM_LAUNCH
     return cudaErrorInvalidValue;

@@ -176,8 +176,7 @@ struct InstDesc {
     int tile0;                // first global tile of this instance
     int np;                   // particles
     int maxk;                 // most tiles a particle's bounding box may cover (list slot k)
-    int part0;                // global index of particle 0 (batched arrays)
-    float tau_inv, keep;      // 1/tau and 1 - 1/tau
+    float keep;               // 1 - 1/tau
     float fpref;              // 1 - 1/(2 tau)
     float alpha;
     float gdrive[3];

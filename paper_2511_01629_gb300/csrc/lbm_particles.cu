@@ -802,9 +802,12 @@ __global__ void k_publish(const InstDesc* __restrict__ insts, const PartRef* __r
     append_tiles(insts[r.inst], r.p, at, cd, lpar, 0, 1);
 }
 
-int particle_blocks_resident(int num_sms) {
+// Blocks of the kernel of dimension D that are resident at once (its grid barriers need all).
+int particle_blocks_resident(int D, int num_sms) {
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_particles<3>, 256, 0) != cudaSuccess) return 0;
+    const cudaError_t e = D == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_particles<2>, 256, 0)
+                                 : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_particles<3>, 256, 0);
+    if (e != cudaSuccess) return 0;
     return nb * num_sms;
 }
 
