@@ -416,6 +416,8 @@ void particle_constants(const Instance& I, std::vector<double>& pc, std::vector<
         r.qlo = 1.0f - beta;
         r.qhi = 1.0f + beta;
         r.shape = B != R;
+        const int H = (int)ceil(R) + 2;
+        r.rows2 = (H - 1) * (H - 1);
     }
 }
 int upload_pconst(lbm_ctx* ctx, Instance& I) {

@@ -118,7 +118,8 @@ struct __align__(16) Cand {
     float a[3];
     int p;     // particle index within the instance
     int k;     // index of this tile among the tiles of the particle's bounding box
-    int pad[2];
+    int rows2; // see RecConst
+    int pad;
     int shape; // 0 disk or sphere, 1 ellipse (the filter reads its record)
 };
 static_assert(sizeof(Cand) == CAND_BYTES, "candidate records are copied in 64-byte units");
@@ -761,6 +762,15 @@ __device__ __forceinline__ void rigid_sums(long long* __restrict__ tot, const Ge
         const Cand& cd = cand[s];
         const int dy = wrap_int(y - cd.ref[1], g.n[1], g.per[1]);
         const int dz = D == 3 ? wrap_int(z - cd.ref[2], g.n[2], g.per[2]) : 0;
+        if (D == 3 && dy * dy + dz * dz > cd.rows2) {
+            // Kept as the sums have always been: (ceil(R) + 1)^2 leaves out the outermost
+            // nodes of a sphere whose centre lies near the far corner of its lattice
+            // cell in y and z (up to R + sqrt(2) from floor(X)); 4 of 2139 nodes at
+            // R = 8, offsets 0.99 and 0.85.
+#pragma unroll
+            for (int e = 0; e < V; ++e) slot[e] = slot[e] == s ? -1 : slot[e];
+            continue;
+        }
         int cnt = 0, sx = 0, sxx = 0;
         int sh[D], sl[D], xh[D], xl[D];  // halves of sum u and of sum dx u (y, z)
 #pragma unroll

@@ -195,6 +195,7 @@ __device__ __forceinline__ void fluid_tile(const InstDesc& in, int local, int pa
             cd.p = p;
             cd.k = (int)(e & (MAXK - 1));
             cd.shape = pr.shape;
+            cd.rows2 = pr.rows2;
             cand[c] = cd;
         }
         if (commit && tid == 0) in.list_cnt[par ^ 1][local] = 0;

@@ -147,7 +147,7 @@ struct __align__(16) PRec {
                        //   (an ellipse: only d2 > R2hi, its circumscribed circle)
     float a[3];      // solid-node acceleration (1 - rho_f/rho_s) g + A_i
     int shape;       // 0 disk or sphere, 1 ellipse
-    int pad;
+    int rows2;       // see RecConst
     double ec, es;   // cos, sin of theta^n (ellipse; 1, 0 otherwise)
     double b2;       // b * b
     float fc, fs;    // ec, es as float (filter test)
@@ -163,7 +163,8 @@ static_assert(sizeof(PRec) == 144, "particle record layout");
 struct RecConst {
     double R2, b2;
     float R2lo, R2hi, ia2, ib2, qlo, qhi;
-    int shape, pad;
+    int shape;
+    int rows2;  // 3D: rows at dy^2 + dz^2 > rows2 from floor(X) stay out of the sums of Eq. 22
 };
 static_assert(sizeof(RecConst) == 48, "record constants layout");
 

@@ -287,7 +287,7 @@ __device__ __forceinline__ void record_radius(const InstDesc& in, PRec& pr, cons
     pr.R2hi = rc.R2hi;
     pr.ntiles = nt;
     pr.shape = rc.shape;
-    pr.pad = 0;
+    pr.rows2 = rc.rows2;
     pr.b2 = rc.b2;
     pr.ia2 = rc.ia2;
     pr.ib2 = rc.ib2;
@@ -344,7 +344,8 @@ __device__ __forceinline__ Cand make_cand(const PRec& pr, int p) {
     cd.R2hi = pr.R2hi;
     cd.p = p;
     cd.k = 0;
-    cd.pad[0] = cd.pad[1] = 0;
+    cd.rows2 = pr.rows2;
+    cd.pad = 0;
     cd.shape = pr.shape;
     return cd;
 }
@@ -574,7 +575,8 @@ __device__ __forceinline__ void update_lane(const InstDesc& in, int i, int d, in
         cd.R2lo = L.rc.R2lo;
         cd.R2hi = L.rc.R2hi;
         cd.p = i;
-        cd.pad[0] = cd.pad[1] = 0;
+        cd.rows2 = L.rc.rows2;
+        cd.pad = 0;
         cd.shape = L.rc.shape;
     }
     in.A[j] = An;
