@@ -317,8 +317,8 @@ __global__ void __launch_bounds__(32 * ADJ_WARPS, Q == 9 ? ADJ_BLOCKS : 3) k_adj
         const bool edge = xb == 0 || xb + 64 >= nx;
         float g0[QS], g1[QS];
         if (row_in) {
-            if (edge) pull_pair<Q, S, true>(in, fin, x, y, z, f);
-            else pull_pair<Q, S, false>(in, fin, x, y, z, f);
+            if (edge) pull_pair<Q, S, true>(in, fin, qs, x, y, z, f);
+            else pull_pair<Q, S, false>(in, fin, qs, x, y, z, f);
         } else {
             pull_pre_all<Q, S>(in, fin, xc0, y, z, qs, g0);
             pull_pre_all<Q, S>(in, fin, xc1, y, z, qs, g1);

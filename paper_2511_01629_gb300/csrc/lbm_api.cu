@@ -40,9 +40,9 @@ cudaError_t launch_fluid_tma(int fp16, const InstDesc* insts, const void* tmaps,
                              const uint16_t* tile_inst, int ntiles, int par, const Shape& sh,
                              int commit, int grid, int* tile_ctr, int stages, int ninst, cudaStream_t st);
 int direct_tile_width();
-int fluid_direct_blocks_per_sm(int Q, int fp16, const Shape& sh);
-cudaError_t launch_fluid_direct(int Q, int fp16, const InstDesc* insts, const uint16_t* tile_inst, int ninst, int ntiles,
-                                int par, const Shape& sh, int commit, cudaStream_t st);
+int fluid_direct_blocks_per_sm(int Q, int fp16, bool wide, const Shape& sh);
+cudaError_t launch_fluid_direct(int Q, int fp16, bool wide, const InstDesc* insts, const uint16_t* tile_inst, int ninst,
+                                int ntiles, int par, const Shape& sh, int commit, cudaStream_t st);
 cudaError_t launch_adj_fluid(int Q, int fp16, const InstDesc* insts, const AdjFluid* afs,
                              const uint16_t* tile_inst, int ninst, int ntiles, int lam_mode, const Shape& sh,
                              int num_sms, cudaStream_t st);
@@ -107,6 +107,7 @@ struct AdjCtx {
 
 struct lbm_ctx {
     int Q = 9, D = 2, fp16 = 0;
+    bool wide = false;  // an instance's populations need 64-bit offsets
     cudaStream_t st = nullptr;
     lbm_allocator alloc{};
     bool has_alloc = false;
@@ -533,7 +534,7 @@ int configure_shape(lbm_ctx* ctx, const Shape& sh_in) {
     CK(cudaStreamSynchronize(ctx->st));
     const int occ = !sh.tma ? fluid_max_blocks_per_sm(ctx->Q, ctx->fp16, sh)
                     : staged(sh) ? fluid_tma_blocks_per_sm(ctx->fp16, sh, sh.stages, (int)ctx->inst.size())
-                                 : fluid_direct_blocks_per_sm(ctx->Q, ctx->fp16, sh);
+                                 : fluid_direct_blocks_per_sm(ctx->Q, ctx->fp16, ctx->wide, sh);
     if (occ < 1) return set_err(ctx, LBM_ERR_INVALID, "kernel shape does not fit on an SM%s");
     ctx->grid = occ * ctx->num_sms;
     if (staged(sh) && (rc = build_tmaps(ctx))) return rc;
@@ -565,7 +566,7 @@ int enqueue_fluid_on(lbm_ctx* ctx, const InstDesc* insts, const void* tmaps, int
         CK(launch_fluid_tma(ctx->fp16, insts, tmaps, P<uint16_t>(ctx->d_tile_inst), ctx->ntiles, par, sh, commit,
                             ctx->grid, P<int>(ctx->d_tile_ctr), sh.stages, (int)ctx->inst.size(), st));
     else if (sh.tma)
-        CK(launch_fluid_direct(ctx->Q, ctx->fp16, insts, P<uint16_t>(ctx->d_tile_inst), (int)ctx->inst.size(), ctx->ntiles,
+        CK(launch_fluid_direct(ctx->Q, ctx->fp16, ctx->wide, insts, P<uint16_t>(ctx->d_tile_inst), (int)ctx->inst.size(), ctx->ntiles,
                                par, sh, commit, st));
     else
         CK(launch_fluid(ctx->Q, ctx->fp16, insts, P<uint16_t>(ctx->d_tile_inst), ctx->ntiles, par, sh, commit,
@@ -750,6 +751,7 @@ int lbm_create_batch(const lbm_config* cfgs, int n, const lbm_allocator* alloc, 
         if (ctx->D == 2) I.n[2] = 1;
         I.pitch = (I.n[0] + 31) & ~31;
         I.qstride = (long long)I.pitch * I.n[1] * I.n[2];
+        ctx->wide |= wide_offsets(ctx->Q, I.qstride);
         I.cap = cfgs[i].max_particles;
         const size_t fb = ssz * (size_t)(ctx->Q - 1) * (size_t)I.qstride;
         rc = slab_alloc(ctx, I.fslab, {{&I.f[0], fb}, {&I.f[1], fb}});

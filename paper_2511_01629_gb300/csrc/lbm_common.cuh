@@ -2,6 +2,8 @@
 // path) and the export kernels of lbmpen.
 #pragma once
 
+#include <type_traits>
+
 #include "lbm_internal.cuh"
 
 namespace lbmpen {
@@ -1055,6 +1057,14 @@ __host__ __device__ __forceinline__ PullSrc pull_source(const InstDesc& in, int 
     return PullSrc{axis >= 0 ? (z * in.n[1] + y) * in.pitch + x : (src[2] * in.n[1] + src[1]) * in.pitch + src[0], axis, face};
 }
 
+// Element off of population q.  The type of qs says how: int where the whole buffer
+// has 32-bit offsets (not wide_offsets), long long for any.
+template <class P>
+__host__ __device__ __forceinline__ P* elem(P* f, int q, int qs, int off) { return f + ((q - 1) * qs + off); }
+template <class P>
+__host__ __device__ __forceinline__ P* elem(P* f, int q, long long qs, int off) { return pop(f, q, qs) + off; }
+template <int Q> using Off9 = std::conditional_t<Q == 9, int, long long>;  // where D3Q19 has one form
+
 // One population value, or two of adjacent nodes, by plain (coherent) loads: the
 // fluid kernels may be resident while the step before writes them (dep_wait).
 __device__ __forceinline__ float load_one(const float* p, float) { return *p; }
@@ -1068,22 +1078,19 @@ __device__ __forceinline__ float2 load_pair(const __half* p, float s) {
 // Pre-collision population q at node (x, y, z): what it pulls, plus across a
 // wall the moving-wall term 2 w_q (c_q . u_w) / cs^2.  Selects instead of
 // branches, so that the lanes of a warp on a face stay together.
-template <int Q, class S, int q>
-__device__ __forceinline__ float pull_pre_any(const InstDesc& in, const S* fin, int x, int y, int z,
-                                              long long qs) {
+template <int Q, class S, int q, class I>
+__device__ __forceinline__ float pull_pre_any(const InstDesc& in, const S* fin, int x, int y, int z, I qs) {
     const PullSrc s = pull_source<Q, q>(in, x, y, z);
     // the wall term is loaded whether it is needed or not: a load under a
     // condition would hold back the next population's (one memory latency each)
     const float term = __ldg(&in.wterm[s.axis >= 0 ? s.axis : 0][s.face][q]);
-    const S* from = s.axis >= 0 ? pop(fin, Lat<Q>::opp(q), qs) : pop(fin, q, qs);
-    const float v = load_one(from + s.off, in.s_load);
+    const float v = load_one(elem(fin, s.axis >= 0 ? Lat<Q>::opp(q) : q, qs, s.off), in.s_load);
     return s.axis >= 0 ? v + term : v;
 }
 
 // All populations of a node by pull_pre_any (independent loads in flight).
-template <int Q, class S, int q = 1>
-__device__ __forceinline__ void pull_pre_all(const InstDesc& in, const S* fin, int x, int y, int z,
-                                             long long qs, float* f) {
+template <int Q, class S, int q = 1, class I>
+__device__ __forceinline__ void pull_pre_all(const InstDesc& in, const S* fin, int x, int y, int z, I qs, float* f) {
     if constexpr (q < Q) {
         f[q - 1] = pull_pre_any<Q, S, q>(in, fin, x, y, z, qs);
         pull_pre_all<Q, S, q + 1>(in, fin, x, y, z, qs, f);
@@ -1100,11 +1107,11 @@ __device__ __forceinline__ void pull_pre_all(const InstDesc& in, const S* fin, i
 // together.  Selecting the address of every load instead cost each lane some
 // 200 instructions a row (backward pass of 16 boxes of 400 x 1600: 19.7 -> 18.1
 // ms; the forward kernels, bound elsewhere, did not change).
-template <int Q, class S, bool EDGE>
-__device__ __forceinline__ void pull_pair(const InstDesc& in, const S* fin, int x, int y, int z, float2* f) {
+template <int Q, class S, bool EDGE, class I>
+__device__ __forceinline__ void pull_pair(const InstDesc& in, const S* fin, I qs, int x, int y, int z, float2* f) {
     using L = Lat<Q>;
     const int nx = in.n[0], pitch = in.pitch, zs = in.n[1] * pitch;
-    const long long qs = in.qstride;
+    constexpr bool narrow = sizeof(I) == 4;
     const float sl = in.s_load;
     const int own = z * zs + y * pitch, xl = EDGE ? min(x, (nx - 1) & ~1) : x;
     auto row_of = [&](int q) { return own - L::c(q, 2) * zs - L::c(q, 1) * pitch; };  // within population q
@@ -1112,22 +1119,23 @@ __device__ __forceinline__ void pull_pair(const InstDesc& in, const S* fin, int 
 #pragma unroll
     for (int q = 1; q < Q; ++q, fq += qs) {
         const int cx = L::c(q, 0), sh = -L::c(q, 2) * zs - L::c(q, 1) * pitch;
-        if (cx == 0) f[q - 1] = load_pair(fq + sh, sl);
-        else f[q - 1] = make_float2(load_one(fq + sh - cx, sl), load_one(fq + sh + (1 - cx), sl));
+        const S* a = narrow ? elem(fin, q, (int)qs, row_of(q) + xl) : fq + sh;
+        if (cx == 0) f[q - 1] = load_pair(a, sl);
+        else f[q - 1] = make_float2(load_one(a - cx, sl), load_one(a + (1 - cx), sl));
     }
     if constexpr (EDGE) {
         const bool wall = !in.periodic[0], lo = x == 0, hi0 = x == nx - 1, hi1 = x + 1 == nx - 1;
-        // at a wall population opp(q) = q + (opp - q): one 64-bit select for all of them.
-        // Selecting each pointer cost 256 x 256 x 512 FP16 656 us a step, this 620 (616
-        // with 32-bit addresses, which do not reach all of a large box)
-        const long long wq = wall ? qs : 0;
+        // wide: at a wall population opp(q) = q + (opp - q), one 64-bit select for all of
+        // them (selecting each pointer cost 256 x 256 x 512 FP16 656 us a step, this 620)
+        const I wq = wall ? qs : 0;
         float v[Q], t[Q];
 #pragma unroll
         for (int q = 1; q < Q; ++q) {
             const int cx = L::c(q, 0);
             if (cx == 0) continue;
-            const S* from = pop(fin, q, qs) + (L::opp(q) - q) * wq +
-                            (wall ? own + (cx > 0 ? 0 : nx - 1) : row_of(q) + (cx > 0 ? nx - 1 : 0));
+            const int at_wall = own + (cx > 0 ? 0 : nx - 1), across = row_of(q) + (cx > 0 ? nx - 1 : 0);
+            const S* from = narrow ? fin + (wall ? (L::opp(q) - 1) * (int)qs + at_wall : (q - 1) * (int)qs + across)
+                                   : pop(fin, q, qs) + (L::opp(q) - q) * wq + (wall ? at_wall : across);
             v[q] = 0.f;
             if (cx > 0 ? lo : hi0 || hi1) v[q] = load_one(from, sl);
             t[q] = __ldg(&in.wterm[0][cx > 0 ? 0 : 1][q]);

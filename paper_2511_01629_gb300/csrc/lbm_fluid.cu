@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(256, Q == 9 ? 4 : 2) k_fields(const InstDesc* 
     const int row = (int)(w / (unsigned)nseg);
     const int y = row % ny, z = row / ny;
     const long long N = (long long)nx * ny * nz;
-    const long long qs = in.qstride;
+    const Off9<Q> qs = (Off9<Q>)in.qstride;
     const S* __restrict__ fin = static_cast<const S*>(in.f[par]);
     const float sl = in.s_load;
     const bool row_in = y >= 1 && y + 1 < ny && (D == 2 || (z >= 1 && z + 1 < nz));
@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(256, Q == 9 ? 4 : 2) k_fields(const InstDesc* 
 #pragma unroll
             for (int q = 1; q < Q; ++q)
                 f[k][q - 1] = VecIO<S, 1 + (sizeof(S) == 2)>::load1(
-                    pop(fin, q, qs) + (at - (L::c(q, 2) * ny + L::c(q, 1)) * pitch - L::c(q, 0)), sl);
+                    elem(fin, q, qs, at - (L::c(q, 2) * ny + L::c(q, 1)) * pitch - L::c(q, 0)), sl);
         } else {
             pull_pre_all<Q, S>(in, fin, x, y, z, qs, f[k]);
         }

@@ -35,7 +35,7 @@ struct DescEnv {
 
 }  // namespace
 
-template <int Q, class S>
+template <int Q, class S, class I>
 __global__ void __launch_bounds__(256, Q == 9 ? 4 : 3) k_fluid_direct(const InstDesc* __restrict__ insts,
                                                          const uint16_t* __restrict__ tile_inst, int ninst, int par, Shape sh,
                                                          int commit) {
@@ -56,6 +56,7 @@ __global__ void __launch_bounds__(256, Q == 9 ? 4 : 3) k_fluid_direct(const Inst
     const bool edge = x0 == 0 || x0 + TW >= nx;
     const float sload = in.s_load;
     const S* fin = static_cast<const S*>(in.f[par]);
+    const I qs = (I)in.qstride;
     float2 f[QS];
     dep_wait();  // the populations and lists of the previous step
     dep_launch();
@@ -63,14 +64,14 @@ __global__ void __launch_bounds__(256, Q == 9 ? 4 : 3) k_fluid_direct(const Inst
         const int y = y0 + (r & (sh.ty - 1)), z = z0 + (r >> lty);
         if (r >= rows || y >= ny || z >= nz) return false;
         if (y >= 1 && y + 1 < ny && (D == 2 || (z >= 1 && z + 1 < nz))) {
-            if (edge) pull_pair<Q, S, true>(in, fin, x, y, z, f);
-            else pull_pair<Q, S, false>(in, fin, x, y, z, f);
+            if (edge) pull_pair<Q, S, true>(in, fin, qs, x, y, z, f);
+            else pull_pair<Q, S, false>(in, fin, qs, x, y, z, f);
         } else {
             float g[QS];
-            pull_pre_all<Q, S>(in, fin, min(x, nx - 1), y, z, in.qstride, g);
+            pull_pre_all<Q, S>(in, fin, min(x, nx - 1), y, z, qs, g);
 #pragma unroll
             for (int q = 0; q < QS; ++q) f[q].x = g[q];
-            pull_pre_all<Q, S>(in, fin, min(x + 1, nx - 1), y, z, in.qstride, g);
+            pull_pre_all<Q, S>(in, fin, min(x + 1, nx - 1), y, z, qs, g);
 #pragma unroll
             for (int q = 0; q < QS; ++q) f[q].y = g[q];
         }
@@ -108,31 +109,29 @@ __global__ void __launch_bounds__(256, Q == 9 ? 4 : 3) k_fluid_direct(const Inst
 
 int direct_tile_width() { return TW; }
 
-template <int Q, class S>
-static int direct_blocks_t(const Shape& sh) {
-    int nb = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_fluid_direct<Q, S>, 32 * sh.warps, 0);
-    return nb;
-}
-int fluid_direct_blocks_per_sm(int Q, int fp16, const Shape& sh) {
-    if (Q == 9) return fp16 ? direct_blocks_t<9, __half>(sh) : direct_blocks_t<9, float>(sh);
-    return fp16 ? direct_blocks_t<19, __half>(sh) : direct_blocks_t<19, float>(sh);
+// The kernel of a lattice, storage type and width of offsets (wide_offsets).  64-bit
+// addresses on every box cost 151 x 133 x 203 FP16 1.5 % (160 steps 21.55 ms against
+// 21.25) and 256 x 256 x 512 FP32 0.2 %.
+template <class F>
+static auto direct_kernel(int Q, int fp16, bool wide, F&& go) {
+    if (Q == 9) return fp16 ? go(k_fluid_direct<9, __half, int>) : go(k_fluid_direct<9, float, int>);
+    if (!wide) return fp16 ? go(k_fluid_direct<19, __half, int>) : go(k_fluid_direct<19, float, int>);
+    return fp16 ? go(k_fluid_direct<19, __half, long long>) : go(k_fluid_direct<19, float, long long>);
 }
 
-cudaError_t launch_fluid_direct(int Q, int fp16, const InstDesc* insts, const uint16_t* tile_inst, int ninst, int ntiles,
-                                int par, const Shape& sh, int commit, cudaStream_t st) {
-    cudaError_t e = cudaSuccess;
-    auto go = [&](auto kern) {
-        e = launch_dep(kern, dim3((unsigned)ntiles), 32 * sh.warps, 0, st, insts, tile_inst, ninst, par, sh, commit);
-    };
-    if (Q == 9) {
-        if (fp16) go(k_fluid_direct<9, __half>);
-        else go(k_fluid_direct<9, float>);
-    } else {
-        if (fp16) go(k_fluid_direct<19, __half>);
-        else go(k_fluid_direct<19, float>);
-    }
-    return e;
+int fluid_direct_blocks_per_sm(int Q, int fp16, bool wide, const Shape& sh) {
+    return direct_kernel(Q, fp16, wide, [&](auto kern) {
+        int nb = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, 32 * sh.warps, 0);
+        return nb;
+    });
+}
+
+cudaError_t launch_fluid_direct(int Q, int fp16, bool wide, const InstDesc* insts, const uint16_t* tile_inst, int ninst,
+                                int ntiles, int par, const Shape& sh, int commit, cudaStream_t st) {
+    return direct_kernel(Q, fp16, wide, [&](auto kern) {
+        return launch_dep(kern, dim3((unsigned)ntiles), 32 * sh.warps, 0, st, insts, tile_inst, ninst, par, sh, commit);
+    });
 }
 
 }  // namespace lbmpen

@@ -577,10 +577,10 @@ __global__ void __launch_bounds__(288, 2) k_fluid_tma(const InstDesc* __restrict
                         // previous buffer (L2 holds it), all loads in flight
                         const S* fin = static_cast<const S*>(h.ti.f[par]);
                         float g[QS];
-                        pull_pre_all<Q, S>(insts[h.inst], fin, min(x, nx - 1), y, 0, h.ti.qstride, g);
+                        pull_pre_all<Q, S>(insts[h.inst], fin, min(x, nx - 1), y, 0, (int)h.ti.qstride, g);
 #pragma unroll
                         for (int q = 0; q < QS; ++q) f[q].x = FOLD ? g[q] * sstore : g[q];
-                        pull_pre_all<Q, S>(insts[h.inst], fin, min(x + 1, nx - 1), y, 0, h.ti.qstride, g);
+                        pull_pre_all<Q, S>(insts[h.inst], fin, min(x + 1, nx - 1), y, 0, (int)h.ti.qstride, g);
 #pragma unroll
                         for (int q = 0; q < QS; ++q) f[q].y = FOLD ? g[q] * sstore : g[q];
                     }

@@ -294,6 +294,13 @@ struct PartRef {
     int p;
 };
 
+// Whether the populations of an instance need 64-bit offsets: a buffer of 2^31
+// elements or more (the loads reach less than a pair of nodes beyond the last row).
+// Never in D2Q9: at most 1.1e8 nodes, and at most 2^20 rows of up to 31 padding nodes.
+__host__ __device__ inline bool wide_offsets(int Q, long long qstride) {
+    return Q == 19 && (Q - 1) * qstride + 64 > 0x7fffffffLL;
+}
+
 __host__ __device__ inline int tile_w(const Shape& s) { return s.tw; }
 
 // Programmatic dependent launch of the kernels of a step: the next kernel's

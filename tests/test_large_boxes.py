@@ -19,6 +19,8 @@ from paper_2511_01629_gb300 import workloads as W
 
 gpu = pytest.mark.gpu
 
+# just below the line, where the whole buffer has 32-bit offsets
+NARROW = [(64, 1300, 1260), (100, 965, 965), (33, 1366, 1364), (2, 1931, 1930)]
 BOXES = [(100, 1000, 1000), (65, 1200, 1300), (129, 900, 900), (33, 1785, 1785), (2, 7200, 7200), (5, 200, 100000)]
 
 PROGRAM = r"""
@@ -30,7 +32,10 @@ template <int q> void offsets(const InstDesc& in, int x, int y, int z) {
     if constexpr (q < 19) {
         const PullSrc s = pull_source<19, q>(in, x, y, z);
         const char* f = reinterpret_cast<const char*>(uintptr_t{1} << 40);  // never dereferenced
-        const char* from = pop(f, s.axis >= 0 ? Lat<19>::opp(q) : q, in.qstride) + s.off;
+        const int src = s.axis >= 0 ? Lat<19>::opp(q) : q;
+        const char* from = pop(f, src, in.qstride) + s.off;
+        if (elem(f, src, in.qstride, s.off) != from) exit(1);
+        if (!wide_offsets(19, in.qstride) && elem(f, src, (int)in.qstride, s.off) != from) exit(2);
         printf("%lld %d %d\n", (long long)(from - f), s.axis, s.face);
         offsets<q + 1>(in, x, y, z);
     }
@@ -64,12 +69,13 @@ def program(tmp_path_factory):
 
 
 @pytest.mark.parametrize("periodic", [(0, 0, 0), (1, 1, 1), (0, 1, 0)])
-@pytest.mark.parametrize("n", BOXES)
+@pytest.mark.parametrize("n", BOXES + NARROW)
 def test_offsets_of_large_boxes(program, n, periodic):
     assert n[0] * n[1] * n[2] * 19 <= 2e9  # accepted by lbm_create
     pitch = (n[0] + 31) // 32 * 32
     qs = pitch * n[1] * n[2]
-    assert qs < 2 ** 31 <= 18 * qs  # one population has 32-bit offsets, the buffer has not
+    assert qs < 2 ** 31  # one population has 32-bit offsets,
+    assert (18 * qs + 64 < 2 ** 31) == (n in NARROW)  # the buffer only in these
     nodes = list(itertools.product(*[sorted({0, 1, m // 2, m - 2, m - 1}) for m in n]))
     out = subprocess.run([program, *map(str, n), *map(str, periodic)], input="\n".join("%d %d %d" % v for v in nodes),
                          capture_output=True, text=True, check=True).stdout.split()
@@ -91,7 +97,14 @@ def test_offsets_of_large_boxes(program, n, periodic):
             assert next(got) == [want, axis, face], (node, c)
             assert 0 <= want < 18 * qs
             top = max(top, want)
-    assert top >= 2 ** 31  # the box reaches the range
+    assert top >= (2 ** 31 if n in BOXES else 2 ** 30)  # the box reaches the range
+
+
+def test_planar_boxes_have_32_bit_offsets():
+    """The largest D2Q9 buffers that lbm_create accepts (nodes 19 <= 2e9, axes up to 2^20)."""
+    for n0 in list(range(2, 4200)) + [2 ** 20]:
+        n1 = min(2 ** 20, int(2e9 / 19 / n0))
+        assert 8 * ((n0 + 31) // 32 * 32) * n1 + 64 < 2 ** 31
 
 
 def _context(n, storage, f):
