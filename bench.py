@@ -31,8 +31,8 @@ MEASURED_PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "fluid_kernel_traffic.json")
 CSRC = os.path.join(ROOT, "paper_2511_01629_gb300", "csrc")
 # sources the fused fluid kernel is built from (the traffic record is void once they change)
-FLUID_SRCS = [os.path.join(CSRC, f) for f in ("lbm_fluid_tma.cu", "lbm_fluid.cu", "lbm_common.cuh",
-                                               "lbm_internal.cuh")]
+FLUID_SRCS = [os.path.join(CSRC, f) for f in ("lbm_fluid_tma.cu", "lbm_fluid.cu", "lbm_fluid_direct.cu",
+                                               "lbm_common.cuh", "lbm_internal.cuh")]
 METRIC = "MLUPS & % HBM peak: FP32 vs FP16-store (err≤1e-3); adjoint/forward time ratio"
 NOMINAL_HBM_GBS = 7900.0  # GB300 HBM3e, nominal (the roofline uses the measured copy peak)
 
@@ -381,7 +381,8 @@ def main():
             fl, bx, pt = sim.step_timed(kn)
             out["step_kernels_ms"] = {"fluid": fl, "box_sums": bx, "particles": pt, "steps": kn,
                                       "note": "steps launched one by one without graphs, CUDA events "
-                                              "between the kernels (lbm_step_timed)"}
+                                              "between the kernels (lbm_step_timed); box_sums: the "
+                                              "interval of two events with nothing between them"}
         if with_e2e:
             blob = sim.save_state()
             pinned = torch.empty(len(blob), dtype=torch.uint8, pin_memory=True)

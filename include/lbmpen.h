@@ -11,7 +11,12 @@
  *      (Eq. 17);
  *   5. per-particle rigid-body projection U, omega over each solid domain
  *      (Eq. 22): the fused kernel adds the solid nodes' velocities up as exact
- *      integers, which give U and omega independent of the order of summation;
+ *      integers, which give U and omega independent of the order of summation.
+ *      In 3D the nodes of a sphere at dy^2 + dz^2 > (ceil(R) + 1)^2 from
+ *      floor(X) do not enter these sums (count included): a few outermost
+ *      nodes (4 of 2139 at R = 8) of a sphere whose centre lies near the far
+ *      corner of its lattice cell in y and z, up to R + sqrt(2) from floor(X).
+ *      lbm_rigid_projection_noalloc counts them;
  *   6. particle update: repulsive collision forces (Eqs. 19-21) and the
  *      predictor-corrector of Algorithm 1, which also yields the collision
  *      acceleration A applied on the particle's nodes in the next step.

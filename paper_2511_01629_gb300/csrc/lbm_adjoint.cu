@@ -765,7 +765,10 @@ cudaError_t launch_adj_fluid(int Q, int fp16, const InstDesc* insts, const AdjFl
     // With few tiles every segment goes to a warp of its own; with two waves of
     // tiles or more one block takes a whole tile and starts up once (backward pass,
     // 1 / 2 / 4 blocks per tile: one 400 x 1600 box, 240 steps 13.4 / 12.2 / 11.9 ms;
-    // 16 of them, 48 steps 19.7 / 20.7 / 22.9 ms).
+    // 48 steps FP32 of 1, 2, 3, 4, 8, 16 of them (800 tiles each): 2.49 / 2.36 / 2.37,
+    // 3.58 / 3.49 / 3.57, 4.59 / 4.58 / 4.68, 5.52 / 5.64 / 5.78, 9.18 / 9.64 / 10.64, 16.4 /
+    // 17.5 / 20.0 ms; FP16, half as tall tiles, 2.32 / 2.33 / 2.34 at 1600 tiles, 3.44 /
+    // 3.49 at 3200; 100 x 200 boxes and D3Q19 do not tell the splits apart).
     const bool many = ntiles >= 2 * ADJ_BLOCKS * num_sms;
     const dim3 grid((unsigned)ntiles, many ? 1u : (unsigned)per);
     auto go = [&](auto kern) { kern<<<grid, 32 * ADJ_WARPS, 0, st>>>(insts, afs, tile_inst, ninst, lam_mode, sh); };

@@ -546,9 +546,13 @@ int configure_shape(lbm_ctx* ctx, const Shape& sh_in) {
 Shape default_shape(int Q, int fp16, long long nodes) {
     // Small D2Q9 grids: straight into registers, one block of 4 rows per 64-node
     // tile.  2^18 nodes are one wave of such blocks (8 per SM); there the staged
-    // kernel's start (tables, work counter, ring) costs more than it gives:
-    // 100x200 10.3 us per step against 12.9, 200x800 (10 disks) 13.1 against 17.0,
-    // 300x1000 (20 disks) 16.7 against 17.7; above, 400x1600 17.4 against 14.9.
+    // kernel's start (tables, work counter, ring) costs more than it gives.  us per
+    // step, direct against staged, FP32 (FP16 within 1.3 us of it on both sides):
+    // 100x200 9.9 against 11.1, 200x800 (10 disks) 11.9 / 15.4, 256x1024 (10) 12.7 /
+    // 15.5, 300x1000 (20) 16.2 / 17.7; above, 400x1000 17.1 / 16.5, 400x1600 (1) 16.3 /
+    // 13.2, 512x2048 (50) 22.5 / 21.0.  Batches cross later (boxes of 128x256, 3 disks
+    // each: 8 of them, 2^18 nodes, 13.1 / 16.9; 12 16.2 / 17.0; 16 17.4 / 18.0; 32 25.9 /
+    // 24.2): the line takes their total all the same, and loses up to 9 % just above it.
     if (Q == 9 && nodes <= (1 << 18)) return Shape{fp16 ? 8 : 4, 4, 1, 4, 1, 1, 0, 64};
     // Larger ones: TMA-staged pipeline, 2 stages: FP32 8 rows and 8 consumer
     // warps (one box of all populations per tile, two blocks per SM); FP16 4

@@ -1,5 +1,5 @@
-// Device helpers shared by the fused fluid kernels (register path and TMA
-// path) and the export kernels of lbmpen.
+// Device helpers shared by the fused fluid kernels (staged, direct and register
+// path), the adjoint and the export kernels of lbmpen.
 #pragma once
 
 #include <type_traits>
