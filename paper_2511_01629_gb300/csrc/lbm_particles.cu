@@ -416,8 +416,9 @@ __device__ __forceinline__ LaneIn load_lane(const InstDesc& in, int i, int d, bo
     const long long j = 3LL * i + d;
     LaneIn L;
     const PState& ps = in.pst[par][i];
-    L.ec = ld_l2(&ps.ec);  // orientation theta^n of this step's record
-    L.es = ld_l2(&ps.es);
+    // orientation theta^n of this step's record
+    L.ec = first ? ld_l2(&ps.ec) : ps.ec;
+    L.es = first ? ld_l2(&ps.es) : ps.es;
     if (first) {
         L.X0 = ld_l2(ps.X + d);
         L.Ub = ld_l2(ps.U + d);  // U^{n-1} until project_lane
@@ -673,8 +674,9 @@ __device__ __forceinline__ void phase_substep(const InstDesc& in, int i0, int D,
     double th = 0.0, wo = 0.0;
     if (warp == 0) li = load_lane(in, i0 + usl, ud, uvalid, src, par, FIRST);
     if (warp == 1 && uvalid) {
-        th = ld_l2(in.theta + 3 * (i0 + usl) + ud);
-        wo = ld_l2(in.W + 3 * (i0 + usl) + ud);
+        const double *pt = in.theta + 3 * (i0 + usl) + ud, *pw = in.W + 3 * (i0 + usl) + ud;
+        th = FIRST ? ld_l2(pt) : *pt;
+        wo = FIRST ? ld_l2(pw) : *pw;
     }
     const bool pairs = in.np > 1;  // one particle: nothing to search
     const bool one = in.np <= XCHUNK;
