@@ -454,10 +454,10 @@ namespace {
 
 // Whether a particle at coordinate Y (radius R) along wall axis d can be within
 // the wall range R + delta/2 of either plane -1/2, n - 1/2: an FP32 test with
-// a 0.01 margin (the forward kernel's filter), so that particles far from the
+// a margin (wall_reach, the forward kernel's filter), so that particles far from the
 // walls skip the FP64 range tests, whose outcome it cannot change.
 __device__ __forceinline__ bool wall_near(const InstDesc& in, int d, double Y, double R) {
-    const float reach = 0.5f * (2.0f * (float)R + (float)in.delta) + 0.01f;
+    const float reach = wall_reach(in, d, R);
     const float yf = (float)Y;
     return !(yf + 0.5f > reach && (float)in.n[d] - 0.5f - yf > reach);
 }

@@ -933,6 +933,13 @@ __device__ __forceinline__ double rcp64(double x) {
     return fma(r, fma(-x, r, 1.0), r);
 }
 
+// Distance from a wall plane of axis d beyond which the FP32 pre-test skips the
+// wall force of a particle of extent R: the range R + delta / 2 and a margin over the
+// error of the FP32 coordinate (2^-24 n).
+__device__ __forceinline__ float wall_reach(const InstDesc& in, int d, double R) {
+    return 0.5f * (2.0f * (float)R + (float)in.delta) + fmaf(1e-7f, (float)in.n[d], 0.01f);
+}
+
 // Rigid-body projection of particle p (Eq. 22 with rho_s cancelled): the
 // sums are exact integers, converted to FP64.
 // Moments about the integer reference floor(X) are shifted to the centre:

@@ -85,13 +85,15 @@ struct PairGeo {
         return dv[0] * dv[0] + dv[1] * dv[1] + dv[2] * dv[2];
     }
 };
-__device__ __forceinline__ float pair_reach(const InstDesc& in, float4 xi) {
-    return xi.w + (float)in.delta + 0.01f;  // FP32 positions carry < 1e-3 error
+// An FP32 position on an axis of n nodes carries an error of 2^-24 n, a predicted
+// one twice that: the distance of two is off by up to 4 sqrt(3) 2^-24 n < 5e-7 n.
+__device__ __forceinline__ float pair_reach(const InstDesc& in, const PairGeo& g, float4 xi) {
+    return xi.w + (float)in.delta + fmaf(5e-7f, fmaxf(fmaxf(g.n[0], g.n[1]), g.n[2]), 0.01f);
 }
 
 __device__ __forceinline__ unsigned pair_mask(const InstDesc& in, int i, int lane, const float4* xs, int j0, int nj, float4 xi) {
     const PairGeo g(in);
-    const float reach = pair_reach(in, xi) + 2.0f;
+    const float reach = pair_reach(in, g, xi) + 2.0f;
     unsigned m = 0;
     for (int jj = lane, k = 0; jj < nj; jj += 32, ++k) {
         const float4 b = xs[jj];
@@ -107,7 +109,7 @@ __device__ __noinline__ void pair_forces(const InstDesc& in, int i, int src, int
                             double* f1, double* f2) {
     if (cp == 0.0) return;  // cp = C / eps_p of particle i
     const PairGeo g(in);
-    const float reach = pair_reach(in, xi);
+    const float reach = pair_reach(in, g, xi);
     // X + h Ubar of a particle in FP32, from its totals (before the first sub-step)
     auto predicted = [&](int j, float4 x) {
         const long long* v = in.tot[par] + (long long)NPV * j;
@@ -188,7 +190,7 @@ __device__ void gather_pairs(const double* f1, const double* f2, double* F1, dou
 __device__ void wall_force_d(const InstDesc& in, int d, double Xi, double& F, double cw, double inv_delta,
                              double Ri) {
     if (cw == 0.0) return;  // cw = C / eps_w of the particle
-    const float reach = 0.5f * (2.0f * (float)Ri + (float)in.delta) + 0.01f;
+    const float reach = wall_reach(in, d, Ri);
     if (in.periodic[d] || in.n[d] <= 1) return;
     const float xf = (float)Xi;  // skip walls farther than (2R + delta)/2
     if (xf + 0.5f > reach && (float)in.n[d] - 0.5f - xf > reach) return;
