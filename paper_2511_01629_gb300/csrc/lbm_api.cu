@@ -1226,7 +1226,7 @@ int lbm_load_state(lbm_ctx* ctx, const void* buf, size_t bytes) {
         CK(cudaMemcpy(I.ratio.ptr, r, sizeof(double) * I.np, cudaMemcpyHostToDevice));
         I.hratio.assign(reinterpret_cast<const double*>(r), reinterpret_cast<const double*>(r) + I.np);
         r += sizeof(double) * I.np;
-            if ((rc = upload_pconst(ctx, I))) return rc;
+        if ((rc = upload_pconst(ctx, I))) return rc;
         CK(cudaMemcpy(I.count.ptr, r, sizeof(int) * I.np, cudaMemcpyHostToDevice));
         r += sizeof(int) * I.np;
     }
